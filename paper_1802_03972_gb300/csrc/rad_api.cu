@@ -304,7 +304,8 @@ rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const do
                               const double* bdot, const double* w, double t, double dt) {
   if (c->prec == RAD_PREC_FP64) {
     return cuda_check(c, launch_fp64(c->d_omega, c->d_dirs, c->n_omega, c->n_dir, n, r, beta,
-                                     bdot, w, t, dt, c->d_state64, c->h_js.status, c->stream));
+                                     bdot, w, t, dt, c->d_state64, c->d_part64, c->d_cnt64,
+                                     c->f64_chunks, c->h_js.status, c->stream));
   }
   const int variant = c->tile.variant;
   const int ck = auto_chunk(c, variant, n, c->h_js.n_tiles);
@@ -481,6 +482,7 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
   wide_geometry(nd.data(), n_dir, js.tau_fast, js.axis, &js.cone_sin, &js.bucket_w);
 
   rad_status s = RAD_OK;
+  size_t f64_words = 0;  // doubles of an FP64 context's allocation
   auto chk = [&](cudaError_t e) {
     if (s == RAD_OK && e != cudaSuccess) s = (e == cudaErrorMemoryAllocation) ? RAD_ENOMEM : RAD_ECUDA;
   };
@@ -504,7 +506,15 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
       chk(dmalloc(&c->d_f2, (size_t)n_omega));
     }
   } else {
-    chk(dmalloc(&c->d_state64, (size_t)12 * c->n_bins));
+    c->f64_chunks = fp64_max_chunks(c->n_bins, device_sm_count());
+    const size_t sums = (size_t)12 * c->n_bins;
+    const size_t parts = c->f64_chunks > 1 ? (size_t)c->f64_chunks * 8 * c->n_bins : 0;
+    f64_words = sums + parts + ((size_t)fp64_blocks(c->n_bins) + 1) / 2;
+    chk(dmalloc(&c->d_state64, f64_words));
+    if (s == RAD_OK) {
+      c->d_part64 = c->d_state64 + sums;
+      c->d_cnt64 = reinterpret_cast<unsigned*>(c->d_part64 + parts);
+    }
   }
   if (s == RAD_OK) {
     chk(cudaMemcpy(c->d_omega, omega, sizeof(double) * n_omega, cudaMemcpyHostToDevice));
@@ -527,7 +537,7 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
         chk(cudaMemcpy(c->d_f2, f2.data(), sizeof(float) * n_omega, cudaMemcpyHostToDevice));
       }
     } else {
-      chk(cudaMemset(c->d_state64, 0, sizeof(double) * 12 * c->n_bins));
+      chk(cudaMemset(c->d_state64, 0, sizeof(double) * f64_words));
     }
   }
   js.om_tab = c->d_om_tab;

@@ -28,7 +28,13 @@ struct rad_ctx {
   radimpl::JobStatic* d_js = nullptr;
   double* d_spec = nullptr;      // [3][n_bins] readout staging for host outputs
   float* d_state = nullptr;      // MIXED: [16][n_bins]
-  double* d_state64 = nullptr;   // FP64:  [12][n_bins]
+  // FP64: [12][n_bins]; in the same allocation, the partial sums of a call cut
+  // into up to f64_chunks particle chunks, [f64_chunks][8][n_bins], and the
+  // arrival counters of its blocks (self-resetting)
+  double* d_state64 = nullptr;
+  double* d_part64 = nullptr;
+  unsigned* d_cnt64 = nullptr;
+  int f64_chunks = 1;
   // in-situ coupling (rad_push_step): three step slots of r, beta, w and beta_dot
   double* d_push = nullptr;      // [3][7 n_push] doubles: r (3n), beta (3n), w (n) per slot
   double* d_push_bdot = nullptr; // [3 n_push]

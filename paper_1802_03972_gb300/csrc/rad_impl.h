@@ -310,8 +310,12 @@ cudaError_t launch_readout(const float* state, int mixed, const double* state64,
                            double* coh, double* inc, double* tot, cudaStream_t s);
 cudaError_t launch_fp64(const double* omega, const double* dirs, int n_omega, int n_dir,
                         long long n, const double* r, const double* beta, const double* bdot,
-                        const double* w, double t, double dt, double* state64, int* status,
-                        cudaStream_t s);
+                        const double* w, double t, double dt, double* state64, double* part,
+                        unsigned* cnt, int max_chunks, int* status, cudaStream_t s);
+// The most particle chunks an FP64 call is cut into (its partial sums:
+// chunks x 8 x n_bins doubles when above one), and its blocks per chunk.
+int fp64_max_chunks(int n_bins, int sms);
+int fp64_blocks(int n_bins);
 cudaError_t launch_state_add(float* state, const float* other, int n_bins, int n_comps,
                              cudaStream_t s);
 cudaError_t launch_state64_add(double* state, const double* other, int n_bins, cudaStream_t s);
