@@ -33,19 +33,16 @@
 //    accumulation FMAs off the FP32 pipe, which together with the phase
 //    arithmetic and MUFU issue is what limits the FP32 variants.
 // Wide calls (particles spread beyond the fast phase range about the call's
-// reference point, sorted by the wide-call kernels) run in a second
-// instantiation (WIDE): their records are relative to the first particle of
-// each 256-particle group, so stage 1 and the update loop are unchanged, and
-// each tile's sums are rotated by e^{i omega tau_group} before they join the
-// chunk sums.
-// Sums are two-level (per particle tile, then per chunk).  Each work item
-// writes its partial sums; the last item of a bin tile to finish (an arrival
-// counter, no float atomics) adds the partials in chunk order, multiplies by
-// e^{i omega tau_ref(n)} (reduced in FP64) and adds the result into the
-// resident state with compensated (Kahan) FP32 sums.  Results are
-// deterministic for a given tile configuration.  Work items are handed out
-// tile-major, so a tile's partials are still in L2 when they are added up;
-// the tensor-core variants then drop those lines from L2 unwritten.
+// reference point, sorted by the wide-call kernels) run in a second pass of
+// the same launch, an instantiation of its own (WIDE): their records are relative to
+// the first particle of each 256-particle group, so stage 1 and the update loop
+// are unchanged, and each tile's sums are rotated by e^{i omega tau_group}
+// before they join the chunk sums.
+// Sums are two-level (per particle tile, then per chunk).  Each chunk's sums go to
+// a buffer of partials; a second kernel (reduce_kernel) adds them in chunk
+// order, multiplies by e^{i omega tau_ref(n)} (reduced in FP64) and adds the
+// result into the resident state with compensated (Kahan) FP32 sums.  No float
+// atomics: results are deterministic for a given chunking.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -88,13 +85,34 @@ __device__ __forceinline__ TileGeom tile_geom(const JobStatic& J, int tile, int 
   return g;
 }
 
-// A work item: its tile and particle chunk, and the chunking of that tile.
-// fine: the tile's index among the tiles of its fine-chunked level (TailPlan),
-// -1 for the coarse tiles.  (The level itself follows from the tile and the
-// call; the item, live across the whole particle loop, holds no more.)
+// A work item: its tile, its particle chunks (run of them from `chunk`), and
+// the chunking of that tile.  fine: the tile's index among the tiles of its
+// fine-chunked level (TailPlan), -1 for the coarse tiles.  (The level itself
+// follows from the tile and the call; the item, live across the whole particle
+// loop, holds no more.)
 struct ItemRef {
-  int tile, chunk, ck, n_chunks, fine;
+  int tile, chunk, run, ck, n_chunks, fine;
 };
+
+// The item in shared memory, for what is used after its first barrier: the hot
+// loops are short of registers.
+struct ItemShared {
+  ItemRef it;
+  int n_item;         // the item's particles
+  long long k_begin;  // its first particle
+};
+
+// q = a / b, r = a - q b; 64-bit division only where 32 bits do not hold a.
+__device__ __forceinline__ void div_rem(long long a, int b, int& q, int& r) {
+  if (a < (1LL << 32)) {
+    const unsigned u = (unsigned)a, v = u / (unsigned)b;
+    q = (int)v;
+    r = (int)(u - v * (unsigned)b);
+  } else {
+    q = (int)(a / b);
+    r = (int)(a - (long long)q * b);
+  }
+}
 
 // Item `local` of a job: the coarse tiles' items tile-major, then level 0's
 // fine tiles' items, then level 1's, each tile-major.  FINE = false: the
@@ -105,26 +123,26 @@ __device__ __forceinline__ ItemRef decode_item(const JobStatic& J, const JobCall
   static_assert(kTailLevels == 2, "two fine levels");
   ItemRef it;
   const int first0 = FINE ? J.n_tiles - K.tail_tiles[0] - K.tail_tiles[1] : J.n_tiles;
-  const long long coarse = (long long)first0 * K.n_chunks;
+  const int per_tile = K.run == 1 ? K.n_chunks : (K.n_chunks + K.run - 1) / K.run;
+  const long long coarse = (long long)first0 * per_tile;
   const long long fine0 = (long long)K.tail_tiles[0] * K.n_chunks_f[0];
   if (!FINE || local < coarse) {
-    it.tile = (int)(local / K.n_chunks);
-    it.chunk = (int)(local - (long long)it.tile * K.n_chunks);
+    div_rem(local, per_tile, it.tile, it.chunk);
+    it.chunk *= K.run;
+    it.run = min(K.run, K.n_chunks - it.chunk);
     it.ck = K.ck;
     it.n_chunks = K.n_chunks;
     it.fine = -1;
   } else if (local - coarse < fine0) {
-    const long long l = local - coarse;
-    it.fine = (int)(l / K.n_chunks_f[0]);
+    div_rem(local - coarse, K.n_chunks_f[0], it.fine, it.chunk);
     it.tile = first0 + it.fine;
-    it.chunk = (int)(l - (long long)it.fine * K.n_chunks_f[0]);
+    it.run = 1;
     it.ck = K.ck_f[0];
     it.n_chunks = K.n_chunks_f[0];
   } else {
-    const long long l = local - coarse - fine0;
-    it.fine = (int)(l / K.n_chunks_f[1]);
+    div_rem(local - coarse - fine0, K.n_chunks_f[1], it.fine, it.chunk);
     it.tile = first0 + K.tail_tiles[0] + it.fine;
-    it.chunk = (int)(l - (long long)it.fine * K.n_chunks_f[1]);
+    it.run = 1;
     it.ck = K.ck_f[1];
     it.n_chunks = K.n_chunks_f[1];
   }
@@ -160,11 +178,6 @@ __device__ __forceinline__ PartMap part_map(const JobStatic& J, const JobCall& K
   m.chunk_stride = (size_t)kComps * m.comp_stride;
   return m;
 }
-__device__ __forceinline__ size_t part_bin(const JobStatic& J, const ItemRef& it, const TileGeom& g,
-                                           int d, int o) {
-  return it.fine < 0 ? (size_t)d * J.n_omega + o : (size_t)(d - g.d0) * g.WT + (o - g.o0);
-}
-
 // Compensated (Kahan) add of x into sum with compensation cmp.
 __device__ __forceinline__ void kahan_add(float* sum, float* cmp, float x) {
   const float y = __fsub_rn(x, *cmp);
@@ -173,195 +186,10 @@ __device__ __forceinline__ void kahan_add(float* sum, float* cmp, float x) {
   *sum = tt;
 }
 
-// Arrival counter of the bin tile; true for the last work item of this call.
-template <int THREADS>
-__device__ __forceinline__ bool last_arrival(const JobStatic& J, const ItemRef& it, int* s_flag) {
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const int tile = it.tile;
-    const unsigned prev = atomicAdd(&J.tile_cnt[tile], 1u);
-    *s_flag = (prev == (unsigned)(it.n_chunks - 1));
-    if (*s_flag) J.tile_cnt[tile] = 0u;  // ready for the next call
-    __threadfence();
-  }
-  __syncthreads();
-  return *s_flag != 0;
-}
-
-// Drops one 128-byte L2 line without writing it back (its contents become
-// undefined; the line must not be read again before it is rewritten).
-__device__ __forceinline__ void discard_l2_line(const void* p) {
-  asm volatile("discard.global.L2 [%0], 128;" ::"l"(p) : "memory");
-}
-
-// The partial sums of a tile are dead once the last arrival has added them up,
-// and every call rewrites each slot before reading it.  Dropping their L2
-// lines saves the write-back to DRAM.  Arrays: n_arrays arrays from base, one
-// every `stride` floats, each laid out as [n_bins] (fine: false) or as a fine
-// level's [level tiles][NT WT] with base at this tile (fine: true); only
-// whole lines inside the tile's bins of each direction are dropped, so the
-// neighbouring tiles' partials are untouched.
-template <int THREADS>
-__device__ __forceinline__ void discard_tile_partials(const float* base, size_t stride,
-                                                      long long n_arrays, const JobStatic& J,
-                                                      const TileGeom& g, bool fine) {
-  // Four arrays per warp, eight lanes per array: a 256-bin row is 8 lines.
-  const int sub = threadIdx.x >> 3, l8 = threadIdx.x & 7;
-  const int n_om = J.n_omega, o1 = min(g.o0 + g.WT, n_om);
-  for (long long arr = sub; arr < n_arrays; arr += THREADS / 8) {
-    const float* ap = base + (size_t)arr * stride;
-    for (int dl = 0; dl < g.NT; ++dl) {
-      const int d = g.d0 + dl;
-      if (d >= J.n_dir) break;
-      // rp + o: the partial of bin (d, o)
-      const float* rp = fine ? ap + (size_t)dl * g.WT - g.o0 : ap + (size_t)d * n_om;
-      const uintptr_t a0 = reinterpret_cast<uintptr_t>(rp + g.o0);
-      const uintptr_t a1 = reinterpret_cast<uintptr_t>(rp + o1);
-      for (uintptr_t line = ((a0 + 127) & ~(uintptr_t)127) + (uintptr_t)l8 * 128; line + 128 <= a1;
-           line += 8 * 128)
-        discard_l2_line(reinterpret_cast<const void*>(line));
-    }
-  }
-}
-
-// Last arrival: for every bin of the tile, add the chunks' partials in chunk
-// order, rotate by e^{i omega tau_ref(n)} and add into the state (Kahan).
-// DISCARD: then drop the partials' L2 lines (tensor-core variants; the FP32
-// variants measured slower with it and keep the write-back).
 // Whether an item's chunks fit the partial-sum buffer it writes.
 __device__ __forceinline__ bool part_fits(const JobStatic& J, const ItemRef& it, const PartMap& m) {
   return it.fine < 0 ? it.n_chunks <= J.chunk_cap
                      : m.room >= (long long)it.n_chunks * (long long)m.chunk_stride;
-}
-
-// Rotation of a bin's chunk sums by e^{i omega tau_ref(n)} (psi in turns).
-__device__ __forceinline__ void bin_rotation(const JobStatic& J, int d, int o, float& cp, float& sp) {
-  const double* nd = J.dirs + 3 * d;
-  const double tref = J.ref[3] - (nd[0] * J.ref[0] + nd[1] * J.ref[1] + nd[2] * J.ref[2]) * kInvC;
-  double psi = J.om_turns[o] * tref;
-  psi -= rint(psi);
-  sincospif(2.0f * (float)psi, &sp, &cp);
-}
-
-// A fine tile's last arrival (TailPlan).  Its bins are contiguous in its
-// level's region ([chunk][comp][level tiles][NT WT], NT WT a multiple of 4,
-// 16-byte aligned), so the chunk sums are read four bins at a time: a unit is
-// (bin quad, component pair), consecutive threads take consecutive quads, and
-// each thread sums two units at once, keeping many loads in flight (a finest
-// tile has over a hundred chunks, and the last of these sums ends the
-// launch).  Every bin's components are still added in chunk order.
-template <int THREADS>
-__device__ __forceinline__ void fine_tile_sums(const JobStatic& J, const TileGeom& g, const PartMap& m,
-                                               int n_chunks) {
-  const int n_quads = g.NT * g.WT / 4, n_units = 4 * n_quads;
-  const int nb = J.n_bins, n_om = J.n_omega;
-  for (int ua = threadIdx.x; ua < n_units; ua += 2 * THREADS) {
-    const int ub = min(ua + THREADS, n_units - 1);  // a repeat of ua's last unit when past the end
-    const bool has_b = ua + THREADS < n_units;
-    const int pa = ua / n_quads, qa = ua - pa * n_quads;
-    const int pb = ub / n_quads, qb = ub - pb * n_quads;
-    const float* ra = m.base + (size_t)(2 * pa) * m.comp_stride + 4 * qa;
-    const float* rb = m.base + (size_t)(2 * pb) * m.comp_stride + 4 * qb;
-    float4 are = make_float4(0.f, 0.f, 0.f, 0.f), aim = are, bre = are, bim = are;
-#pragma unroll 4
-    for (int ch = 0; ch < n_chunks; ++ch) {
-      const size_t co = (size_t)ch * m.chunk_stride;
-      const float4 x0 = __ldcg(reinterpret_cast<const float4*>(ra + co));
-      const float4 x1 = __ldcg(reinterpret_cast<const float4*>(ra + co + m.comp_stride));
-      const float4 y0 = __ldcg(reinterpret_cast<const float4*>(rb + co));
-      const float4 y1 = __ldcg(reinterpret_cast<const float4*>(rb + co + m.comp_stride));
-      are.x += x0.x; are.y += x0.y; are.z += x0.z; are.w += x0.w;
-      aim.x += x1.x; aim.y += x1.y; aim.z += x1.z; aim.w += x1.w;
-      bre.x += y0.x; bre.y += y0.y; bre.z += y0.z; bre.w += y0.w;
-      bim.x += y1.x; bim.y += y1.y; bim.z += y1.z; bim.w += y1.w;
-    }
-    float* st = J.state;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (h == 1 && !has_b) break;
-      const int p = h ? pb : pa, q = h ? qb : qa;
-      const float re4[4] = {h ? bre.x : are.x, h ? bre.y : are.y, h ? bre.z : are.z, h ? bre.w : are.w};
-      const float im4[4] = {h ? bim.x : aim.x, h ? bim.y : aim.y, h ? bim.z : aim.z, h ? bim.w : aim.w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int i = 4 * q + k, dl = i / g.WT;
-        const int d = g.d0 + dl, o = g.o0 + (i - dl * g.WT);
-        if (d >= J.n_dir || o >= n_om) continue;
-        const int bin = d * n_om + o, c = 2 * p;
-        float cp, sp;
-        bin_rotation(J, d, o, cp, sp);
-        const float re = re4[k] * cp - im4[k] * sp;
-        const float im = re4[k] * sp + im4[k] * cp;
-        kahan_add(&st[(size_t)c * nb + bin], &st[(size_t)(kComps + c) * nb + bin], re);
-        kahan_add(&st[(size_t)(c + 1) * nb + bin], &st[(size_t)(kComps + c + 1) * nb + bin], im);
-      }
-    }
-  }
-}
-
-template <int THREADS, bool DISCARD>
-__device__ __forceinline__ void tile_epilogue(const JobStatic& J, const JobCall& K,
-                                              const ItemRef& it) {
-  const int tile = it.tile;
-  const TileGeom g = tile_geom(J, tile, THREADS);
-  const PartMap m = part_map(J, K, it, g);
-  const int nb = J.n_bins, n_om = J.n_omega;
-  if (!bounds_ok(part_fits(J, it, m) && tile < J.n_tiles, J.status)) return;
-  // (literal contexts run an FP32 variant: never fine tiles)
-  const bool vec = it.fine >= 0 && !J.literal && ((g.NT * g.WT) & 3) == 0;
-  if (vec) fine_tile_sums<THREADS>(J, g, m, it.n_chunks);
-  for (int i = threadIdx.x; i < (vec ? 0 : g.NT * g.WT); i += THREADS) {
-    const int dl = i / g.WT;
-    const int d = g.d0 + dl, o = g.o0 + (i - dl * g.WT);
-    if (d >= J.n_dir || o >= n_om) continue;
-    const int bin = d * n_om + o;
-    const size_t off = part_bin(J, it, g, d, o);
-    float s[kComps];
-#pragma unroll
-    for (int c = 0; c < kComps; ++c) s[c] = 0.0f;
-    // (unrolled so that several chunks' loads are in flight; the adds keep chunk order)
-#pragma unroll 4
-    for (int ch = 0; ch < it.n_chunks; ++ch) {
-      const float* pc = m.base + (size_t)ch * m.chunk_stride;
-#pragma unroll
-      for (int c = 0; c < kComps; ++c) s[c] += __ldcg(&pc[(size_t)c * m.comp_stride + off]);
-    }
-    float sp, cp;
-    bin_rotation(J, d, o, cp, sp);
-    float* st = J.state;
-#pragma unroll
-    for (int c = 0; c < kComps; c += 2) {
-      const float re = s[c] * cp - s[c + 1] * sp;
-      const float im = s[c] * sp + s[c + 1] * cp;
-      kahan_add(&st[(size_t)c * nb + bin], &st[(size_t)(kComps + c) * nb + bin], re);
-      kahan_add(&st[(size_t)(c + 1) * nb + bin], &st[(size_t)(kComps + c + 1) * nb + bin], im);
-    }
-    if (J.literal) {  // (literal contexts run an FP32 variant: never fine tiles)
-      float p[4] = {0.f, 0.f, 0.f, 0.f};
-      for (int ch = 0; ch < it.n_chunks; ++ch) {
-        const float* pc = J.partials_p + (size_t)ch * 4 * nb;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) p[c] += __ldcg(&pc[(size_t)c * nb + bin]);
-      }
-      float* sp_ = J.state_p;
-#pragma unroll
-      for (int c = 0; c < 4; c += 2) {
-        const float re = p[c] * cp - p[c + 1] * sp;
-        const float im = p[c] * sp + p[c + 1] * cp;
-        kahan_add(&sp_[(size_t)c * nb + bin], &sp_[(size_t)(4 + c) * nb + bin], re);
-        kahan_add(&sp_[(size_t)(c + 1) * nb + bin], &sp_[(size_t)(4 + c + 1) * nb + bin], im);
-      }
-    }
-  }
-  if constexpr (DISCARD) {
-    __syncthreads();  // every thread's reads of the partials are done
-    discard_tile_partials<THREADS>(m.base, m.comp_stride, (long long)it.n_chunks * kComps, J, g,
-                                   it.fine >= 0);
-    if (J.literal)
-      discard_tile_partials<THREADS>(J.partials_p, (size_t)nb, (long long)it.n_chunks * 4, J, g,
-                                     false);
-  }
 }
 
 __device__ __forceinline__ float sqrt_approx(float x) {
@@ -378,12 +206,21 @@ __device__ __forceinline__ double group_tau(const JobStatic& J, long long kt, in
   return -(nd[0] * D[0] + nd[1] * D[1] + nd[2] * D[2]) * kInvC;
 }
 
-// Loads one raw particle tile; thread 0 only.
-__device__ __forceinline__ void issue_tile(const JobStatic& J, long long k0, int KT, float* raw,
+// Loads kn raw particle records; thread 0 only.
+__device__ __forceinline__ void issue_tile(const JobStatic& J, long long k0, int kn, float* raw,
                                            uint64_t* bar) {
   // (skipped in a debug build when out of range: the block's bounded wait then gives up)
-  if (!bounds_ok(k0 + KT <= J.n_cap, J.status)) return;
-  tma_load_1d(raw, J.rec + (size_t)k0 * kRecFields, (uint32_t)KT * kRecFields * sizeof(float), bar);
+  if (!bounds_ok(k0 + kn <= J.n_cap, J.status)) return;
+  tma_load_1d(raw, J.rec + (size_t)k0 * kRecFields, (uint32_t)kn * kRecFields * sizeof(float), bar);
+}
+
+// Loads the tile at position `next` of the item, if there is one: it ends with
+// its chunk (c_end: the current chunk's end).
+__device__ __forceinline__ void issue_next(const JobStatic& J, const ItemShared& si, int next, int c_end,
+                                           int KT, float* raw, uint64_t* bar) {
+  if (next >= si.n_item) return;
+  const int end = next == c_end ? min(c_end + si.it.ck, si.n_item) : c_end;
+  issue_tile(J, si.k_begin + next, min(KT, end - next), raw, bar);
 }
 
 // ------------------------------------------------------------ FP32 variant
@@ -391,9 +228,10 @@ __device__ __forceinline__ void issue_tile(const JobStatic& J, long long k0, int
 // g = sqrt(1 + (w - 1) f(omega)^2), i.e. F_k(omega) dt a_i (Eq. 13 with Eq. 12).
 template <int THREADS, int W, int UNROLL, bool LIT = false, bool WIDE = false>
 __device__ __forceinline__ bool process_item_fma(const JobStatic& J, const JobCall& K,
-                                                 const ItemRef& item, unsigned char* __restrict__ smem,
-                                                 uint64_t* bar, uint32_t& phase, int* s_flag) {
-  const int tile = item.tile, chunk = item.chunk;
+                                                 const ItemRef& item0, const ItemShared& si,
+                                                 unsigned char* __restrict__ smem, uint64_t* bar,
+                                                 uint32_t& phase) {
+  const int tile = item0.tile;
   constexpr int NP = W / 2;
   constexpr int REC = LIT ? 4 : 3;                 // float4 per record
   constexpr int NC = kComps + (LIT ? 4 : 0);       // accumulated components per frequency
@@ -434,16 +272,18 @@ __device__ __forceinline__ bool process_item_fma(const JobStatic& J, const JobCa
     for (int c = 0; c < NC; ++c) acc1[p][c] = acc2[p][c] = make_float2(0.f, 0.f);
   const float2 kOne = make_float2(1.0f, 1.0f);
 
-  const long long k_begin = (long long)chunk * item.ck;
-  const long long k_end = min(k_begin + (long long)item.ck, K.n);
-  const int n_kt = (int)((k_end - k_begin + g.KT - 1) / g.KT);
-  // Whole tiles are copied: k_begin is a multiple of KT and the record buffer
-  // holds at least round_up(n, 256) particles, so every copy stays in bounds.
-  if (threadIdx.x == 0) issue_tile(J, k_begin, g.KT, raw, bar);
-  for (int it = 0; it < n_kt; ++it) {
-    const long long kt = k_begin + (long long)it * g.KT;
-    const int kn = (int)min((long long)g.KT, k_end - kt);
-    float4* rec = reinterpret_cast<float4*>(smem + S::raw_bytes + (size_t)(it & 1) * S::rec_bytes);
+  // The item's particles are walked in tiles of at most KT that end with their
+  // chunk (c_end; positions from the item's first particle).
+  int pos = 0, c_end;
+  {
+    const long long k_begin = (long long)item0.chunk * item0.ck;
+    c_end = (int)min((long long)item0.ck, K.n - k_begin);
+    if (threadIdx.x == 0) issue_tile(J, k_begin, min(g.KT, c_end), raw, bar);
+  }
+  const int nb = J.n_bins;
+  do {
+    const int kn = min(g.KT, c_end - pos);
+    float4* rec = reinterpret_cast<float4*>(smem + S::raw_bytes + (size_t)phase * S::rec_bytes);
     const bool landed = mbar_wait(bar, phase);
     phase ^= 1u;
     bool slow = false;
@@ -470,7 +310,7 @@ __device__ __forceinline__ bool process_item_fma(const JobStatic& J, const JobCa
       }
       return false;
     }
-    if (threadIdx.x == 0 && it + 1 < n_kt) issue_tile(J, kt + g.KT, g.KT, raw, bar);
+    if (threadIdx.x == 0) issue_next(J, si, pos + kn, c_end, g.KT, raw, bar);
     const float4* rc = rec + my_dl * REC;
     if (!(flags & 1)) {
       // kend particles at a record stride of nt; a full tile of one direction
@@ -517,7 +357,7 @@ __device__ __forceinline__ bool process_item_fma(const JobStatic& J, const JobCa
       // every update is formed in FP64.
       if (threadIdx.x == 0) atomicOr(J.status, ST_SLOW_PHASE);
       double tau_g = 0.0;
-      if constexpr (wide) tau_g = group_tau(J, kt, my_d);
+      if constexpr (wide) tau_g = group_tau(J, si.k_begin + pos, my_d);
       double omt[W];
 #pragma unroll
       for (int i = 0; i < W; ++i) omt[i] = J.om_turns[min(om_first + i, n_om - 1)];
@@ -558,7 +398,7 @@ __device__ __forceinline__ bool process_item_fma(const JobStatic& J, const JobCa
     // has tau_g in every phase).
     if constexpr (wide) {
       if (!(flags & 1)) {
-        const double tau_g = group_tau(J, kt, my_d);
+        const double tau_g = group_tau(J, si.k_begin + pos, my_d);
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
           float2 cs, sn;
@@ -581,34 +421,39 @@ __device__ __forceinline__ bool process_item_fma(const JobStatic& J, const JobCa
         acc2[p][c] = __fadd2_rn(acc2[p][c], acc1[p][c]);
         acc1[p][c] = make_float2(0.f, 0.f);
       }
-  }
-
-  // Partial sums of this work item.  (FP32 variants never take fine-chunked
-  // tiles, TailPlan: their items write the coarse partials directly, which
-  // keeps the fine tiles' bookkeeping out of this loop's registers.)
-  const int nb = J.n_bins;
-  float* part = J.partials + (size_t)chunk * kComps * nb;
-  if (my_d_raw < J.n_dir) {
+    pos += kn;
+    if (pos < c_end) continue;
+    const int chunk = si.it.chunk + (pos - 1) / si.it.ck;
+    // The chunk's partial sums.  (FP32 variants never take fine-chunked tiles,
+    // TailPlan: their items write the coarse partials directly, which keeps the
+    // fine tiles' bookkeeping out of this loop's registers.)
+    float* part = J.partials + (size_t)chunk * kComps * nb;
+    float* part_p = LIT ? J.partials_p + (size_t)chunk * 4 * nb : nullptr;
+    const size_t cs = nb, off = (size_t)my_d * n_om + om_first;
+    if (my_d_raw < J.n_dir) {
+#pragma unroll
+      for (int p = 0; p < NP; ++p)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int o = om_first + 2 * p + e;
+          if (o < n_om && bounds_ok(chunk < J.chunk_cap && si.it.fine < 0, J.status)) {
+#pragma unroll
+            for (int c = 0; c < kComps; ++c)
+              part[(size_t)c * cs + off + 2 * p + e] = e ? acc2[p][c].y : acc2[p][c].x;
+            if (LIT) {
+#pragma unroll
+              for (int c = 0; c < 4; ++c)
+                part_p[(size_t)c * cs + off + 2 * p + e] = e ? acc2[p][NC - 4 + c].y : acc2[p][NC - 4 + c].x;
+            }
+          }
+        }
+    }
 #pragma unroll
     for (int p = 0; p < NP; ++p)
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int o = om_first + 2 * p + e;
-        if (o < n_om && bounds_ok(chunk < J.chunk_cap && item.fine < 0, J.status)) {
-          const int bin = my_d * n_om + o;
-#pragma unroll
-          for (int c = 0; c < kComps; ++c)
-            part[(size_t)c * nb + bin] = e ? acc2[p][c].y : acc2[p][c].x;
-          if (LIT) {
-            float* pp = J.partials_p + (size_t)chunk * 4 * nb;
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-              pp[(size_t)c * nb + bin] = e ? acc2[p][NC - 4 + c].y : acc2[p][NC - 4 + c].x;
-          }
-        }
-      }
-  }
-  if (last_arrival<THREADS>(J, item, s_flag)) tile_epilogue<THREADS, false>(J, K, item);
+      for (int c = 0; c < NC; ++c) acc2[p][c] = make_float2(0.f, 0.f);
+    c_end = min(c_end + si.it.ck, si.n_item);
+  } while (pos < si.n_item);
   return true;
 }
 
@@ -620,9 +465,10 @@ __device__ __forceinline__ bool process_item_fma(const JobStatic& J, const JobCa
 // pairs instead of frequency pairs.
 template <int THREADS, int PASSES, int NB, bool WIDE = false, bool XT = false>
 __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCall& K,
-                                                const ItemRef& item, unsigned char* __restrict__ smem,
-                                                uint64_t* bar, uint32_t& phase, int* s_flag) {
-  const int tile = item.tile, chunk = item.chunk;
+                                                const ItemRef& item0, const ItemShared& si,
+                                                unsigned char* __restrict__ smem, uint64_t* bar,
+                                                uint32_t& phase) {
+  const int tile = item0.tile;
   // NB: 16-frequency blocks per warp; GQ: second-level float4 groups per pass
   constexpr int GQ = 2 * NB;
   using S = Smem<THREADS, true, false, PASSES * NB / 2, XT>;
@@ -643,6 +489,24 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
   const int s1_d = min(g.d0 + s1_dl, J.n_dir - 1);
   // WIDE: a wide call, whose records are relative to their group's reference point.
   constexpr bool wide = WIDE;
+
+  // The item's particles are walked in tiles of at most KT that end with their
+  // chunk (c_end; positions from the item's first particle).
+  int pos = 0, c_end;
+  {
+    const long long k_begin = (long long)item0.chunk * item0.ck;
+    c_end = (int)min((long long)item0.ck, K.n - k_begin);
+    if (threadIdx.x == 0) issue_tile(J, k_begin, min(g.KT, c_end), raw, bar);
+  }
+  // XT: the tile's direction rows, staged once per item for stage 1 (the
+  // previous item's last reads of them precede its closing barriers).
+  float* sdir = reinterpret_cast<float*>(smem + S::raw_bytes + 2 * S::rec_bytes + S::l2_bytes);
+  if constexpr (XT) {
+    for (int t = threadIdx.x; t < 12 * g.NT; t += THREADS) {
+      const int dl = t / 12, k = t - dl * 12;
+      sdir[t] = __ldg(J.dir_tab + (size_t)k * J.n_dir + min(g.d0 + dl, J.n_dir - 1));
+    }
+  }
 
   float2 omh[NB], wh[NB], wl[NB];
   // XT: omega/2pi (hi) of rows r and r + 8 of each block, each in both halves
@@ -688,27 +552,13 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
   for (int b = 0; b < NB; ++b)
 #pragma unroll
     for (int e = 0; e < 4; ++e) dre[b][e] = dim[b][e] = 0.0f;
+
 #pragma unroll
   for (int v = 0; v < GQ * PASSES; ++v) l2[v * THREADS + threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-
-  const long long k_begin = (long long)chunk * item.ck;
-  const long long k_end = min(k_begin + (long long)item.ck, K.n);
-  const int n_kt = (int)((k_end - k_begin + g.KT - 1) / g.KT);
-  if (threadIdx.x == 0) issue_tile(J, k_begin, g.KT, raw, bar);
-  // XT: the tile's direction rows, staged once per item for stage 1 (the
-  // previous item's last reads of them precede its closing barriers).
-  float* sdir = reinterpret_cast<float*>(smem + S::raw_bytes + 2 * S::rec_bytes + S::l2_bytes);
-  if constexpr (XT) {
-    for (int t = threadIdx.x; t < 12 * g.NT; t += THREADS) {
-      const int dl = t / 12, k = t - dl * 12;
-      sdir[t] = __ldg(J.dir_tab + (size_t)k * J.n_dir + min(g.d0 + dl, J.n_dir - 1));
-    }
-    __syncthreads();
-  }
-  for (int it = 0; it < n_kt; ++it) {
-    const long long kt = k_begin + (long long)it * g.KT;
-    const int kn = (int)min((long long)g.KT, k_end - kt);
-    unsigned char* recb = smem + S::raw_bytes + (size_t)(it & 1) * S::rec_bytes;
+  if constexpr (XT) __syncthreads();
+  do {
+    const int kn = min(g.KT, c_end - pos);
+    unsigned char* recb = smem + S::raw_bytes + (size_t)phase * S::rec_bytes;
     float2* tau2 = reinterpret_cast<float2*>(recb);                     // [NT][KT]
     float* ampb = reinterpret_cast<float*>(recb + (size_t)THREADS * 8);  // [NT][KT][8]
     // XT records: dtau hi [NT][KT]; the cross-term B rows [NT][KT][8] as four
@@ -768,7 +618,7 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
       }
       return false;
     }
-    if (threadIdx.x == 0 && it + 1 < n_kt) issue_tile(J, kt + g.KT, g.KT, raw, bar);
+    if (threadIdx.x == 0) issue_next(J, si, pos + kn, c_end, g.KT, raw, bar);
     const float2* tw = tau2 + my_dl * g.KT;
     const float* aw = ampb + (size_t)my_dl * g.KT * 8;
     const float* xtw = xth + my_dl * g.KT;
@@ -789,8 +639,8 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
       const int o_warp = o_warp0 + ps * PW;
       if (PASSES > 1) load_omega(o_warp);
       if (!(flags & 1)) {
-        // Unrolled 2x with two 16-frequency blocks per warp, 8x with four (measured: 1, 2, 4, 8).
-        constexpr int kUnroll = NB >= 4 ? 8 : 2;
+        // Unrolled 2x with two 16-frequency blocks per warp, 16x with four (LWFA step: 8x 6.88 ms, 16x 6.82).
+        constexpr int kUnroll = NB >= 4 ? 16 : 2;
         auto fast_loop = [&](const int kend) {
 #pragma unroll kUnroll
           for (int kk = 0; kk < kend; kk += 8) {
@@ -798,13 +648,16 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
               const float2 th2 = *reinterpret_cast<const float2*>(xtw + kk + 2 * c);
               const uint2 rt = *reinterpret_cast<const uint2*>(xrw + (size_t)(kk + r) * 8 + xr_off);
               const uint2 bb = xamp(kk);
+              // cr: rows r, r + 8 x particles kk + 2c, kk + 2c + 1.  All blocks'
+              // products first: one block's wait covers the next (0.1-1.3 % of a call).
+              float cr[NB][4];
+#pragma unroll
+              for (int b = 0; b < NB; ++b)
+                mma_tf32_zero(cr[b], xa[b][0], xa[b][1], xa[b][2], xa[b][3], rt.x, rt.y);
 #pragma unroll
               for (int b = 0; b < NB; ++b) {
-                // cr: rows r, r + 8 x particles kk + 2c, kk + 2c + 1
-                float cr[4];
-                mma_tf32_zero(cr, xa[b][0], xa[b][1], xa[b][2], xa[b][3], rt.x, rt.y);
-                const float2 p0 = phase2x(omr[b], th2, make_float2(cr[0], cr[1]));
-                const float2 p8 = phase2x(omr8[b], th2, make_float2(cr[2], cr[3]));
+                const float2 p0 = phase2x(omr[b], th2, make_float2(cr[b][0], cr[b][1]));
+                const float2 p8 = phase2x(omr8[b], th2, make_float2(cr[b][2], cr[b][3]));
                 tc_block(make_float2(p0.x, p8.x), make_float2(p0.y, p8.y), bb.x, bb.y, dre[b],
                          dim[b]);
               }
@@ -831,7 +684,7 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
       } else {
         if (threadIdx.x == 0) atomicOr(J.status, ST_SLOW_PHASE);
         double tau_g = 0.0;
-        if constexpr (wide) tau_g = group_tau(J, kt, my_d);
+        if constexpr (wide) tau_g = group_tau(J, si.k_begin + pos, my_d);
         double omt[NB][2];
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
@@ -877,7 +730,7 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
       // every block from their owners by shuffles.
       if constexpr (wide) {
         if (!(flags & 1)) {
-          const double tau_g = group_tau(J, kt, my_d);
+          const double tau_g = group_tau(J, si.k_begin + pos, my_d);
           float cA, sA, cB = 1.0f, sB = 0.0f;
           group_rotation(J.om_turns[min(o_warp + lane, n_om - 1)], tau_g, cA, sA);
           if constexpr (NB > 2)
@@ -908,7 +761,7 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
       float4* l2p = l2 + ps * GQ * THREADS + threadIdx.x;
 #pragma unroll
       for (int b = 0; b < NB; ++b) {
-        float4 x = l2p[b * THREADS], y = l2p[(NB + b) * THREADS];
+        const float4 x = l2p[b * THREADS], y = l2p[(NB + b) * THREADS];
         const float2 x01 = __fadd2_rn(make_float2(x.x, x.y), make_float2(dre[b][0], dre[b][1]));
         const float2 x23 = __fadd2_rn(make_float2(x.z, x.w), make_float2(dre[b][2], dre[b][3]));
         const float2 y01 = __fadd2_rn(make_float2(y.x, y.y), make_float2(dim[b][0], dim[b][1]));
@@ -919,91 +772,305 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
         for (int e = 0; e < 4; ++e) dre[b][e] = dim[b][e] = 0.0f;
       }
     }
-  }
-
-  // The D fragment holds rows (r, r+8) and columns (2c, 2c+1); columns 0-3 are
-  // the hi parts of (U.e1, U.e2, V.e1, V.e2), columns 4-7 the lo parts: lane c
-  // (c < 2) adds lane c+2's values.
-  const PartMap pm = part_map(J, K, item, g);
-  float* part = pm.base + (size_t)chunk * pm.chunk_stride;
+    pos += kn;
+    if (pos < c_end) continue;
+    // The chunk's partial sums.  The D fragment holds rows (r, r+8) and columns
+    // (2c, 2c+1); columns 0-3 are the hi parts of (U.e1, U.e2, V.e1, V.e2),
+    // columns 4-7 the lo parts: lane c (c < 2) adds lane c+2's values.  One base
+    // pointer per column and part, the rows at constant offsets.
+    {
+      const int chunk = si.it.chunk + (pos - 1) / si.it.ck;
+      const PartMap pm = part_map(J, K, si.it, g);
+      float* part = pm.base + (size_t)chunk * pm.chunk_stride;
+      const size_t cs = pm.comp_stride;
+      const size_t off = si.it.fine < 0 ? (size_t)my_d * n_om + o_warp0
+                                        : (size_t)my_dl * g.WT + (o_warp0 - g.o0);
+      float* q = part + off + r + (size_t)(4 * c) * cs;
+      const int left = n_om - o_warp0 - r;  // rows past the grid are not written
+      const bool mine = c < 2 && my_d_raw < J.n_dir &&
+                        bounds_ok(chunk < si.it.n_chunks && part_fits(J, si.it, pm), J.status);
 #pragma unroll 1
-  for (int ps = 0; ps < PASSES; ++ps)
+      for (int ps = 0; ps < PASSES; ++ps)
 #pragma unroll
-  for (int b = 0; b < NB; ++b)
+        for (int b = 0; b < NB; ++b) {
+          const float4 re4 = l2[(ps * GQ + b) * THREADS + threadIdx.x];
+          const float4 im4 = l2[(ps * GQ + NB + b) * THREADS + threadIdx.x];
+          const float re[4] = {re4.x, re4.y, re4.z, re4.w}, im[4] = {im4.x, im4.y, im4.z, im4.w};
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float* l2p = reinterpret_cast<const float*>(l2 + ps * GQ * THREADS + threadIdx.x);
-      const float lre = l2p[4 * b * THREADS + e];
-      const float lim = l2p[4 * (NB + b) * THREADS + e];
-      const float re = lre + __shfl_xor_sync(0xffffffffu, lre, 2);
-      const float im = lim + __shfl_xor_sync(0xffffffffu, lim, 2);
-      const int o = o_warp0 + ps * PW + 16 * b + r + ((e >> 1) << 3);
-      const int j = 2 * c + (e & 1);  // amplitude column
-      if (c < 2 && my_d_raw < J.n_dir && o < n_om &&
-          bounds_ok(chunk < item.n_chunks && part_fits(J, item, pm), J.status)) {
-        const size_t off = part_bin(J, item, g, my_d, o);
-        part[(size_t)(2 * j) * pm.comp_stride + off] = re;
-        part[(size_t)(2 * j + 1) * pm.comp_stride + off] = im;
-      }
+          for (int e = 0; e < 4; ++e) {
+            const float vr = re[e] + __shfl_xor_sync(0xffffffffu, re[e], 2);
+            const float vi = im[e] + __shfl_xor_sync(0xffffffffu, im[e], 2);
+            const int row = ps * PW + 16 * b + ((e >> 1) << 3);
+            if (mine && row < left) {  // amplitude column 2c + (e & 1)
+              q[(size_t)(2 * (e & 1)) * cs + row] = vr;
+              q[(size_t)(2 * (e & 1) + 1) * cs + row] = vi;
+            }
+          }
+        }
     }
-  if (last_arrival<THREADS>(J, item, s_flag)) tile_epilogue<THREADS, true>(J, K, item);
+    c_end = min(c_end + si.it.ck, si.n_item);
+    if (pos < si.n_item)
+#pragma unroll
+      for (int v = 0; v < GQ * PASSES; ++v) l2[v * THREADS + threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
+  } while (pos < si.n_item);
   return true;
 }
 
-// WIDE = false: the work items of jobs whose call is not wide; true: those of
-// wide calls (exits at once when no job of the launch is wide).  The two run
-// one after the other on the same stream, each with its own item counter, so
-// the common path keeps its register allocation free of the wide-call code.
-template <int THREADS, int W, int MINB, bool TC, bool LIT, int PASSES = 1, bool WIDE = false,
-          bool XT = false>
-__global__ void __launch_bounds__(THREADS, MINB) accumulate_kernel(LaunchArgs a) {
-  // Whether any job of the launch is wide is final before either kernel starts:
-  // the wide one leaves at once without, and the ordinary one then takes every
-  // item without looking at the jobs' flags.
-  const bool any_wide = a.any_wide != nullptr && *a.any_wide != 0;
-  if (WIDE && !any_wide) return;
+// The block's shared state: the current item and its job (one round trip to
+// global memory per job instead of one per use).
+struct BlockState {
+  JobStatic J;
+  JobCall K;
+  ItemShared it;
+  long long item;          // -1: a pass's first item is still to come
+  int job, cur_job;        // the item's job, and the one loaded (-1: none)
+  int any_wide;            // some job of the launch is wide
+};
+
+template <int THREADS>
+__device__ __forceinline__ void load_job(BlockState& b, const LaunchArgs& a, int j) {
+  copy_words<THREADS>(&b.J, &a.js[j], sizeof(JobStatic));
+  copy_words<THREADS>(&b.K, a.use_inline ? &a.inline_call : &a.jc[j], sizeof(JobCall));
+}
+
+// The work items of the jobs whose call is not wide (WIDE = false) or is (true),
+// each from its own counter.  Two instantiations, so the common path keeps
+// its register allocation free of the wide-call code.  False: a wait gave up.
+template <int THREADS, int W, bool TC, bool LIT, int PASSES, bool WIDE, bool XT>
+__device__ __forceinline__ bool run_items(const LaunchArgs& a, BlockState& b, unsigned char* smem,
+                                          uint64_t* bar, uint32_t& phase) {
+  for (;;) {
+    __syncthreads();  // the last item's shared state is used up
+    if (threadIdx.x < 32) {
+      long long item = blockIdx.x;  // a block's first item is its index, the others come from the counter
+      if (b.item >= 0) {
+        unsigned long long v = 0;
+        if (threadIdx.x == 0) v = atomicAdd(a.item_counter + (WIDE ? 1 : 0), 1ULL);
+        item = (long long)(gridDim.x + __shfl_sync(0xffffffffu, v, 0));
+      }
+      const int j = item < a.n_items ? find_job_warp(a, item) : 0;
+      __syncwarp();
+      if (threadIdx.x == 0) {
+        b.item = item;
+        b.job = j;
+      }
+    }
+    __syncthreads();
+    const long long item = b.item;
+    if (item >= a.n_items) return true;
+    if (b.job != b.cur_job) {
+      __syncthreads();
+      if (threadIdx.x == 0) b.cur_job = b.job;
+      load_job<THREADS>(b, a, b.job);
+      __syncthreads();
+    }
+    if (b.any_wide && (b.J.wide_flag != nullptr && *b.J.wide_flag != 0) != WIDE) continue;  // the other pass's
+    // Tile-major order: one tile's chunks run close together in time.
+    const ItemRef it = decode_item<TC>(b.J, b.K, item - b.K.item_begin);
+    if (threadIdx.x == 0) {
+      b.it.it = it;
+      b.it.k_begin = (long long)it.chunk * it.ck;
+      b.it.n_item = (int)min((long long)it.run * it.ck, b.K.n - b.it.k_begin);
+    }
+    bool ok;
+    if constexpr (TC)
+      ok = process_item_tc<THREADS, PASSES, 2 * W, WIDE, XT>(b.J, b.K, it, b.it, smem, bar, phase);
+    else
+      ok = process_item_fma<THREADS, W, 8, LIT, WIDE>(b.J, b.K, it, b.it, smem, bar, phase);
+    if (!ok) return false;
+  }
+}
+
+template <int THREADS, int W, int MINB, bool TC, bool LIT, int PASSES = 1, bool XT = false>
+__global__ void __launch_bounds__(THREADS, MINB) accumulate_kernel(const __grid_constant__ LaunchArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t bar;
-  __shared__ long long s_item[2];
-  __shared__ int s_flag;
-  if (threadIdx.x == 0) {
-    mbar_init(&bar, 1);
-    mbar_fence_init();
-  }
+  __shared__ __align__(8) BlockState b;
   // Profiling: the block's start, kept in shared memory rather than in
   // registers live across the whole loop.
   __shared__ long long s_clk0;
   __shared__ unsigned long long s_ns0;
+  pdl_trigger();
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    mbar_fence_init();
+  }
+  // A single job's tables do not depend on the kernels before this one.
+  if (a.n_jobs == 1) load_job<THREADS>(b, a, 0);
+  pdl_wait();
+  // Whether any job of the launch is wide is final by now; without, the first
+  // pass takes every item without looking at the jobs' flags.
+  if (threadIdx.x == 0) {
+    b.any_wide = a.any_wide != nullptr && *a.any_wide != 0;
+    b.cur_job = a.n_jobs == 1 ? 0 : -1;
+    b.item = -1;
+  }
   if (a.prof_clk && threadIdx.x == 0) {
     s_clk0 = clock64();
     s_ns0 = global_ns();
   }
-  __syncthreads();
   uint32_t phase = 0u;
-  int buf = 0;
-  for (;;) {
-    if (threadIdx.x == 0) s_item[buf] = (long long)atomicAdd(a.item_counter + (WIDE ? 1 : 0), 1ULL);
+  const bool ok = run_items<THREADS, W, TC, LIT, PASSES, false, XT>(a, b, smem, &bar, phase);
+  if (ok && b.any_wide) {
     __syncthreads();
-    const long long item = s_item[buf];
-    buf ^= 1;
-    if (item >= a.n_items) break;
-    const int j = find_job(a, item);
-    const JobStatic& J = a.js[j];
-    if (any_wide && (J.wide_flag != nullptr && *J.wide_flag != 0) != WIDE) continue;  // the other kernel's
-    const JobCall K = a.use_inline ? a.inline_call : a.jc[j];
-    // Tile-major order: the chunks of one tile run close together in time, so
-    // their partial sums are still in L2 when the tile's last arrival reads them.
-    const ItemRef it = decode_item<TC>(J, K, item - K.item_begin);
-    bool ok;
-    if constexpr (TC)
-      ok = process_item_tc<THREADS, PASSES, 2 * W, WIDE, XT>(J, K, it, smem, &bar, phase, &s_flag);
-    else
-      ok = process_item_fma<THREADS, W, 8, LIT, WIDE>(J, K, it, smem, &bar, phase, &s_flag);
-    if (!ok) break;
+    if (threadIdx.x == 0) b.item = -1;
+    run_items<THREADS, W, TC, LIT, PASSES, true, XT>(a, b, smem, &bar, phase);
   }
-  if (a.prof_clk && threadIdx.x == 0) {
-    atomicAdd(&a.prof_clk[0], (unsigned long long)(clock64() - s_clk0));
-    atomicAdd(&a.prof_clk[1], global_ns() - s_ns0);
+  if (threadIdx.x == 0) {
+    if (a.prof_clk) {
+      atomicAdd(&a.prof_clk[0], (unsigned long long)(clock64() - s_clk0));
+      atomicAdd(&a.prof_clk[1], global_ns() - s_ns0);
+    }
+    // The last block to leave puts the counter block back to zero for the next
+    // call (no block claims an item after it has counted itself out).
+    unsigned* out = reinterpret_cast<unsigned*>(a.item_counter + kCounterExit);
+    if (atomicAdd(out, 1u) == gridDim.x - 1) {
+      a.item_counter[0] = a.item_counter[1] = 0ULL;
+      *out = 0u;
+      if (a.any_wide) *a.any_wide = 0;
+    }
+  }
+}
+
+// ------------------------------------------------------------ tile reduction
+// Adds the chunks' partial sums of every bin, multiplies by e^{i omega
+// tau_ref(n)} (reduced in FP64) and adds the result into the resident state
+// with compensated (Kahan) FP32 sums.  A kernel of its own after the accumulate
+// kernel: summed by the block that finished a tile last, a tile of many chunks
+// was read by one SM at the end of the launch (90 of 157 us for 79 chunks of 4
+// tiles, 35 us of the 6.9 ms LWFA step), and every item paid a fence and a
+// counter.  Bound by the partials' bytes (mostly in L2) and, for small
+// grids, by latency: kRedBins bins per block, a thread takes a quad of bins and
+// a component pair over a quarter of the chunks, several chunks' loads in
+// flight.  The quarters are added in chunk order, so results are a function of the
+// chunking alone.  With it and the chunks of small calls (auto_chunk_for):
+// 20000 particles, 128 x 16 bins, FP32 variant, 467 -> 76 us a call; 1777
+// particles, 96 x 25 bins 64 -> 32 us; the LWFA step 6.96 -> 6.82 ms.
+constexpr int kRedBins = 128;
+constexpr int kRedGroups = 4;  // chunk ranges
+constexpr int kRedThreads = kRedBins / 4 * 4 * kRedGroups;
+
+// Four bins' values at p (vec: 16-byte aligned and all inside the grid).
+__device__ __forceinline__ float4 load_quad(const float* p, bool vec, int live) {
+  if (vec) return __ldcg(reinterpret_cast<const float4*>(p));
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (live > 0) v.x = __ldcg(p);
+  if (live > 1) v.y = __ldcg(p + 1);
+  if (live > 2) v.z = __ldcg(p + 2);
+  if (live > 3) v.w = __ldcg(p + 3);
+  return v;
+}
+
+__global__ void __launch_bounds__(kRedThreads) reduce_kernel(const __grid_constant__ LaunchArgs a) {
+  __shared__ __align__(8) BlockState b;
+  __shared__ float4 part[kRedGroups - 1][2][kRedBins];
+  __shared__ float2 rot[kRedBins];
+  pdl_trigger();
+  if (a.n_jobs == 1) {
+    load_job<kRedThreads>(b, a, 0);
+  } else {
+    if (threadIdx.x < 32) {
+      int n = 0;
+      for (int i = threadIdx.x; i < a.n_jobs; i += 32) n += a.jc[i].red_begin <= blockIdx.x;
+      n = __reduce_add_sync(0xffffffffu, n) - 1;
+      if (threadIdx.x == 0) b.job = n;
+    }
+    __syncthreads();
+    load_job<kRedThreads>(b, a, b.job);
+  }
+  pdl_wait();
+  __syncthreads();
+  const JobStatic& J = b.J;
+  const JobCall& K = b.K;
+  const int per_tile = J.nt * J.wt / kRedBins;
+  const long long local = (long long)blockIdx.x - K.red_begin;
+  ItemRef it;
+  int s;
+  div_rem(local, per_tile, it.tile, s);
+  const int first1 = J.n_tiles - K.tail_tiles[1], first0 = first1 - K.tail_tiles[0];
+  it.fine = it.tile >= first1 ? it.tile - first1 : (it.tile >= first0 ? it.tile - first0 : -1);
+  it.n_chunks = it.fine < 0 ? K.n_chunks : K.n_chunks_f[it.tile >= first1 ? 1 : 0];
+  it.chunk = it.run = it.ck = 0;
+  const TileGeom g = tile_geom(J, it.tile, 256);
+  const PartMap m = part_map(J, K, it, g);
+  if (!bounds_ok(part_fits(J, it, m), J.status)) return;
+  const int nb = J.n_bins, n_om = J.n_omega, sh = __ffs(g.WT) - 1;  // tile widths are powers of two
+  const int q = threadIdx.x & 31, pair = (threadIdx.x >> 5) & 3, cg = threadIdx.x >> 7;
+  const int i = s * kRedBins + 4 * q;  // first of the thread's bins within the tile
+  const int d = g.d0 + (i >> sh), o = g.o0 + (i & (g.WT - 1));
+  const int live = d < J.n_dir ? min(4, n_om - o) : 0;  // bins inside the grid (<= 0: none)
+  const size_t bin = (size_t)d * n_om + o;
+  const bool om4 = (n_om & 3) == 0;
+  const bool vec = live > 0 && (it.fine >= 0 || om4);
+  // rotations: the last chunk range's threads, one bin each
+  if (cg == kRedGroups - 1) {
+    const int t = threadIdx.x & (kRedBins - 1), ti = s * kRedBins + t;
+    const double* nd = J.dirs + 3 * (size_t)min(g.d0 + (ti >> sh), J.n_dir - 1);
+    const double tref = J.ref[3] - (nd[0] * J.ref[0] + nd[1] * J.ref[1] + nd[2] * J.ref[2]) * kInvC;
+    double psi = J.om_turns[min(g.o0 + (ti & (g.WT - 1)), n_om - 1)] * tref;  // turns
+    psi -= rint(psi);
+    float2 cs;
+    sincospif(2.0f * (float)psi, &cs.y, &cs.x);
+    rot[t] = cs;
+  }
+  const int per = (it.n_chunks + kRedGroups - 1) / kRedGroups;
+  const int c0 = min(cg * per, it.n_chunks), c1 = min(c0 + per, it.n_chunks);
+  // set 0: U and V; set 1: the literal sum's two pairs
+  for (int set = 0; set < (J.literal ? 2 : 1); ++set) {
+    const bool mine = live > 0 && (set == 0 || pair < 2);
+    const float* base = set ? J.partials_p + bin : m.base + (it.fine < 0 ? bin : (size_t)i);
+    const size_t cs = set ? (size_t)nb : m.comp_stride, chs = set ? (size_t)4 * nb : m.chunk_stride;
+    float4 re = make_float4(0.f, 0.f, 0.f, 0.f), im = re;
+    if (mine) {
+      const float* p = base + (size_t)(2 * pair) * cs + (size_t)c0 * chs;
+#pragma unroll 8
+      for (int ch = c0; ch < c1; ++ch, p += chs) {
+        const float4 x = load_quad(p, vec, live), y = load_quad(p + cs, vec, live);
+        re.x += x.x; re.y += x.y; re.z += x.z; re.w += x.w;
+        im.x += y.x; im.y += y.y; im.z += y.z; im.w += y.w;
+      }
+    }
+    __syncthreads();  // (set 1: the first set's sums are used up)
+    if (cg > 0) {
+      part[cg - 1][0][threadIdx.x & 127] = re;
+      part[cg - 1][1][threadIdx.x & 127] = im;
+    }
+    __syncthreads();
+    if (cg > 0 || !mine) continue;
+#pragma unroll
+    for (int k = 0; k < kRedGroups - 1; ++k) {
+      const float4 x = part[k][0][threadIdx.x], y = part[k][1][threadIdx.x];
+      re.x += x.x; re.y += x.y; re.z += x.z; re.w += x.w;
+      im.x += y.x; im.y += y.y; im.z += y.z; im.w += y.w;
+    }
+    float* st = (set ? J.state_p : J.state) + bin;
+    const int nc = set ? 4 : kComps, c = 2 * pair;
+    const bool st4 = om4 && (reinterpret_cast<uintptr_t>(set ? J.state_p : J.state) & 15) == 0;
+    float* sp[4] = {st + (size_t)c * nb, st + (size_t)(c + 1) * nb, st + (size_t)(nc + c) * nb,
+                    st + (size_t)(nc + c + 1) * nb};
+    float v[4][4];  // sum re, sum im, compensation re, compensation im of the four bins
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float4 x = load_quad(sp[k], st4, live);
+      v[k][0] = x.x, v[k][1] = x.y, v[k][2] = x.z, v[k][3] = x.w;
+    }
+    const float re4[4] = {re.x, re.y, re.z, re.w}, im4[4] = {im.x, im.y, im.z, im.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float2 t = rot[4 * q + k];
+      kahan_add(&v[0][k], &v[2][k], re4[k] * t.x - im4[k] * t.y);
+      kahan_add(&v[1][k], &v[3][k], re4[k] * t.y + im4[k] * t.x);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (st4) {
+        *reinterpret_cast<float4*>(sp[k]) = make_float4(v[k][0], v[k][1], v[k][2], v[k][3]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (e < live) sp[k][e] = v[k][e];
+      }
+    }
   }
 }
 
@@ -1014,37 +1081,36 @@ cudaError_t launch_acc(const LaunchArgs& a, int grid, cudaStream_t s) {
   static std::atomic<bool> attr_set[kMaxDevices];
   const int dev = current_device();
   if (dev < 0 || dev >= kMaxDevices || !attr_set[dev].load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(accumulate_kernel<T, W, MINB, TC, LIT, P, false, XT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(accumulate_kernel<T, W, MINB, TC, LIT, P, true, XT>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = cudaFuncSetAttribute(accumulate_kernel<T, W, MINB, TC, LIT, P, XT>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < kMaxDevices) attr_set[dev].store(true, std::memory_order_release);
   }
-  accumulate_kernel<T, W, MINB, TC, LIT, P, false, XT><<<grid, T, smem, s>>>(a);
   count_launches(1);
-  if (a.any_wide != nullptr) {
-    accumulate_kernel<T, W, MINB, TC, LIT, P, true, XT><<<grid, T, smem, s>>>(a);
-    count_launches(1);
-  }
-  return cudaGetLastError();
+  return launch_pdl(accumulate_kernel<T, W, MINB, TC, LIT, P, XT>, grid, T, smem, s, a);
 }
 
 template <int T, int W, int MINB, bool TC, bool LIT, int P = 1, bool XT = false>
 int blocks_per_sm() {
   int nb = 0;
   const size_t smem = Smem<T, TC, LIT, TC ? P * W : P, XT>::bytes;
-  cudaFuncSetAttribute(accumulate_kernel<T, W, MINB, TC, LIT, P, false, XT>,
+  cudaFuncSetAttribute(accumulate_kernel<T, W, MINB, TC, LIT, P, XT>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-          &nb, accumulate_kernel<T, W, MINB, TC, LIT, P, false, XT>, T, smem) != cudaSuccess ||
+          &nb, accumulate_kernel<T, W, MINB, TC, LIT, P, XT>, T, smem) != cudaSuccess ||
       nb < 1)
     nb = 1;
   return nb;
 }
 
 }  // namespace
+
+int reduce_blocks(const JobStatic& js) { return js.n_tiles * (js.nt * js.wt / kRedBins); }
+
+cudaError_t launch_reduce(const LaunchArgs& a, long long blocks, cudaStream_t s) {
+  count_launches(1);
+  return launch_pdl(reduce_kernel, blocks, kRedThreads, 0, s, a);
+}
 
 // Variants (rad_impl.h: variant_info): 0 FP32 256x2, 1 FP32 256x4, 2 FP32 128x2,
 // 3 tensor-core 256 (3 CTAs/SM), 4 tensor-core 256 (4 CTAs/SM), 5 FP32 256x2 (4 CTAs/SM),

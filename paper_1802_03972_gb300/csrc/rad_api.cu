@@ -146,22 +146,35 @@ int resident_ctas(int variant) {
   return device_sm_count() * accumulate_blocks_per_sm(variant);
 }
 
-// Particles per (coarse) work item: kItemsPerCta items per resident CTA in
-// total when the job's last tiles are fine-chunked (fine_tail), else
-// kItemsPerCtaUniform; items a multiple of the shared-memory tile.  Depends only
-// on the job's shape, n and the device, so a job is chunked the same way alone
-// and in a batch.
+// Particles per chunk.  A job with work enough takes kItemsPerCta items per
+// resident CTA in total when its last tiles are fine-chunked (fine_tail), else
+// kItemsPerCtaUniform, of kMinChunk particles or more.  Below that the launch is a few
+// waves of items on the resident CTAs, and the chunk is the one whose waves end
+// first: waves x (particles + an item's fixed cost in particles, kItemCost).
+// Chunks below kChunkAlign only while one wave holds them.  Depends only on the
+// job's shape, n and the device, so a job is chunked the same way alone and in a
+// batch.
 int auto_chunk_for(int variant, long long n, int n_tiles, bool fine_tail) {
-  const long long target =
-      (long long)(fine_tail ? kItemsPerCta : kItemsPerCtaUniform) * resident_ctas(variant);
+  const long long resident = resident_ctas(variant);
+  const long long target = (long long)(fine_tail ? kItemsPerCta : kItemsPerCtaUniform) * resident;
   long long chunks = (target + n_tiles - 1) / n_tiles;
   const long long max_chunks = (n + kChunkAlign - 1) / kChunkAlign;
   chunks = std::max(1LL, std::min(chunks, max_chunks));
   long long ck = (n + chunks - 1) / chunks;
   ck = (ck + kChunkAlign - 1) / kChunkAlign * kChunkAlign;
-  if (ck < kMinChunk && n > kMinChunk) ck = kMinChunk;
-  if (ck > (1LL << 30)) ck = 1LL << 30;
-  return (int)ck;
+  if (ck >= kMinChunk) return (int)std::min(ck, 1LL << 30);
+  long long best = 0, best_cost = 0;
+  for (long long c = kSmallestChunk; c <= kMinChunk; c += c < kChunkAlign ? c : kChunkAlign) {
+    const long long per_tile = (n + c - 1) / c, waves = (per_tile * n_tiles + resident - 1) / resident;
+    if (c < kChunkAlign && waves > 1) continue;
+    const long long cost = waves * (std::min(c, n) + kItemCost);
+    if (best == 0 || cost <= best_cost) {
+      best = c;
+      best_cost = cost;
+    }
+    if (per_tile == 1) break;
+  }
+  return (int)best;
 }
 
 int auto_chunk(const rad_ctx* c, int variant, long long n, int n_tiles) {
@@ -335,12 +348,10 @@ rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const do
   K.dt = dt;
   K.ck = ck;
   K.n_chunks = n_chunks;
+  K.run = 1;
   set_tail(K, tail);
   K.item_begin = 0;
   K.block_begin = 0;
-  s = cuda_check(c, cudaMemsetAsync(c->d_counter, 0, kCounterWords * sizeof(unsigned long long),
-                                    c->stream));
-  if (s != RAD_OK) return s;
   cudaEvent_t* ev = nullptr;
   if (c->prof_on) {
     if (c->prof_used + 3 > c->prof_ev.size()) {
@@ -364,6 +375,7 @@ rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const do
   if (ev) cudaEventRecord(ev[1], c->stream);
   const long long grid = std::min<long long>(a.n_items, resident_ctas(variant));
   s = cuda_check(c, launch_accumulate(variant, a, (int)grid, c->stream));
+  if (s == RAD_OK) s = cuda_check(c, launch_reduce(a, reduce_blocks(c->h_js), c->stream));
   if (ev) cudaEventRecord(ev[2], c->stream);
   return s;
 }
@@ -498,9 +510,6 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
   chk(dmalloc(&c->d_spec, (size_t)3 * c->n_bins));
   if (prec == RAD_PREC_MIXED) {
     chk(dmalloc(&c->d_state, (size_t)2 * kComps * c->n_bins));
-    // Enough arrival counters for any tiling (frequency tiles are >= 32 wide).
-    c->tile_cnt_cap = ((n_omega + 31) / 32) * n_dir + 1;
-    chk(dmalloc(&c->d_tile_cnt, (size_t)c->tile_cnt_cap));
     if (literal) {
       chk(dmalloc(&c->d_state_p, (size_t)8 * c->n_bins));
       chk(dmalloc(&c->d_f2, (size_t)n_omega));
@@ -523,10 +532,10 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
     chk(cudaMemcpy(c->d_dirs, nd.data(), sizeof(double) * nd.size(), cudaMemcpyHostToDevice));
     chk(cudaMemcpy(c->d_dir_tab, dir_tab.data(), sizeof(float) * dir_tab.size(), cudaMemcpyHostToDevice));
     chk(cudaMemset(c->d_status, 0, sizeof(int)));
+    chk(cudaMemset(c->d_counter, 0, kCounterWords * sizeof(unsigned long long)));
     chk(cudaMemset(c->d_ref, 0, 4 * sizeof(double)));
     if (prec == RAD_PREC_MIXED) {
       chk(cudaMemset(c->d_state, 0, sizeof(float) * 2 * kComps * c->n_bins));
-      chk(cudaMemset(c->d_tile_cnt, 0, sizeof(unsigned) * c->tile_cnt_cap));
       if (literal && s == RAD_OK) {
         std::vector<float> f2(n_omega);
         for (int i = 0; i < n_omega; ++i) {
@@ -546,13 +555,12 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
   js.dir_tab = c->d_dir_tab;
   js.dirs = c->d_dirs;
   js.state = c->d_state;
-  js.tile_cnt = c->d_tile_cnt;
   js.ref = c->d_ref;
   js.status = c->d_status;
   js.literal = literal ? 1 : 0;
   js.f2_tab = c->d_f2;
   js.state_p = c->d_state_p;
-  // the wide flag lives in the counter block, zeroed before every call
+  // the wide flag lives in the counter block, zero between calls
   js.wide_flag = c->d_counter ? reinterpret_cast<int*>(c->d_counter + 2) : nullptr;
   if (literal) {
     c->tile.variant = kLiteralVariant;
@@ -573,7 +581,7 @@ void rad_destroy(rad_ctx* c) {
   cudaStreamSynchronize(c->stream);
   void* ptrs[] = {c->d_omega, c->d_om_turns, c->d_om_tab, c->d_dirs, c->d_dir_tab, c->d_ref,
                   c->d_status, c->d_counter, c->d_js, c->d_spec, c->d_state, c->d_state64,
-                  c->d_tile_cnt, c->h_js.rec, c->h_js.partials, c->d_stage, c->d_state_p,
+                  c->h_js.rec, c->h_js.partials, c->d_stage, c->d_state_p,
                   c->d_f2, c->h_js.partials_p, c->d_push, c->d_push_bdot, c->h_js.perm,
                   c->h_js.sort_counts, c->h_js.bucket_base, c->h_js.gref, c->h_js.partials_f};
   for (void* p : ptrs)
@@ -940,7 +948,6 @@ rad_status rad_set_tile(rad_ctx* c, const rad_tile* t) {
   if (s != RAD_OK) return s;
   JobStatic js = c->h_js;
   fill_tiles(js, t->variant, wt);
-  if (js.n_tiles > c->tile_cnt_cap) return fail(c, RAD_EINVAL);
   c->h_js = js;
   c->tile.variant = t->variant;
   c->tile.omega_tile = wt;

@@ -174,12 +174,24 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
     invalidate_graphs();
   }
 
+  // Runs of chunks per item (jobs without the fine-chunked tail): the chunks are
+  // the job's own, so results do not depend on it; items of a few hundred
+  // particles or more spread their fixed costs (kBatchItemsPerCta).
+  long long total = 0;  // particles x tiles over all jobs
+  for (const Plan& q : plan) total += q.n * q.js.n_tiles;
+  const long long per_item = total / ((long long)kBatchItemsPerCta * resident_ctas(variant));
+  auto run_of = [&](const Plan& q) {
+    if (q.tail.tiles() > 0) return 1;
+    return (int)std::max<long long>(1, std::min<long long>(per_item, 1LL << 30) / q.ck);
+  };
+
   // Per-call table in the next pinned slot.
   const int s = slot;
   slot = (slot + 1) % kSlots;
   if (cudaEventSynchronize(slot_done[s]) != cudaSuccess) return RAD_ECUDA;
   long long items = 0;
   int blocks = 0, sort_blocks = 0;
+  unsigned red_blocks = 0;
   std::vector<rad_step> sorted(plan.size());
   for (size_t p = 0; p < plan.size(); ++p) {
     const rad_step& st = steps[plan[p].job];
@@ -195,11 +207,14 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
     K.dt = st.dt;
     K.ck = plan[p].ck;
     K.n_chunks = plan[p].n_chunks;
+    K.run = run_of(plan[p]);
     set_tail(K, plan[p].tail);
     K.item_begin = items;
     K.block_begin = blocks;
     K.sort_block_begin = sort_blocks;
-    items += plan[p].tail.items(plan[p].js.n_tiles, plan[p].n_chunks);
+    K.red_begin = red_blocks;
+    items += plan[p].tail.items(plan[p].js.n_tiles, (plan[p].n_chunks + K.run - 1) / K.run);
+    red_blocks += (unsigned)reduce_blocks(plan[p].js);
     blocks += (int)((st.n + 255) / 256);
     sort_blocks += (int)((st.n + kSortBlock - 1) / kSortBlock);
   }
@@ -221,9 +236,10 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
     if (e == cudaSuccess) e = launch_prepass(a, blocks, st);
     if (e == cudaSuccess) e = launch_wide(a, sort_blocks, blocks, st);
     if (e == cudaSuccess) e = launch_accumulate(variant, a, grid, st);
+    if (e == cudaSuccess) e = launch_reduce(a, red_blocks, st);
     return e;
   };
-  // kernels per round: pre-pass, the wide-call kernels, both accumulate kernels
+  // kernels per round: pre-pass, the wide-call kernels, accumulate, reduction
   const int launches = 1 + kWideLaunches + 2;
 
   // Order after the caller's stream (its inputs), run on the internal stream.

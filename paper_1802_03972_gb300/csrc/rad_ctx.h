@@ -44,8 +44,6 @@ struct rad_ctx {
   double push_t[3] = {0, 0, 0}, push_dt[3] = {0, 0, 0};
   float* d_state_p = nullptr;    // literal mode: [8][n_bins]
   float* d_f2 = nullptr;         // literal mode: [n_omega] f(omega)^2
-  unsigned* d_tile_cnt = nullptr;
-  int tile_cnt_cap = 0;
   double* d_stage = nullptr;     // staging for host particle arrays
   size_t stage_cap = 0;
   radimpl::JobStatic h_js{};     // host mirror of d_js

@@ -89,16 +89,28 @@ __device__ __forceinline__ void tma_load_1d(void* dst, const void* src, uint32_t
       : "memory");
 }
 
-// Job of a global work item (jobs ordered by item_begin).
-__device__ __forceinline__ int find_job(const LaunchArgs& a, long long item) {
+// Job of a global work item (jobs ordered by item_begin), by a whole warp: each
+// lane counts the jobs of its share that begin at or before the item
+// (independent loads, one round trip).
+__device__ __forceinline__ int find_job_warp(const LaunchArgs& a, long long item) {
   if (a.n_jobs == 1) return 0;
-  int lo = 0, hi = a.n_jobs - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (a.jc[mid].item_begin <= item) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
+  int n = 0;
+  for (int i = threadIdx.x & 31; i < a.n_jobs; i += 32) n += a.jc[i].item_begin <= item;
+  return __reduce_add_sync(0xffffffffu, n) - 1;
+}
+
+// Programmatic dependent launch: the next kernel of the stream may be set up
+// once every block of this one has called pdl_trigger (or left); it then waits
+// in pdl_wait until this one is complete and its writes are visible.  Every
+// kernel of a call's chain waits before it leaves, so completion is transitive.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Copies a struct of 8-byte words with the whole block (src: global or parameter space).
+template <int THREADS>
+__device__ __forceinline__ void copy_words(void* dst, const void* src, int bytes) {
+  for (int i = threadIdx.x; i < bytes / 8; i += THREADS)
+    reinterpret_cast<unsigned long long*>(dst)[i] = reinterpret_cast<const unsigned long long*>(src)[i];
 }
 
 // Job of a pre-pass block (jobs ordered by block_begin).

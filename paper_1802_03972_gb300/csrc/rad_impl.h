@@ -29,10 +29,11 @@ constexpr int kRecFields = 20;
 constexpr int kComps = 8;
 constexpr int kDirTab = 12;
 constexpr int kOmTab = 3;
-// Work items hold a multiple of 256 macro-particles: a whole number of
-// shared-memory tiles (threads / directions-per-tile particles) for every
-// kernel variant and tile shape.
+// Chunks hold a multiple of 256 macro-particles, or a power of two below that
+// (small calls): no shared-memory tile (threads / directions-per-tile particles
+// at most) then crosses a 256-particle group of a wide call.
 constexpr int kChunkAlign = 256;
+constexpr int kSmallestChunk = 32;
 // Levels of fine-chunked last tiles (TailPlan).
 constexpr int kTailLevels = 2;
 // Automatic chunking aims at this many (coarse) work items per resident
@@ -54,6 +55,12 @@ constexpr int kItemsPerCtaUniform = 24;
 // spread: on the batched job mix of small jobs this measured 1 % faster.
 constexpr int kMinChunk = 2048;
 static_assert(kMinChunk % kChunkAlign == 0, "the minimum chunk is a whole number of tiles");
+// Small calls (auto_chunk_for): an item's fixed cost in units of one particle
+// of a tile.
+constexpr int kItemCost = 60;
+// A batch hands out runs of consecutive chunks as one work item: about this
+// many items per resident block over all its jobs.
+constexpr int kBatchItemsPerCta = 5;
 
 // Wide calls (particles farther than half the fast phase range from the
 // call's reference point): a stable bucket sort along the grid's mean
@@ -63,10 +70,12 @@ static_assert(kMinChunk % kChunkAlign == 0, "the minimum chunk is a whole number
 // each sorted kGroup-particle group; the accumulate kernel rotates each tile's
 // sums by the group's reference phase.
 constexpr int kSortBlock = 2048;
-// A context's counter block (unsigned long long words, zeroed before every
-// call): [0], [1] the two accumulate kernels' work-item counters, [2] the
-// call's wide flag (an int).
-constexpr int kCounterWords = 3;
+// A context's counter block (unsigned long long words, zero between calls: the
+// last block of the accumulate kernel to leave zeroes it):
+// [0], [1] the accumulate kernel's work-item counters for ordinary and wide
+// calls, [2] the call's wide flag (an int), [3] the count of blocks that have left.
+constexpr int kCounterWords = 4;
+constexpr int kCounterExit = 3;
 constexpr int kSortBuckets = 4096;
 constexpr int kGroup = 256;
 static_assert(kGroup == kChunkAlign, "a work item holds whole sorted groups");
@@ -98,7 +107,6 @@ struct JobStatic {
   // fine_cap floats
   float* partials_f;
   long long fine_cap;
-  unsigned* tile_cnt;             // [n_tiles] arrival counters (self-resetting)
   float* rec;
   double* ref;                    // [4]: reference position xyz, t (per call)
   int* status;
@@ -128,11 +136,13 @@ struct JobCall {
   const double* bdot;
   const double* w;
   double t, dt;
-  int ck;                // macro-particles per work item (multiple of kChunkAlign)
+  int ck;                // macro-particles per chunk (see kChunkAlign)
   int n_chunks;
+  int run;               // consecutive chunks per (coarse) work item
   long long item_begin;  // first global work item of this job
   int block_begin;       // first pre-pass block of this job
   int sort_block_begin;  // first sort-histogram block of this job
+  unsigned red_begin;    // first block of this job in the tile reduction
   // Fine-chunked last tiles (TailPlan), level 0 then level 1 in tile order
   // (level 1 the job's last tail_tiles[1] tiles): tail_tiles[l] tiles with
   // chunks of ck_f[l] (n_chunks_f[l] per tile)
@@ -218,15 +228,14 @@ struct LaunchArgs {
   int n_jobs;
   int use_inline;        // 1: single job, call passed by value below
   long long n_items;
-  // [2] work-item counters: [0] the kernel for ordinary calls, [1] the kernel
-  // for wide calls (both zeroed before the launch)
+  // the counter block (kCounterWords), zero before the launch
   unsigned long long* item_counter;
   JobCall inline_call;
   // Profiling only (else null): [0] SM clock cycles and [1] nanoseconds, each
   // summed over the accumulate CTAs' lifetimes.
   unsigned long long* prof_clk;
   // Set (non-zero) by the pre-pass when some job's call is wide; null when no
-  // job can be (the wide kernels are then not launched).
+  // job can be (the wide-call kernels are then not launched).
   int* any_wide;
 };
 
@@ -261,6 +270,26 @@ inline Variant variant_info(int v) {
 }
 // Tensor-core (mma.sync) accumulation variants.
 inline bool variant_tensor_core(int v) { return v == 3 || v == 4 || v == 7 || v == 8 || v == 9; }
+
+#ifdef __CUDACC__
+// Launches a kernel of a call's chain with programmatic dependent launch (see
+// pdl_trigger): its set-up overlaps the kernel before it.
+template <class Kernel, class Args>
+inline cudaError_t launch_pdl(Kernel k, long long grid, int threads, size_t smem, cudaStream_t s,
+                              const Args& a) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, a);
+}
+#endif
 cudaError_t launch_readout_literal(const float* state_p, int n_bins, double* out, cudaStream_t s);
 
 // Launchers (rad_kernels.cu). All enqueue on `s` and return the launch error.
@@ -274,9 +303,11 @@ constexpr int kWideLaunches = 4;
 // Sort axis and bucket width of a job (host, at creation).
 void wide_geometry(const double* unit_dirs, int n_dir, float tau_fast, double axis[3],
                    double* cone_sin, double* bucket_w);
-// Launches the accumulate kernel for ordinary calls and, when a.any_wide is
-// set, the one for wide calls after it (one or two launches).
+// Launches the accumulate kernel, and the reduction of its partial sums into the
+// states (blocks: reduce_blocks summed over the jobs).
 cudaError_t launch_accumulate(int variant, const LaunchArgs& a, int grid, cudaStream_t s);
+cudaError_t launch_reduce(const LaunchArgs& a, long long blocks, cudaStream_t s);
+int reduce_blocks(const JobStatic& js);
 int accumulate_blocks_per_sm(int variant);
 // Per-device caches of launch properties cover device ordinals below this.
 constexpr int kMaxDevices = 64;

@@ -78,7 +78,8 @@ __device__ __forceinline__ void store_record(float* dst_rec, const float v[kRecF
     dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
 }
 
-__global__ void __launch_bounds__(256) prepass_kernel(LaunchArgs a) {
+__global__ void __launch_bounds__(256) prepass_kernel(const __grid_constant__ LaunchArgs a) {
+  dev::pdl_trigger();
   const int j = dev::find_job_block(a, blockIdx.x);
   const JobStatic& J = a.js[j];
   const JobCall K = a.use_inline ? a.inline_call : a.jc[j];
@@ -155,7 +156,9 @@ __device__ __forceinline__ int find_job_sort_block(const LaunchArgs& a, int bloc
 }
 
 // Per kSortBlock particles: bucket counts.
-__global__ void __launch_bounds__(256) wide_hist_kernel(LaunchArgs a) {
+__global__ void __launch_bounds__(256) wide_hist_kernel(const __grid_constant__ LaunchArgs a) {
+  dev::pdl_trigger();
+  dev::pdl_wait();
   const int j = find_job_sort_block(a, blockIdx.x);
   const JobStatic& J = a.js[j];
   if (!call_is_wide(J)) return;
@@ -174,7 +177,9 @@ __global__ void __launch_bounds__(256) wide_hist_kernel(LaunchArgs a) {
 
 // One block per job: per bucket, the prefix of the counts over the histogram
 // blocks (in place), and the first sorted position of every bucket.
-__global__ void __launch_bounds__(1024) wide_scan_kernel(LaunchArgs a) {
+__global__ void __launch_bounds__(1024) wide_scan_kernel(const __grid_constant__ LaunchArgs a) {
+  dev::pdl_trigger();
+  dev::pdl_wait();
   const JobStatic& J = a.js[blockIdx.x];
   if (!call_is_wide(J)) return;
   const JobCall K = a.use_inline ? a.inline_call : a.jc[blockIdx.x];
@@ -235,7 +240,9 @@ __global__ void __launch_bounds__(1024) wide_scan_kernel(LaunchArgs a) {
 // (particles of one bucket keep their order), so the order is a function of
 // the input alone.  The block computes the buckets into shared memory, then
 // one warp hands out the positions in particle order.
-__global__ void __launch_bounds__(256) wide_scatter_kernel(LaunchArgs a) {
+__global__ void __launch_bounds__(256) wide_scatter_kernel(const __grid_constant__ LaunchArgs a) {
+  dev::pdl_trigger();
+  dev::pdl_wait();
   const int j = find_job_sort_block(a, blockIdx.x);
   const JobStatic& J = a.js[j];
   if (!call_is_wide(J)) return;
@@ -273,7 +280,9 @@ __global__ void __launch_bounds__(256) wide_scatter_kernel(LaunchArgs a) {
 // Records in sorted order, positions relative to the first particle of each
 // kGroup-particle group (its reference point); the group references relative
 // to the call's reference go to gref.
-__global__ void __launch_bounds__(256) wide_records_kernel(LaunchArgs a) {
+__global__ void __launch_bounds__(256) wide_records_kernel(const __grid_constant__ LaunchArgs a) {
+  dev::pdl_trigger();
+  dev::pdl_wait();
   const int j = dev::find_job_block(a, blockIdx.x);
   const JobStatic& J = a.js[j];
   if (!call_is_wide(J)) return;
@@ -649,12 +658,12 @@ cudaError_t launch_prepass(const LaunchArgs& a, int total_blocks, cudaStream_t s
 
 cudaError_t launch_wide(const LaunchArgs& a, int sort_blocks, int prepass_blocks, cudaStream_t s) {
   if (sort_blocks <= 0 || prepass_blocks <= 0) return cudaSuccess;
-  wide_hist_kernel<<<sort_blocks, 256, 0, s>>>(a);
-  wide_scan_kernel<<<a.n_jobs, 1024, 0, s>>>(a);
-  wide_scatter_kernel<<<sort_blocks, 256, 0, s>>>(a);
-  wide_records_kernel<<<prepass_blocks, 256, 0, s>>>(a);
+  cudaError_t e = launch_pdl(wide_hist_kernel, sort_blocks, 256, 0, s, a);
+  if (e == cudaSuccess) e = launch_pdl(wide_scan_kernel, a.n_jobs, 1024, 0, s, a);
+  if (e == cudaSuccess) e = launch_pdl(wide_scatter_kernel, sort_blocks, 256, 0, s, a);
+  if (e == cudaSuccess) e = launch_pdl(wide_records_kernel, prepass_blocks, 256, 0, s, a);
   count_launches(kWideLaunches);
-  return cudaGetLastError();
+  return e;
 }
 
 void wide_geometry(const double* nd, int n_dir, float tau_fast, double axis[3], double* cone_sin,

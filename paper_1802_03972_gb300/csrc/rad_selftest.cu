@@ -126,6 +126,9 @@ rad_status rad_selftest_stage1(rad_ctx* c, int64_t n, const double* r, const dou
   K.ck = (int)std::min<int64_t>(n, 1 << 30);
   K.n_chunks = 1;
   s = cuda_check(c, launch_prepass(a, (int)((n + 255) / 256), c->stream));
+  // (no accumulate kernel follows to clear a wide flag)
+  if (s == RAD_OK)
+    s = cuda_check(c, cudaMemsetAsync(c->d_counter, 0, kCounterWords * sizeof(unsigned long long), c->stream));
   if (s != RAD_OK) return s;
   float* d_out = nullptr;
   s = cuda_check(c, cudaMalloc(&d_out, sizeof(float) * 8 * (size_t)n));

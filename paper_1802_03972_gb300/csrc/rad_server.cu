@@ -77,10 +77,13 @@ size_t estimate_footprint(const rad_job_desc& d) {
   // at kItemsPerCta work items per resident block with the fine-chunked tail
   // and kItemsPerCtaUniform (the larger) without it; with B bins per tile,
   // chunks x bins <= kItemsPerCtaUniform x resident blocks x B + bins.  There
-  // are also never more chunks than 256-particle groups.
+  // are also never more chunks than 256-particle groups, except for a small
+  // call's, which fit one wave: chunks x bins <= resident blocks x B.
   const Variant v = variant_info(kDefaultVariant);
   const size_t bins_per_tile = (size_t)v.threads * v.w * v.passes;
-  const size_t by_particles = nb * (size_t)((d.max_particles + kChunkAlign - 1) / kChunkAlign);
+  const size_t by_particles =
+      std::max(nb * (size_t)((d.max_particles + kChunkAlign - 1) / kChunkAlign),
+               (size_t)resident_ctas(kDefaultVariant) * bins_per_tile);
   const size_t by_items = (size_t)kItemsPerCtaUniform * resident_ctas(kDefaultVariant) * bins_per_tile + nb;
   const size_t partials = 32 * std::min(by_particles, by_items);
   // The fine-chunked last tiles' partial sums (TailPlan), 32 B per tile bin
