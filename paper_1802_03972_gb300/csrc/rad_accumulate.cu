@@ -76,12 +76,16 @@ struct TileGeom {
 
 __device__ __forceinline__ TileGeom tile_geom(const JobStatic& J, int tile, int threads) {
   TileGeom g;
-  g.WT = J.wt;
-  g.NT = J.nt;
+  int s = 0;
+  while (s + 1 < J.n_seg && tile >= J.seg[s + 1].tile0) ++s;
+  const TileSeg& sg = J.seg[s];
+  g.WT = sg.wt;
+  g.NT = sg.nt;
   g.KT = threads / g.NT;
-  const int tile_d = tile / J.tiles_om;
+  tile -= sg.tile0;
+  const int tile_d = tile / sg.tiles_om;
   g.d0 = tile_d * g.NT;
-  g.o0 = (tile - tile_d * J.tiles_om) * g.WT;
+  g.o0 = sg.o0 + (tile - tile_d * sg.tiles_om) * g.WT;
   return g;
 }
 
@@ -982,7 +986,7 @@ __global__ void __launch_bounds__(kRedThreads) reduce_kernel(const __grid_consta
   __syncthreads();
   const JobStatic& J = b.J;
   const JobCall& K = b.K;
-  const int per_tile = J.nt * J.wt / kRedBins;
+  const int per_tile = J.bpt / kRedBins;
   const long long local = (long long)blockIdx.x - K.red_begin;
   ItemRef it;
   int s;
@@ -1105,7 +1109,7 @@ int blocks_per_sm() {
 
 }  // namespace
 
-int reduce_blocks(const JobStatic& js) { return js.n_tiles * (js.nt * js.wt / kRedBins); }
+int reduce_blocks(const JobStatic& js) { return js.n_tiles * (js.bpt / kRedBins); }
 
 cudaError_t launch_reduce(const LaunchArgs& a, long long blocks, cudaStream_t s) {
   count_launches(1);

@@ -121,7 +121,7 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
     // chunked as the job alone would be (results equal bit for bit)
     const TailPlan tail = tail_plan(variant_tensor_core(variant) && !js.literal, steps[i].n,
                                     js.n_tiles, ck, nch, resident_ctas(variant));
-    const long long fine = tail.fine_floats(js.nt * js.wt);
+    const long long fine = tail.fine_floats(js.bpt);
     if (steps[i].n > c->h_js.n_cap || nch > c->h_js.chunk_cap || fine > c->h_js.fine_cap) {
       if (!drained) {
         if (cudaStreamSynchronize(work) != cudaSuccess) return RAD_ECUDA;

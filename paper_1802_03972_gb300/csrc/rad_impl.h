@@ -60,7 +60,7 @@ static_assert(kMinChunk % kChunkAlign == 0, "the minimum chunk is a whole number
 constexpr int kItemCost = 60;
 // A batch hands out runs of consecutive chunks as one work item: about this
 // many items per resident block over all its jobs.
-constexpr int kBatchItemsPerCta = 5;
+constexpr int kBatchItemsPerCta = 8;
 
 // Wide calls (particles farther than half the fast phase range from the
 // call's reference point): a stable bucket sort along the grid's mean
@@ -87,11 +87,19 @@ static_assert(kGroup == kChunkAlign, "a work item holds whole sorted groups");
 // skipped.
 enum : int { ST_BAD_PARTICLE = 1, ST_SLOW_PHASE = 2, ST_TIMEOUT = 4, ST_BOUNDS = 8, ST_BAD_GRID = 16 };
 
+// A segment of the frequency range, from frequency o0: tiles_om tiles of wt
+// frequencies x nt directions, for all directions; tile0: its first tile.
+struct TileSeg {
+  int tile0, o0, wt, nt, tiles_om;
+};
+constexpr int kMaxSegs = 4;  // one per tile width: a block's 8, 4, 2 and 1 warps per direction
+
 // Per-job data that does not change between calls.
 struct JobStatic {
   int n_omega, n_dir, n_bins;
-  int wt, nt;                     // tile: wt frequencies x nt directions
-  int tiles_om, tiles_dir, n_tiles;
+  // bin tiles of bpt bins each, in segments of the frequency range (fill_tiles)
+  int bpt, n_tiles, n_seg;
+  TileSeg seg[kMaxSegs];
   float tau_fast;                 // |delta tau| bound of the fast phase path, s
   int chunk_cap;                  // capacity of partials, in chunks
   long long n_cap;                // capacity of rec, in particles

@@ -83,3 +83,14 @@ def test_accumulate_replayed_from_a_captured_graph(n):
     torch.cuda.synchronize()
     for x, y in zip(direct.spectrum(), ctx.spectrum()):
         np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("variant", [0, 2, 7, 9])
+@pytest.mark.parametrize("n_omega,n_dir", [(65, 8), (150, 3), (300, 9), (330, 2), (450, 1), (520, 5), (800, 11), (850, 1)])
+def test_frequency_segments_of_every_width(n_omega, n_dir, variant):
+    """Frequency counts that leave 1 to 7 warps' worth past the last full tile: covered by narrower tiles."""
+    wl = workload(500, n_omega, n_dir)
+    ctx = gpu_run(wl, range(2), tile=(variant, 0, 0))
+    ref = spectra_grid(oracle_run(wl, range(2)), wl)
+    for k, g in zip(("coh", "inc", "tot"), ctx.spectrum()):
+        assert_parity(g, ref[k], what=k)
