@@ -47,6 +47,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include "rad_device.cuh"
@@ -587,25 +588,12 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
                                  th, tl, a);
       }
       // Particles past kn are zero padding of the last 8-particle MMA step.
-      const int slot = s1_dl * g.KT + s1_kk;
-      const uint32_t h0 = tf32_hi(a[0]), h1 = tf32_hi(a[1]), h2 = tf32_hi(a[2]), h3 = tf32_hi(a[3]);
       if constexpr (XT) {
-        xth[slot] = th;
-        uint32_t thh, thl, tlh, tll;
-        split_tf32(th, thh, thl);
-        split_tf32(tl, tlh, tll);
-        float4* rp = reinterpret_cast<float4*>(xrt + (size_t)slot * 8);
-        const int sw = (s1_kk >> 2) & 1;  // pairs 0, 1 and 2, 3 swap places
-        rp[sw] = make_float4(__uint_as_float(thh), __uint_as_float(tll), __uint_as_float(thl),
-                             __uint_as_float(tlh));
-        rp[sw ^ 1] = make_float4(__uint_as_float(thh), __uint_as_float(thl),
-                                 __uint_as_float(tlh), __uint_as_float(tll));
-        float4* ap = reinterpret_cast<float4*>(xam + (size_t)slot * 12);
-        ap[0] = make_float4(__uint_as_float(h0), __uint_as_float(h1), __uint_as_float(h2),
-                            __uint_as_float(h3));
-        ap[1] = make_float4(a[0] - __uint_as_float(h0), a[1] - __uint_as_float(h1),
-                            a[2] - __uint_as_float(h2), a[3] - __uint_as_float(h3));
+        store_record_xt(th, tl, a, s1_kk, xth + s1_dl * g.KT, xrt + (size_t)s1_dl * g.KT * 8,
+                        xam + (size_t)s1_dl * g.KT * 12);
       } else {
+        const int slot = s1_dl * g.KT + s1_kk;
+        const uint32_t h0 = tf32_hi(a[0]), h1 = tf32_hi(a[1]), h2 = tf32_hi(a[2]), h3 = tf32_hi(a[3]);
         tau2[slot] = make_float2(th, tl);
         float4* ap = reinterpret_cast<float4*>(ampb + (size_t)slot * 8);
         ap[0] = make_float4(__uint_as_float(h0), __uint_as_float(h1), __uint_as_float(h2),
@@ -820,6 +808,257 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
   return true;
 }
 
+// ------------------------------------------------------------------ low band
+// One item of a call's low band (LowSet): 8 directions, one per warp, and a chunk
+// of the cell-sorted particles.  A warp's 64 frequencies are the nodes; its
+// records are relative to the cell's centre and weighted by the interpolation's
+// particle-side factor.  Warps share only the raw particles (two buffers of
+// kLowTile, one barrier each): every warp computes its own direction's
+// records.  At a cell's end the warp interpolates its node sums to the
+// band's bins, rotates them by e^{i omega tau_c} (tau_c the centre's time) and
+// adds them to the chunk's sums.  Bound: MUFU, as the direct bins, for 64
+// frequencies instead of js; the interpolation is 10 taps x 8 sums per bin and
+// cell.  LWFA step (1e5 particles, 512 x 256 bins, 256 bins from nodes): 6.79 ->
+// 4.93 ms; 1e6 particles, 1024 x 256 bins (512 from nodes) 132.2 -> 77.4 ms.
+constexpr int kLowTile = 128;
+constexpr int kLowDirs = 8;
+
+struct LowTile {
+  long long pos;  // first particle (sorted)
+  int kn, cell;
+  int last;       // ends its cell or the chunk
+};
+
+// The tile from pos in `cell`, whose particles end at cell_end.
+__device__ __forceinline__ LowTile low_tile(long long pos, long long cell_end, int cell) {
+  LowTile t;
+  t.pos = pos;
+  t.kn = (int)min((long long)kLowTile, cell_end - pos);
+  t.cell = cell;
+  t.last = pos + t.kn == cell_end;
+  return t;
+}
+
+// Particle-side factor of the interpolation, 1 / (the window's Fourier transform
+// at x / (2 kLowOversample), x = tau / H): a polynomial in x^2 fitted to
+// quadratures of the transform (relative error 1e-7 in FP32 on |x| <= 1).
+__device__ __forceinline__ float low_factor(float x) {
+  const float y = x * x;
+  float p = 0.00316812399f;
+  p = fmaf(p, y, -0.00347217099f);
+  p = fmaf(p, y, 0.0177691517f);
+  p = fmaf(p, y, 0.0227779421f);
+  p = fmaf(p, y, 0.0826435269f);
+  p = fmaf(p, y, 0.189933115f);
+  p = fmaf(p, y, 0.381905146f);
+  p = fmaf(p, y, 0.599662798f);
+  p = fmaf(p, y, 0.657055849f);
+  return fmaf(p, y, 0.376632672f);
+}
+
+template <int THREADS>
+__device__ __forceinline__ bool process_item_low(const JobStatic& J, const JobCall& K, const LowPlan& P,
+                                                 const LowSet& L, int tile, int chunk, LowTile* desc,
+                                                 unsigned char* __restrict__ smem, uint64_t* bars,
+                                                 uint32_t& phases) {
+  constexpr int NB = kLowNodes / 16, GQ = 2 * NB;
+  static_assert(THREADS / 32 == kLowDirs, "one direction per warp");
+  using S = Smem<THREADS, true, false, NB / 2, true>;
+  static_assert(2 * kLowTile * kRecFields * sizeof(float) <= S::raw_bytes, "two raw tiles");
+  static_assert(kLowDirs * kLowNodes * kComps * sizeof(float) <= S::rec_bytes, "node sums");
+  float* raw = reinterpret_cast<float*>(smem);
+  unsigned char* recb = smem + S::raw_bytes;
+  float4* l2 = reinterpret_cast<float4*>(smem + S::raw_bytes + 2 * S::rec_bytes);
+  float* sdir = reinterpret_cast<float*>(smem + S::raw_bytes + 2 * S::rec_bytes + S::l2_bytes);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r = lane >> 2, c = lane & 3;
+  float* ns = reinterpret_cast<float*>(smem + S::raw_bytes + S::rec_bytes) + warp * kLowNodes * kComps;
+  float* xth = reinterpret_cast<float*>(recb) + warp * 32;
+  float* xrt = reinterpret_cast<float*>(recb + (size_t)THREADS * 4) + warp * 32 * 8;
+  float* xam = reinterpret_cast<float*>(recb + (size_t)THREADS * 36) + warp * 32 * 12;
+  const int my_d = min(tile * kLowDirs + warp, J.n_dir - 1);
+  const bool live = tile * kLowDirs + warp < J.n_dir;
+  const int ck = K.low[P.set].ck_lo;
+  const long long k0 = (long long)chunk * ck, k1 = min(k0 + ck, K.n);
+
+  for (int t = lane; t < 12; t += 32) sdir[warp * 12 + t] = __ldg(J.dir_tab + (size_t)t * J.n_dir + my_d);
+  auto issue = [&](const LowTile& t, int buf) {
+    if (!bounds_ok(t.pos + t.kn <= J.n_cap, J.status)) return;
+    tma_load_1d(raw + (size_t)buf * kLowTile * kRecFields, J.rec_s + (size_t)t.pos * kRecFields,
+                (uint32_t)t.kn * kRecFields * sizeof(float), &bars[buf]);
+  };
+  // first sorted position after the cell's particles, within the chunk
+  auto cell_end = [&](int cell) {
+    return cell + 1 < P.cells ? min((long long)J.bucket_base[cell + 1], k1) : k1;
+  };
+  if (threadIdx.x == 0) {
+    int lo = 0, hi = P.cells - 1;  // the last cell that begins at or before k0
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (J.bucket_base[mid] <= k0) lo = mid;
+      else hi = mid - 1;
+    }
+    desc[0] = low_tile(k0, cell_end(lo), lo);
+    issue(desc[0], 0);
+  }
+  // the nodes' frequency factors, as load_omega's
+  float2 omr[NB], omr8[NB];
+  uint32_t xa[NB][4];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = 16 * b + r + 8 * h;
+      const float h0 = __ldg(L.nodes + i);
+      (h ? omr8 : omr)[b] = make_float2(h0, h0);
+      uint32_t whh, whl, wlh, wll;
+      split_tf32(__ldg(L.nodes + kLowNodes + i), whh, whl);
+      split_tf32(__ldg(L.nodes + 2 * kLowNodes + i), wlh, wll);
+      xa[b][h] = c == 3 ? whh : (c == 2 ? wll : wlh);
+      xa[b][2 + h] = c == 0 ? whh : (c == 2 ? wll : whl);
+    }
+  }
+  float dre[NB][4], dim[NB][4];
+#pragma unroll
+  for (int b = 0; b < NB; ++b)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) dre[b][e] = dim[b][e] = 0.0f;
+#pragma unroll
+  for (int v = 0; v < GQ; ++v) l2[v * THREADS + threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int xr_off = 2 * (c ^ ((r >> 1) & 2));
+  float* part = J.partials_l + (size_t)chunk * kComps * J.n_dir * L.js + (size_t)my_d * L.js;
+  const size_t cs = (size_t)J.n_dir * L.js;
+  const bool slot = bounds_ok((chunk + 1) * (long long)(kComps * cs) <= J.low_cap, J.status);
+  bool first = true;  // the chunk's first cell starts its sums
+  int cell = -1;
+  float tch = 0.0f, tcl = 0.0f;
+  const float inv_h = 1.0f / L.H;
+  __syncthreads();
+  for (int buf = 0;; buf ^= 1) {
+    const LowTile t = desc[buf];
+    // the next tile, into the other buffer (used up before the last barrier)
+    const long long next = t.pos + t.kn;
+    if (threadIdx.x == 0 && next < k1) {
+      int nc = t.cell;
+      long long ce = cell_end(nc);
+      while (ce <= next) ce = cell_end(++nc);  // (past empty cells)
+      desc[buf ^ 1] = low_tile(next, ce, nc);
+      issue(desc[buf ^ 1], buf ^ 1);
+    }
+    if (t.cell != cell) {
+      cell = t.cell;
+      const double sc = (double)P.s0 + ((double)cell + 0.5) * (double)P.h;
+      const double* nd = J.dirs + 3 * (size_t)my_d;
+      double tc = 0.0;
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+        tc -= nd[i] * ((double)P.c1 * J.fr1[i] + (double)P.c2 * J.fr2[i] + sc * J.axis[i]);
+      split_ff(tc, tch, tcl);
+    }
+    const bool landed = mbar_wait(&bars[buf], (phases >> buf) & 1u);
+    phases ^= 1u << buf;
+    if (landed) {
+      for (int s0 = 0; s0 < t.kn; s0 += 32) {
+        const int kn = min(32, t.kn - s0);
+        float th = 0.f, tl = 0.f, a[4] = {0.f, 0.f, 0.f, 0.f};
+        if (lane < kn) {
+          compute_record(raw + ((size_t)buf * kLowTile + s0 + lane) * kRecFields,
+                         dir_row_staged(sdir + 12 * warp), J.tau_fast, th, tl, a);
+          // relative to the cell's centre (TwoDiff)
+          const float d = __fsub_rn(th, tch), bb = __fsub_rn(d, th);
+          const float e = __fsub_rn(__fsub_rn(th, __fsub_rn(d, bb)), __fadd_rn(tch, bb));
+          const float lo = __fadd_rn(e, __fsub_rn(tl, tcl));
+          th = __fadd_rn(d, lo);
+          tl = __fsub_rn(lo, __fsub_rn(th, d));
+          const float f = low_factor(th * inv_h);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) a[i] *= f;
+        }
+        store_record_xt(th, tl, a, lane, xth, xrt, xam);
+        __syncwarp();
+        const int kn8 = (kn + 7) & ~7;
+        if (kn8 == 32) {
+#pragma unroll
+          for (int kk = 0; kk < 32; kk += 8)
+            xt_step<NB>(xth, xrt, xam, kk, r, c, xr_off, omr, omr8, xa, dre, dim);
+        } else {
+#pragma unroll 1
+          for (int kk = 0; kk < kn8; kk += 8)
+            xt_step<NB>(xth, xrt, xam, kk, r, c, xr_off, omr, omr8, xa, dre, dim);
+        }
+        __syncwarp();
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      float4* p = l2 + b * THREADS + threadIdx.x;
+      float4* q = p + NB * THREADS;
+      const float4 x = *p, y = *q;
+      *p = make_float4(x.x + dre[b][0], x.y + dre[b][1], x.z + dre[b][2], x.w + dre[b][3]);
+      *q = make_float4(y.x + dim[b][0], y.y + dim[b][1], y.z + dim[b][2], y.w + dim[b][3]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) dre[b][e] = dim[b][e] = 0.0f;
+    }
+    if (t.last && live && slot) {
+      // node sums, hi and lo parts together (lane c < 2 holds columns 2c, 2c + 1)
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {
+        const float4 re4 = l2[b * THREADS + threadIdx.x], im4 = l2[(NB + b) * THREADS + threadIdx.x];
+        l2[b * THREADS + threadIdx.x] = l2[(NB + b) * THREADS + threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float re[4] = {re4.x, re4.y, re4.z, re4.w}, im[4] = {im4.x, im4.y, im4.z, im4.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float vr = re[e] + __shfl_xor_sync(0xffffffffu, re[e], 2);
+          const float vi = im[e] + __shfl_xor_sync(0xffffffffu, im[e], 2);
+          if (c < 2)
+            *reinterpret_cast<float2*>(ns + (16 * b + r + 8 * (e >> 1)) * kComps + 2 * (2 * c + (e & 1))) =
+                make_float2(vr, vi);
+        }
+      }
+      __syncwarp();
+#pragma unroll 1
+      for (int j = lane; j < L.js; j += 32) {
+        const float4* wt = reinterpret_cast<const float4*>(L.wts + (size_t)j * kLowWt);
+        const float4 w0 = __ldg(wt), w1 = __ldg(wt + 1), w2 = __ldg(wt + 2);
+        const float w[kLowTaps] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w, w2.x, w2.y};
+        const float4* p = reinterpret_cast<const float4*>(ns) + 2 * __float_as_int(w2.z);
+        float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u;
+#pragma unroll
+        for (int k = 0; k < kLowTaps; ++k) {
+          const float4 x = p[2 * k], y = p[2 * k + 1];
+          u.x = fmaf(w[k], x.x, u.x), u.y = fmaf(w[k], x.y, u.y), u.z = fmaf(w[k], x.z, u.z), u.w = fmaf(w[k], x.w, u.w);
+          v.x = fmaf(w[k], y.x, v.x), v.y = fmaf(w[k], y.y, v.y), v.z = fmaf(w[k], y.z, v.z), v.w = fmaf(w[k], y.w, v.w);
+        }
+        const float oh = __ldg(J.om_tab + j), wh = __ldg(J.om_tab + J.n_omega + j),
+                    wl = __ldg(J.om_tab + 2 * J.n_omega + j);
+        const float2 ph = phase2(make_float2(oh, oh), make_float2(wh, wh), make_float2(wl, wl),
+                                 make_float2(tch, tch), make_float2(tcl, tcl));
+        const float cp = cos_approx(ph.x), sp = sin_approx(ph.x);
+        const float sum[kComps] = {u.x * cp - u.y * sp, u.x * sp + u.y * cp, u.z * cp - u.w * sp, u.z * sp + u.w * cp,
+                                   v.x * cp - v.y * sp, v.x * sp + v.y * cp, v.z * cp - v.w * sp, v.z * sp + v.w * cp};
+#pragma unroll
+        for (int k = 0; k < kComps; ++k) {
+          float* o = part + k * cs + j;
+          __stcg(o, first ? sum[k] : __ldcg(o) + sum[k]);
+        }
+      }
+      first = false;
+      __syncwarp();
+    }
+    if (__syncthreads_or(landed ? 0 : 1)) {
+      // a copy did not land within the bound: record it, wait (bounded) for both
+      // buffers' copies in flight, and leave
+      if (threadIdx.x == 0) {
+        atomicOr(J.status, ST_TIMEOUT);
+        mbar_wait(&bars[buf], ((phases >> buf) & 1u) ^ 1u);
+        if (next < k1) mbar_wait(&bars[buf ^ 1], (phases >> (buf ^ 1)) & 1u);
+      }
+      return false;
+    }
+    if (next >= k1) return true;
+  }
+}
+
 // The block's shared state: the current item and its job (one round trip to
 // global memory per job instead of one per use).
 struct BlockState {
@@ -828,13 +1067,68 @@ struct BlockState {
   ItemShared it;
   long long item;          // -1: a pass's first item is still to come
   int job, cur_job;        // the item's job, and the one loaded (-1: none)
-  int any_wide;            // some job of the launch is wide
+  int any_wide, any_low;   // some job of the launch is wide, takes the low band
+  LowPlan plan;            // the job's low-band plan (set -1: none), and its alternative
+  LowSet low;
+  LowTile tiles[2];
 };
 
 template <int THREADS>
 __device__ __forceinline__ void load_job(BlockState& b, const LaunchArgs& a, int j) {
   copy_words<THREADS>(&b.J, &a.js[j], sizeof(JobStatic));
   copy_words<THREADS>(&b.K, a.use_inline ? &a.inline_call : &a.jc[j], sizeof(JobCall));
+}
+
+// One thread, once the kernels before this one are complete: the job's low-band
+// plan; a call that takes the band has its tiles over the other bins only,
+// chunked for them.
+__device__ __forceinline__ void settle_plan(BlockState& b) {
+  b.plan.set = -1;
+  if (!b.K.low_ok) return;
+  b.plan = *b.J.plan;
+  if (b.plan.set < 0) return;
+  b.low = b.J.low[b.plan.set];
+  const LowSet& L = b.low;
+  const LowCall& C = b.K.low[b.plan.set];
+  b.J.n_tiles = L.n_tiles;
+  b.J.n_seg = L.n_seg;
+  for (int i = 0; i < kMaxSegs; ++i) b.J.seg[i] = L.seg[i];
+  b.K.ck = C.ck_hi;
+  b.K.n_chunks = C.n_hi;
+  b.K.run = 1;
+  for (int l = 0; l < kTailLevels; ++l) b.K.tail_tiles[l] = 0;
+}
+
+// Claims the pass's next item (thread 0's counter; a block's first item is its
+// index) and finds its job, into b.item and b.job; by the first warp.
+__device__ __forceinline__ void claim_item(const LaunchArgs& a, BlockState& b, int counter, long long n_items,
+                                           bool low) {
+  long long item = blockIdx.x;
+  if (b.item >= 0) {
+    unsigned long long v = 0;
+    if (threadIdx.x == 0) v = atomicAdd(a.item_counter + counter, 1ULL);
+    item = (long long)(gridDim.x + __shfl_sync(0xffffffffu, v, 0));
+  }
+  const int j = item < n_items ? find_job_warp(a, item, low) : 0;
+  __syncwarp();
+  if (threadIdx.x == 0) {
+    b.item = item;
+    b.job = j;
+  }
+}
+
+// Loads the claimed item's job if it is another than the last.
+template <int THREADS>
+__device__ __forceinline__ void switch_job(const LaunchArgs& a, BlockState& b) {
+  if (b.job == b.cur_job) return;
+  __syncthreads();
+  load_job<THREADS>(b, a, b.job);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    b.cur_job = b.job;
+    settle_plan(b);
+  }
+  __syncthreads();
 }
 
 // The work items of the jobs whose call is not wide (WIDE = false) or is (true),
@@ -845,32 +1139,17 @@ __device__ __forceinline__ bool run_items(const LaunchArgs& a, BlockState& b, un
                                           uint64_t* bar, uint32_t& phase) {
   for (;;) {
     __syncthreads();  // the last item's shared state is used up
-    if (threadIdx.x < 32) {
-      long long item = blockIdx.x;  // a block's first item is its index, the others come from the counter
-      if (b.item >= 0) {
-        unsigned long long v = 0;
-        if (threadIdx.x == 0) v = atomicAdd(a.item_counter + (WIDE ? 1 : 0), 1ULL);
-        item = (long long)(gridDim.x + __shfl_sync(0xffffffffu, v, 0));
-      }
-      const int j = item < a.n_items ? find_job_warp(a, item) : 0;
-      __syncwarp();
-      if (threadIdx.x == 0) {
-        b.item = item;
-        b.job = j;
-      }
-    }
+    if (threadIdx.x < 32) claim_item(a, b, WIDE ? 1 : 0, a.n_items, false);
     __syncthreads();
     const long long item = b.item;
     if (item >= a.n_items) return true;
-    if (b.job != b.cur_job) {
-      __syncthreads();
-      if (threadIdx.x == 0) b.cur_job = b.job;
-      load_job<THREADS>(b, a, b.job);
-      __syncthreads();
-    }
+    switch_job<THREADS>(a, b);
     if (b.any_wide && (b.J.wide_flag != nullptr && *b.J.wide_flag != 0) != WIDE) continue;  // the other pass's
     // Tile-major order: one tile's chunks run close together in time.
-    const ItemRef it = decode_item<TC>(b.J, b.K, item - b.K.item_begin);
+    const long long local = item - b.K.item_begin;
+    // (a call with the low band may have fewer items than its share of the range)
+    if (XT && b.plan.set >= 0 && local >= (long long)b.J.n_tiles * b.K.n_chunks) continue;
+    const ItemRef it = decode_item<TC>(b.J, b.K, local);
     if (threadIdx.x == 0) {
       b.it.it = it;
       b.it.k_begin = (long long)it.chunk * it.ck;
@@ -885,10 +1164,30 @@ __device__ __forceinline__ bool run_items(const LaunchArgs& a, BlockState& b, un
   }
 }
 
+// The low bands' work items.
+template <int THREADS>
+__device__ __forceinline__ bool run_low(const LaunchArgs& a, BlockState& b, unsigned char* smem, uint64_t* bars) {
+  uint32_t phases = 0u;
+  for (;;) {
+    __syncthreads();  // the last item's shared state is used up
+    if (threadIdx.x < 32) claim_item(a, b, kCounterLow, a.n_items_low, true);
+    __syncthreads();
+    const long long item = b.item;
+    if (item >= a.n_items_low) return true;
+    switch_job<THREADS>(a, b);
+    if (b.plan.set < 0) continue;
+    int tile, chunk;
+    div_rem(item - b.K.low_begin, b.K.low[b.plan.set].n_lo, tile, chunk);
+    if (tile * kLowDirs >= b.J.n_dir) continue;
+    if (!process_item_low<THREADS>(b.J, b.K, b.plan, b.low, tile, chunk, b.tiles, smem, bars, phases)) return false;
+  }
+}
+
 template <int THREADS, int W, int MINB, bool TC, bool LIT, int PASSES = 1, bool XT = false>
 __global__ void __launch_bounds__(THREADS, MINB) accumulate_kernel(const __grid_constant__ LaunchArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t bar;
+  __shared__ __align__(8) uint64_t bars_low[2];
   __shared__ __align__(8) BlockState b;
   // Profiling: the block's start, kept in shared memory rather than in
   // registers live across the whole loop.
@@ -897,6 +1196,8 @@ __global__ void __launch_bounds__(THREADS, MINB) accumulate_kernel(const __grid_
   pdl_trigger();
   if (threadIdx.x == 0) {
     mbar_init(&bar, 1);
+    mbar_init(&bars_low[0], 1);
+    mbar_init(&bars_low[1], 1);
     mbar_fence_init();
   }
   // A single job's tables do not depend on the kernels before this one.
@@ -904,17 +1205,27 @@ __global__ void __launch_bounds__(THREADS, MINB) accumulate_kernel(const __grid_
   pdl_wait();
   // Whether any job of the launch is wide is final by now; without, the first
   // pass takes every item without looking at the jobs' flags.
+  if (a.n_jobs == 1) __syncthreads();
   if (threadIdx.x == 0) {
-    b.any_wide = a.any_wide != nullptr && *a.any_wide != 0;
+    b.any_wide = a.any_wide != nullptr && a.any_wide[0] != 0;
+    b.any_low = a.n_items_low > 0 && a.any_wide[1] != 0;
     b.cur_job = a.n_jobs == 1 ? 0 : -1;
     b.item = -1;
+    if (a.n_jobs == 1) settle_plan(b);
   }
   if (a.prof_clk && threadIdx.x == 0) {
     s_clk0 = clock64();
     s_ns0 = global_ns();
   }
   uint32_t phase = 0u;
-  const bool ok = run_items<THREADS, W, TC, LIT, PASSES, false, XT>(a, b, smem, &bar, phase);
+  bool ok = run_items<THREADS, W, TC, LIT, PASSES, false, XT>(a, b, smem, &bar, phase);
+  if constexpr (XT) {
+    if (ok && b.any_low) {
+      __syncthreads();
+      if (threadIdx.x == 0) b.item = -1;
+      ok = run_low<THREADS>(a, b, smem, bars_low);
+    }
+  }
   if (ok && b.any_wide) {
     __syncthreads();
     if (threadIdx.x == 0) b.item = -1;
@@ -929,9 +1240,9 @@ __global__ void __launch_bounds__(THREADS, MINB) accumulate_kernel(const __grid_
     // call (no block claims an item after it has counted itself out).
     unsigned* out = reinterpret_cast<unsigned*>(a.item_counter + kCounterExit);
     if (atomicAdd(out, 1u) == gridDim.x - 1) {
-      a.item_counter[0] = a.item_counter[1] = 0ULL;
+      a.item_counter[0] = a.item_counter[1] = a.item_counter[kCounterLow] = 0ULL;
       *out = 0u;
-      if (a.any_wide) *a.any_wide = 0;
+      if (a.any_wide) a.any_wide[0] = a.any_wide[1] = 0;
     }
   }
 }
@@ -984,45 +1295,73 @@ __global__ void __launch_bounds__(kRedThreads) reduce_kernel(const __grid_consta
   }
   pdl_wait();
   __syncthreads();
+  if (threadIdx.x == 0) settle_plan(b);
+  __syncthreads();
   const JobStatic& J = b.J;
   const JobCall& K = b.K;
   const int per_tile = J.bpt / kRedBins;
   const long long local = (long long)blockIdx.x - K.red_begin;
-  ItemRef it;
-  int s;
-  div_rem(local, per_tile, it.tile, s);
-  const int first1 = J.n_tiles - K.tail_tiles[1], first0 = first1 - K.tail_tiles[0];
-  it.fine = it.tile >= first1 ? it.tile - first1 : (it.tile >= first0 ? it.tile - first0 : -1);
-  it.n_chunks = it.fine < 0 ? K.n_chunks : K.n_chunks_f[it.tile >= first1 ? 1 : 0];
-  it.chunk = it.run = it.ck = 0;
-  const TileGeom g = tile_geom(J, it.tile, 256);
-  const PartMap m = part_map(J, K, it, g);
-  if (!bounds_ok(part_fits(J, it, m), J.status)) return;
-  const int nb = J.n_bins, n_om = J.n_omega, sh = __ffs(g.WT) - 1;  // tile widths are powers of two
+  const long long hi_blocks = (long long)J.n_tiles * per_tile;
+  const int nb = J.n_bins, n_om = J.n_omega;
+  const bool om4 = (n_om & 3) == 0;
   const int q = threadIdx.x & 31, pair = (threadIdx.x >> 5) & 3, cg = threadIdx.x >> 7;
-  const int i = s * kRedBins + 4 * q;  // first of the thread's bins within the tile
-  const int d = g.d0 + (i >> sh), o = g.o0 + (i & (g.WT - 1));
+  ItemRef it;
+  PartMap m;
+  int d, o, rd, ro;  // direction and frequency of the thread's first bin, and of its rotation
+  size_t off;        // the first bin's offset in the partials
+  bool part4;        // four bins at 16-byte aligned addresses
+  it.chunk = it.run = it.ck = 0;
+  const int rt = threadIdx.x & (kRedBins - 1);
+  if (local < hi_blocks) {
+    int s;
+    div_rem(local, per_tile, it.tile, s);
+    const int first1 = J.n_tiles - K.tail_tiles[1], first0 = first1 - K.tail_tiles[0];
+    it.fine = it.tile >= first1 ? it.tile - first1 : (it.tile >= first0 ? it.tile - first0 : -1);
+    it.n_chunks = it.fine < 0 ? K.n_chunks : K.n_chunks_f[it.tile >= first1 ? 1 : 0];
+    const TileGeom g = tile_geom(J, it.tile, 256);
+    m = part_map(J, K, it, g);
+    if (!bounds_ok(part_fits(J, it, m), J.status)) return;
+    const int sh = __ffs(g.WT) - 1;  // tile widths are powers of two
+    const int i = s * kRedBins + 4 * q, ti = s * kRedBins + rt;
+    d = g.d0 + (i >> sh), o = g.o0 + (i & (g.WT - 1));
+    rd = g.d0 + (ti >> sh), ro = g.o0 + (ti & (g.WT - 1));
+    off = it.fine < 0 ? (size_t)d * n_om + o : (size_t)i;
+    part4 = it.fine >= 0 || om4;
+  } else {
+    // the low band's bins, direction by direction
+    const long long f = (local - hi_blocks) * kRedBins;
+    const int js = b.plan.set >= 0 ? b.low.js : 0;
+    if (f >= (long long)J.n_dir * js) return;
+    div_rem(f + 4 * q, js, d, o);
+    div_rem(f + rt, js, rd, ro);
+    it.n_chunks = K.low[b.plan.set].n_lo;
+    it.fine = -1;
+    m.base = J.partials_l;
+    m.comp_stride = (size_t)J.n_dir * js;
+    m.chunk_stride = kComps * m.comp_stride;
+    off = (size_t)f + 4 * q;
+    part4 = true;  // (js is a multiple of 64)
+    if (!bounds_ok(it.n_chunks * (long long)m.chunk_stride <= J.low_cap, J.status)) return;
+  }
   const int live = d < J.n_dir ? min(4, n_om - o) : 0;  // bins inside the grid (<= 0: none)
   const size_t bin = (size_t)d * n_om + o;
-  const bool om4 = (n_om & 3) == 0;
-  const bool vec = live > 0 && (it.fine >= 0 || om4);
+  const bool vec = live > 0 && part4;
   // rotations: the last chunk range's threads, one bin each
   if (cg == kRedGroups - 1) {
-    const int t = threadIdx.x & (kRedBins - 1), ti = s * kRedBins + t;
-    const double* nd = J.dirs + 3 * (size_t)min(g.d0 + (ti >> sh), J.n_dir - 1);
+    const double* nd = J.dirs + 3 * (size_t)min(rd, J.n_dir - 1);
     const double tref = J.ref[3] - (nd[0] * J.ref[0] + nd[1] * J.ref[1] + nd[2] * J.ref[2]) * kInvC;
-    double psi = J.om_turns[min(g.o0 + (ti & (g.WT - 1)), n_om - 1)] * tref;  // turns
+    double psi = J.om_turns[min(ro, n_om - 1)] * tref;  // turns
     psi -= rint(psi);
     float2 cs;
     sincospif(2.0f * (float)psi, &cs.y, &cs.x);
-    rot[t] = cs;
+    rot[rt] = cs;
   }
   const int per = (it.n_chunks + kRedGroups - 1) / kRedGroups;
   const int c0 = min(cg * per, it.n_chunks), c1 = min(c0 + per, it.n_chunks);
   // set 0: U and V; set 1: the literal sum's two pairs
   for (int set = 0; set < (J.literal ? 2 : 1); ++set) {
     const bool mine = live > 0 && (set == 0 || pair < 2);
-    const float* base = set ? J.partials_p + bin : m.base + (it.fine < 0 ? bin : (size_t)i);
+    const float* base = set ? J.partials_p + bin : m.base + off;
     const size_t cs = set ? (size_t)nb : m.comp_stride, chs = set ? (size_t)4 * nb : m.chunk_stride;
     float4 re = make_float4(0.f, 0.f, 0.f, 0.f), im = re;
     if (mine) {
@@ -1109,7 +1448,15 @@ int blocks_per_sm() {
 
 }  // namespace
 
-int reduce_blocks(const JobStatic& js) { return js.n_tiles * (js.bpt / kRedBins); }
+int reduce_blocks(const JobStatic& js, const LowSet* low_sets) {
+  const int per_tile = js.bpt / kRedBins;
+  long long n = (long long)js.n_tiles * per_tile;
+  for (int s = 0; s < js.n_low; ++s) {
+    const long long low = ((long long)js.n_dir * low_sets[s].js + kRedBins - 1) / kRedBins;
+    n = std::max(n, (long long)low_sets[s].n_tiles * per_tile + low);
+  }
+  return (int)n;
+}
 
 cudaError_t launch_reduce(const LaunchArgs& a, long long blocks, cudaStream_t s) {
   count_launches(1);

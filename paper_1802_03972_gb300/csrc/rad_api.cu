@@ -1,6 +1,7 @@
 // C ABI of the radiation library: contexts, accumulate/readout, checkpoint and
 // merge, tile configuration, batched persistent launches with CUDA graphs.
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
@@ -142,30 +143,29 @@ bool valid_omega_tile(int variant, int wt) {
 // against the full tile's (1e5 particles, 512 x 128 bins, tensor-core variant:
 // 3387, 3553, 4034, 4625 us with 8, 4, 2, 1 warps per direction; FP32: 3955,
 // 4165, 4432, 5223).  1e5 particles, 300 x 144 bins: 3930 -> 2825 us.
-void fill_tiles(JobStatic& js, int variant, int wt) {
+namespace {
+
+// Segments of the default tiling over the frequencies from o0 on; returns their
+// tiles' cost in full tiles.
+double make_segments(int variant, int n_omega, int n_dir, int o0, TileSeg seg[kMaxSegs], int& n_seg,
+                     int& n_tiles) {
   const Variant v = variant_info(variant);
-  js.bpt = v.threads * v.w * v.passes;
-  js.n_seg = js.n_tiles = 0;
-  int o0 = 0;
+  const int bpt = v.threads * v.w * v.passes, unit = 32 * v.w * v.passes, warps = v.threads / 32;
+  n_seg = n_tiles = 0;
   auto add = [&](int width, int tiles_om) {
-    const int nt = js.bpt / width;
-    js.seg[js.n_seg++] = {js.n_tiles, o0, width, nt, tiles_om};
-    js.n_tiles += tiles_om * ((js.n_dir + nt - 1) / nt);
+    const int nt = bpt / width;
+    seg[n_seg++] = {n_tiles, o0, width, nt, tiles_om};
+    n_tiles += tiles_om * ((n_dir + nt - 1) / nt);
     o0 += width * tiles_om;
   };
-  const int unit = 32 * v.w * v.passes, warps = v.threads / 32;
-  if (wt != default_omega_tile(variant, js.n_omega)) {
-    add(wt, (js.n_omega + wt - 1) / wt);
-    return;
-  }
-  const int units = (js.n_omega + unit - 1) / unit, full = units / warps, rest = units % warps;
+  const int units = (n_omega - o0 + unit - 1) / unit, full = units / warps, rest = units % warps;
   static const double kTileCost[4] = {1.365, 1.19, 1.05, 1.0};  // 1, 2, 4, 8 warps per direction
   auto cost = [&](int m, int lg) {  // of one tile width m = 2^lg for all directions
     const int nt = warps / m;
-    return ((js.n_dir + nt - 1) / nt) * (m == warps ? 1.0 : kTileCost[lg]);
+    return ((n_dir + nt - 1) / nt) * (m == warps ? 1.0 : kTileCost[lg]);
   };
   int best = -1;  // bits 0-2: widths of 1, 2, 4 units used for the rest; -1: one more full tile
-  double best_cost = cost(warps, 3);
+  double best_cost = rest > 0 ? cost(warps, 3) : 0.0;
   for (int mask = 1; rest > 0 && mask < 8; ++mask) {
     if (mask < rest || mask >= warps) continue;  // (the widths are the mask's bits)
     double t = 0.0;
@@ -180,6 +180,89 @@ void fill_tiles(JobStatic& js, int variant, int wt) {
   if (n_full > 0) add(warps * unit, n_full);
   for (int lg = 2; rest > 0 && best > 0 && lg >= 0; --lg)
     if (best >> lg & 1) add(unit << lg, 1);
+  return full * cost(warps, 3) + best_cost;
+}
+
+}  // namespace
+
+void fill_tiles(JobStatic& js, int variant, int wt, int n_low) {
+  const Variant v = variant_info(variant);
+  js.bpt = v.threads * v.w * v.passes;
+  js.n_low = 0;
+  if (wt != default_omega_tile(variant, js.n_omega)) {
+    const int nt = js.bpt / wt, tiles_om = (js.n_omega + wt - 1) / wt;
+    js.seg[0] = {0, 0, wt, nt, tiles_om};
+    js.n_seg = 1;
+    js.n_tiles = tiles_om * ((js.n_dir + nt - 1) / nt);
+    return;
+  }
+  make_segments(variant, js.n_omega, js.n_dir, 0, js.seg, js.n_seg, js.n_tiles);
+  if (variant == kDefaultVariant) js.n_low = n_low;  // the low band uses variant 9's blocks
+}
+
+// The low band's alternatives of a grid (LowSet): for ascending frequencies, the
+// numbers of bins js that pay when taken from nodes (the remaining tiles and
+// the nodes, kLowCost of a full tile per direction group, below 0.92 of the full
+// tiling), cheapest first, a factor of two apart in H at least.  Tables: per
+// alternative the nodes' frequency table and the interpolation weights, appended
+// to `tab`; L.nodes and L.wts hold their offsets until they are uploaded.
+constexpr double kLowCost = 1.3;
+// Particles of a tile per resident block that the low band has to save: the sort and the
+// waves of smaller launches (about 200 us).  20000 particles, 512 x 64 bins
+// would take 475 us with it, 450 without; 40000, 1000 x 32 865 and 815; 1e5,
+// 512 x 256 4930 and 6790; 1e6, 1024 x 256 77.4 and 132.2 ms.
+constexpr double kLowFixed = 2500.0;
+int low_alternatives(const JobStatic& js, const double* omega, std::vector<float>& tab, LowSet* low, double* full) {
+  for (int i = 1; i < js.n_omega; ++i)
+    if (!(omega[i] > omega[i - 1])) return 0;
+  struct Cand { int js; double cost; };
+  std::vector<Cand> cand;
+  TileSeg seg[kMaxSegs];
+  int n_seg, n_tiles;
+  const double all = make_segments(kDefaultVariant, js.n_omega, js.n_dir, 0, seg, n_seg, n_tiles);
+  *full = all;
+  const double nodes = kLowCost * ((js.n_dir + 7) / 8);
+  for (int j = 2 * kLowNodes; j < js.n_omega; j += kLowNodes) {
+    const double c = nodes + make_segments(kDefaultVariant, js.n_omega, js.n_dir, j, seg, n_seg, n_tiles);
+    if (c < 0.92 * all) cand.push_back({j, c});
+  }
+  std::stable_sort(cand.begin(), cand.end(), [](const Cand& a, const Cand& b) { return a.cost < b.cost; });
+  int n = 0;
+  double last = 0.0;
+  for (const Cand& q : cand) {
+    const double f = omega[q.js - 1] / kTwoPi, dnu = f / kLowReach, H = 1.0 / (2.0 * kLowOversample * dnu);
+    if (n == kLowSets) break;
+    if (n > 0 && H < 2.0 * last) continue;
+    last = H;
+    LowSet& L = low[n++];
+    L.js = q.js;
+    L.hi_cost = (float)(make_segments(kDefaultVariant, js.n_omega, js.n_dir, q.js, L.seg, L.n_seg, L.n_tiles));
+    L.H = (float)H;
+    L.nodes = reinterpret_cast<const float*>(tab.size());
+    for (int part = 0; part < kOmTab; ++part)
+      for (int i = 0; i < kLowNodes; ++i) {
+        const double nu = (i - kLowTaps / 2) * dnu;
+        const float hi = (float)nu;
+        tab.push_back(part == 0 ? hi : (float)(kTwoPi * (part == 1 ? (double)hi : nu - (double)hi)));
+      }
+    while (tab.size() & 3) tab.push_back(0.0f);  // (read 16 bytes at a time)
+    L.wts = reinterpret_cast<const float*>(tab.size());
+    for (int i = 0; i < q.js; ++i) {
+      const double s = omega[i] / kTwoPi / dnu;  // in node spacings, from frequency 0
+      const int base = (int)std::min(floor(s), (double)kLowReach);
+      // taps at base - kLowTaps/2 + 1 .. base + kLowTaps/2; node 0 is -kLowTaps/2
+      for (int t = 0; t < kLowTaps; ++t) {
+        const double u = (s - (base - kLowTaps / 2 + 1 + t)) / (0.5 * kLowTaps);
+        tab.push_back(fabs(u) < 1.0 ? (float)exp(kLowBeta * (sqrt(1.0 - u * u) - 1.0)) : 0.0f);
+      }
+      float index;
+      const int first = base + 1;
+      memcpy(&index, &first, sizeof(float));
+      tab.push_back(index);
+      tab.push_back(0.0f);
+    }
+  }
+  return n;
 }
 
 int resident_ctas(int variant) {
@@ -228,17 +311,17 @@ rad_status upload_static(rad_ctx* c) {
                                        cudaMemcpyHostToDevice, c->stream));
 }
 
-rad_status ensure_capacity(rad_ctx* c, long long n, int n_chunks, long long fine_floats) {
+rad_status ensure_capacity(rad_ctx* c, long long n, int n_chunks, long long fine_floats, long long low_floats) {
   bool changed = false;
   if (n > c->h_js.n_cap) {
     long long cap = std::max(n, c->h_js.n_cap * 3 / 2);
     cap = (cap + 255) / 256 * 256;
     JobStatic& js = c->h_js;
     if (js.rec) cudaStreamSynchronize(c->stream);
-    void* old[] = {js.rec, js.perm, js.sort_counts, js.bucket_base, js.gref};
+    void* old[] = {js.rec, js.perm, js.sort_counts, js.bucket_base, js.gref, js.rec_s};
     for (void* p : old)
       if (p) cudaFree(p);
-    js.rec = nullptr;
+    js.rec = js.rec_s = nullptr;
     js.perm = js.sort_counts = js.bucket_base = nullptr;
     js.gref = nullptr;
     // the record buffer, and the sort buffers of wide calls (12 B per particle)
@@ -250,6 +333,9 @@ rad_status ensure_capacity(rad_ctx* c, long long n, int n_chunks, long long fine
                                   (size_t)((cap + kSortBlock - 1) / kSortBlock) * kSortBuckets));
       if (s == RAD_OK) s = cuda_check(c, dmalloc(&js.bucket_base, (size_t)kSortBuckets));
       if (s == RAD_OK) s = cuda_check(c, dmalloc(&js.gref, (size_t)3 * ((cap + kGroup - 1) / kGroup)));
+      // (a context that may take the low band, at any tile set later)
+      if (s == RAD_OK && c->n_low > 0 && cap >= kLowMin)
+        s = cuda_check(c, dmalloc(&js.rec_s, (size_t)cap * kRecFields));
     }
     if (s != RAD_OK) {
       js.n_cap = 0;
@@ -296,7 +382,72 @@ rad_status ensure_capacity(rad_ctx* c, long long n, int n_chunks, long long fine
     c->h_js.fine_cap = cap;
     changed = true;
   }
+  if (low_floats > c->h_js.low_cap) {
+    const long long cap = std::max(low_floats, c->h_js.low_cap * 3 / 2);
+    if (c->h_js.partials_l) {
+      cudaStreamSynchronize(c->stream);
+      cudaFree(c->h_js.partials_l);
+      c->h_js.partials_l = nullptr;
+    }
+    rad_status s = cuda_check(c, dmalloc(&c->h_js.partials_l, (size_t)cap));
+    if (s != RAD_OK) {
+      c->h_js.low_cap = 0;
+      return s;
+    }
+    c->h_js.low_cap = cap;
+    changed = true;
+  }
   return changed ? upload_static(c) : RAD_OK;
+}
+
+CallPlan plan_call(const rad_ctx* c, const JobStatic& js, int variant, long long n) {
+  CallPlan p;
+  p.ck = auto_chunk(c, variant, n, js.n_tiles);
+  p.n_chunks = (int)((n + p.ck - 1) / p.ck);
+  p.tail = tail_plan(variant_tensor_core(variant) && !js.literal, n, js.n_tiles, p.ck, p.n_chunks,
+                     resident_ctas(variant));
+  p.most_chunks = p.n_chunks;
+  // The low band (automatic chunks, calls that are sorted when wide): per
+  // alternative, the other bins' tiles chunked as a job of their own (without the
+  // fine tail: the low band's items follow), and about kLowItemsPerCta items per
+  // resident block of the band.
+  if (js.n_low == 0 || c->tile.chunk != 0 || js.wide_flag == nullptr || n < kLowMin || n >= (1LL << 31))
+    return p;
+  const long long dirs8 = (js.n_dir + 7) / 8;
+  for (int s = 0; s < js.n_low; ++s) {
+    const LowSet& L = c->low[s];
+    LowCall& C = p.low[s];
+    C.ck_hi = auto_chunk_for(variant, n, L.n_tiles, true);
+    C.n_hi = (int)((n + C.ck_hi - 1) / C.ck_hi);
+    long long ck = n * dirs8 / ((long long)kLowItemsPerCta * resident_ctas(variant)) + kChunkAlign;
+    ck = std::max<long long>(kLowChunkMin, std::min<long long>(ck, 1LL << 30) / kChunkAlign * kChunkAlign);
+    C.ck_lo = (int)ck;
+    C.n_lo = (int)((n + ck - 1) / ck);
+    // What it saves, in particles of a tile: the bins' tiles against the nodes and
+    // an interpolation per direction and piece of a cell (about 64 cells).
+    const double saved = (c->low_full - L.hi_cost) * (double)n -
+                         (double)dirs8 * (kLowCost * (double)n + (C.n_lo + 64) * (64 + 0.5 * L.js));
+    if (saved < kLowFixed * resident_ctas(variant)) continue;
+    p.low_ok |= 1u << s;
+    p.most_chunks = std::max(p.most_chunks, C.n_hi);
+    p.hi_items = std::max(p.hi_items, (long long)L.n_tiles * C.n_hi);
+    p.low_items = std::max(p.low_items, dirs8 * C.n_lo);
+    p.low_floats = std::max(p.low_floats, (long long)C.n_lo * kComps * js.n_dir * L.js);
+  }
+  return p;
+}
+
+long long CallPlan::items(const JobStatic& js, int run) const {
+  return std::max(tail.items(js.n_tiles, (n_chunks + run - 1) / run), hi_items);
+}
+
+void CallPlan::fill(JobCall& K, const JobStatic& js, int run) const {
+  K.ck = ck;
+  K.n_chunks = n_chunks;
+  K.run = run;
+  set_tail(K, tail);
+  K.low_ok = low_ok;
+  for (int s = 0; low_ok && s < js.n_low; ++s) K.low[s] = low[s];
 }
 
 // Host copy of the amplitude form factor of Table 1 (f(0) = 1), for the
@@ -361,11 +512,8 @@ rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const do
                                      c->f64_chunks, c->h_js.status, c->stream));
   }
   const int variant = c->tile.variant;
-  const int ck = auto_chunk(c, variant, n, c->h_js.n_tiles);
-  const int n_chunks = (int)((n + ck - 1) / ck);
-  const TailPlan tail = tail_plan(variant_tensor_core(variant) && !c->h_js.literal, n,
-                                  c->h_js.n_tiles, ck, n_chunks, resident_ctas(variant));
-  rad_status s = ensure_capacity(c, n, n_chunks, tail.fine_floats(c->h_js.bpt));
+  const CallPlan plan = plan_call(c, c->h_js, variant, n);
+  rad_status s = ensure_capacity(c, n, plan.most_chunks, plan.tail.fine_floats(c->h_js.bpt), plan.low_floats);
   if (s != RAD_OK) return s;
   LaunchArgs a;
   memset(&a, 0, sizeof(a));
@@ -373,7 +521,8 @@ rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const do
   a.jc = nullptr;
   a.n_jobs = 1;
   a.use_inline = 1;
-  a.n_items = tail.items(c->h_js.n_tiles, n_chunks);
+  a.n_items = plan.items(c->h_js, 1);
+  a.n_items_low = plan.low_items;
   a.item_counter = c->d_counter;  // [0], [1]: item counters; [2]: the wide flag
   // A call of at most one sorted group is never wide (the pre-pass does not
   // flag it): it needs neither the wide-call kernels nor the second kernel.
@@ -386,10 +535,7 @@ rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const do
   K.w = w;
   K.t = t;
   K.dt = dt;
-  K.ck = ck;
-  K.n_chunks = n_chunks;
-  K.run = 1;
-  set_tail(K, tail);
+  plan.fill(K, c->h_js, 1);
   K.item_begin = 0;
   K.block_begin = 0;
   cudaEvent_t* ev = nullptr;
@@ -415,7 +561,7 @@ rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const do
   if (ev) cudaEventRecord(ev[1], c->stream);
   const long long grid = std::min<long long>(a.n_items, resident_ctas(variant));
   s = cuda_check(c, launch_accumulate(variant, a, (int)grid, c->stream));
-  if (s == RAD_OK) s = cuda_check(c, launch_reduce(a, reduce_blocks(c->h_js), c->stream));
+  if (s == RAD_OK) s = cuda_check(c, launch_reduce(a, reduce_blocks(c->h_js, c->low), c->stream));
   if (ev) cudaEventRecord(ev[2], c->stream);
   return s;
 }
@@ -529,9 +675,11 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
   js.n_omega = n_omega;
   js.n_dir = n_dir;
   js.n_bins = c->n_bins;
-  fill_tiles(js, c->tile.variant, c->tile.omega_tile);
   js.tau_fast = (float)(2097152.0 / std::max(om_hi_max, 1e-300));  // 2^21 turns
   wide_geometry(nd.data(), n_dir, js.tau_fast, js.axis, &js.cone_sin, &js.bucket_w);
+  low_geometry(nd.data(), n_dir, js);
+  if (prec == RAD_PREC_MIXED && !literal) c->n_low = low_alternatives(js, omega, om_tab, c->low, &c->low_full);
+  fill_tiles(js, c->tile.variant, c->tile.omega_tile, c->n_low);
 
   rad_status s = RAD_OK;
   size_t f64_words = 0;  // doubles of an FP64 context's allocation
@@ -544,7 +692,7 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
   chk(dmalloc(&c->d_dirs, nd.size()));
   chk(dmalloc(&c->d_dir_tab, dir_tab.size()));
   chk(dmalloc(&c->d_ref, 4));
-  chk(dmalloc(&c->d_status, 1));
+  chk(dmalloc(&c->d_status, kStatusWords + sizeof(c->low) / sizeof(int)));
   chk(dmalloc(&c->d_counter, kCounterWords));
   chk(dmalloc(&c->d_js, 1));
   chk(dmalloc(&c->d_spec, (size_t)3 * c->n_bins));
@@ -565,13 +713,23 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
       c->d_cnt64 = reinterpret_cast<unsigned*>(c->d_part64 + parts);
     }
   }
+  // the low band's alternatives go after the status words
+  js.low = reinterpret_cast<const LowSet*>(c->d_status + kStatusWords);
+  for (int i = 0; i < c->n_low; ++i) {
+    c->low[i].nodes = c->d_om_tab + reinterpret_cast<size_t>(c->low[i].nodes);
+    c->low[i].wts = c->d_om_tab + reinterpret_cast<size_t>(c->low[i].wts);
+  }
   if (s == RAD_OK) {
     chk(cudaMemcpy(c->d_omega, omega, sizeof(double) * n_omega, cudaMemcpyHostToDevice));
     chk(cudaMemcpy(c->d_om_turns, om_turns.data(), sizeof(double) * n_omega, cudaMemcpyHostToDevice));
     chk(cudaMemcpy(c->d_om_tab, om_tab.data(), sizeof(float) * om_tab.size(), cudaMemcpyHostToDevice));
     chk(cudaMemcpy(c->d_dirs, nd.data(), sizeof(double) * nd.size(), cudaMemcpyHostToDevice));
     chk(cudaMemcpy(c->d_dir_tab, dir_tab.data(), sizeof(float) * dir_tab.size(), cudaMemcpyHostToDevice));
-    chk(cudaMemset(c->d_status, 0, sizeof(int)));
+    // the status word, then (low band) the extents, the plan and the alternatives
+    int words[kStatusWords + sizeof(c->low) / sizeof(int)] = {0};
+    for (int e = 0; e < 6; ++e) words[kStatusExt + e] = e & 1 ? INT_MIN : INT_MAX;
+    memcpy(words + kStatusWords, c->low, sizeof(c->low));
+    chk(cudaMemcpy(c->d_status, words, sizeof(words), cudaMemcpyHostToDevice));
     chk(cudaMemset(c->d_counter, 0, kCounterWords * sizeof(unsigned long long)));
     chk(cudaMemset(c->d_ref, 0, 4 * sizeof(double)));
     if (prec == RAD_PREC_MIXED) {
@@ -590,6 +748,8 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
     }
   }
   js.om_tab = c->d_om_tab;
+  js.ext = c->d_status + kStatusExt;
+  js.plan = reinterpret_cast<LowPlan*>(c->d_status + kStatusPlan);
   js.om_turns = c->d_om_turns;
   js.omega = c->d_omega;
   js.dir_tab = c->d_dir_tab;
@@ -605,7 +765,7 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
   if (literal) {
     c->tile.variant = kLiteralVariant;
     c->tile.omega_tile = default_omega_tile(kLiteralVariant, n_omega);
-    fill_tiles(js, c->tile.variant, c->tile.omega_tile);
+    fill_tiles(js, c->tile.variant, c->tile.omega_tile, 0);
   }
   if (s == RAD_OK) chk(cudaMemcpy(c->d_js, &js, sizeof(JobStatic), cudaMemcpyHostToDevice));
   if (s != RAD_OK) {
@@ -623,7 +783,8 @@ void rad_destroy(rad_ctx* c) {
                   c->d_status, c->d_counter, c->d_js, c->d_spec, c->d_state, c->d_state64,
                   c->h_js.rec, c->h_js.partials, c->d_stage, c->d_state_p,
                   c->d_f2, c->h_js.partials_p, c->d_push, c->d_push_bdot, c->h_js.perm,
-                  c->h_js.sort_counts, c->h_js.bucket_base, c->h_js.gref, c->h_js.partials_f};
+                  c->h_js.sort_counts, c->h_js.bucket_base, c->h_js.gref, c->h_js.partials_f,
+                  c->h_js.rec_s, c->h_js.partials_l};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (cudaEvent_t e : c->prof_ev) cudaEventDestroy(e);
@@ -987,7 +1148,7 @@ rad_status rad_set_tile(rad_ctx* c, const rad_tile* t) {
   rad_status s = cuda_check(c, cudaStreamSynchronize(c->stream));
   if (s != RAD_OK) return s;
   JobStatic js = c->h_js;
-  fill_tiles(js, t->variant, wt);
+  fill_tiles(js, t->variant, wt, c->n_low);
   c->h_js = js;
   c->tile.variant = t->variant;
   c->tile.omega_tile = wt;

@@ -106,7 +106,7 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
     if (jobs[i]->tile.variant != variant) variant = kDefaultVariant;
 
   // Per-job chunking, capacities (may reallocate: drain this stream first).
-  struct Plan { int job; long long n; int ck, n_chunks; TailPlan tail; long long cost; JobStatic js; };
+  struct Plan { int job; long long n; CallPlan call; long long cost; JobStatic js; };
   std::vector<Plan> plan;
   plan.reserve(n_jobs);
   bool drained = false;
@@ -115,19 +115,18 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
     if (steps[i].n <= 0) continue;
     JobStatic js = c->h_js;
     if (c->tile.variant != variant)
-      fill_tiles(js, variant, default_omega_tile(variant, c->n_omega));
-    const int ck = auto_chunk(c, variant, steps[i].n, js.n_tiles);
-    const int nch = (int)((steps[i].n + ck - 1) / ck);
+      fill_tiles(js, variant, default_omega_tile(variant, c->n_omega), c->n_low);
     // chunked as the job alone would be (results equal bit for bit)
-    const TailPlan tail = tail_plan(variant_tensor_core(variant) && !js.literal, steps[i].n,
-                                    js.n_tiles, ck, nch, resident_ctas(variant));
-    const long long fine = tail.fine_floats(js.bpt);
-    if (steps[i].n > c->h_js.n_cap || nch > c->h_js.chunk_cap || fine > c->h_js.fine_cap) {
+    const CallPlan call = plan_call(c, js, variant, steps[i].n);
+    const int nch = call.most_chunks;
+    const long long fine = call.tail.fine_floats(js.bpt);
+    if (steps[i].n > c->h_js.n_cap || nch > c->h_js.chunk_cap || fine > c->h_js.fine_cap ||
+        call.low_floats > c->h_js.low_cap) {
       if (!drained) {
         if (cudaStreamSynchronize(work) != cudaSuccess) return RAD_ECUDA;
         drained = true;
       }
-      rad_status s = ensure_capacity(c, steps[i].n, nch, fine);
+      rad_status s = ensure_capacity(c, steps[i].n, nch, fine, call.low_floats);
       if (s != RAD_OK) return s;
       if (cudaStreamSynchronize(c->stream) != cudaSuccess) return RAD_ECUDA;
       js.rec = c->h_js.rec;
@@ -140,8 +139,11 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
       js.sort_counts = c->h_js.sort_counts;
       js.bucket_base = c->h_js.bucket_base;
       js.gref = c->h_js.gref;
+      js.rec_s = c->h_js.rec_s;
+      js.partials_l = c->h_js.partials_l;
+      js.low_cap = c->h_js.low_cap;
     }
-    plan.push_back({i, steps[i].n, ck, nch, tail, (long long)js.n_tiles * nch * (long long)ck, js});
+    plan.push_back({i, steps[i].n, call, (long long)js.n_tiles * call.n_chunks * (long long)call.ck, js});
   }
   if (plan.empty()) return RAD_OK;
   // Largest jobs first, so the dynamic scheduler's tail holds small items.
@@ -181,15 +183,15 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
   for (const Plan& q : plan) total += q.n * q.js.n_tiles;
   const long long per_item = total / ((long long)kBatchItemsPerCta * resident_ctas(variant));
   auto run_of = [&](const Plan& q) {
-    if (q.tail.tiles() > 0) return 1;
-    return (int)std::max<long long>(1, std::min<long long>(per_item, 1LL << 30) / q.ck);
+    if (q.call.tail.tiles() > 0) return 1;
+    return (int)std::max<long long>(1, std::min<long long>(per_item, 1LL << 30) / q.call.ck);
   };
 
   // Per-call table in the next pinned slot.
   const int s = slot;
   slot = (slot + 1) % kSlots;
   if (cudaEventSynchronize(slot_done[s]) != cudaSuccess) return RAD_ECUDA;
-  long long items = 0;
+  long long items = 0, low_items = 0;
   int blocks = 0, sort_blocks = 0;
   unsigned red_blocks = 0;
   std::vector<rad_step> sorted(plan.size());
@@ -205,16 +207,16 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
     K.w = st.w;
     K.t = st.t;
     K.dt = st.dt;
-    K.ck = plan[p].ck;
-    K.n_chunks = plan[p].n_chunks;
-    K.run = run_of(plan[p]);
-    set_tail(K, plan[p].tail);
+    const int run = run_of(plan[p]);
+    plan[p].call.fill(K, plan[p].js, run);
     K.item_begin = items;
+    K.low_begin = low_items;
     K.block_begin = blocks;
     K.sort_block_begin = sort_blocks;
     K.red_begin = red_blocks;
-    items += plan[p].tail.items(plan[p].js.n_tiles, (plan[p].n_chunks + K.run - 1) / K.run);
-    red_blocks += (unsigned)reduce_blocks(plan[p].js);
+    items += plan[p].call.items(plan[p].js, run);
+    low_items += plan[p].call.low_items;
+    red_blocks += (unsigned)reduce_blocks(plan[p].js, jobs[plan[p].job]->low);
     blocks += (int)((st.n + 255) / 256);
     sort_blocks += (int)((st.n + kSortBlock - 1) / kSortBlock);
   }
@@ -225,6 +227,7 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
   a.n_jobs = (int)plan.size();
   a.use_inline = 0;
   a.n_items = items;
+  a.n_items_low = low_items;
   a.item_counter = d_counter;
   a.any_wide = reinterpret_cast<int*>(d_counter + 2);
   const int grid = (int)std::min<long long>(items, resident_ctas(variant));

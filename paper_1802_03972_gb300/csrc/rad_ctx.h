@@ -52,6 +52,9 @@ struct rad_ctx {
   std::vector<cudaEvent_t> prof_ev;  // 3 per timed call
   size_t prof_used = 0;
   unsigned long long* d_prof_clk = nullptr;  // [2] cycles, ns of the accumulate CTAs
+  int n_low = 0;                 // low-band alternatives of the grid (host copies)
+  double low_full = 0.0;         // cost of the full tiling, in full tiles
+  radimpl::LowSet low[radimpl::kLowSets]{};
   long long generation = 0;      // bumped whenever d_js changes
   uint64_t grid_hash = 0;        // FNV-1a of the frequencies and unit directions
   int device = -1;               // the CUDA device current at rad_create
@@ -77,14 +80,29 @@ rad_status check_device(rad_ctx* c);
 rad_status cuda_check(rad_ctx* c, cudaError_t e);
 int default_omega_tile(int variant, int n_omega);
 bool valid_omega_tile(int variant, int wt);
-void fill_tiles(JobStatic& js, int variant, int wt);
+// n_low: the context's low-band alternatives, used with the default tiling
+void fill_tiles(JobStatic& js, int variant, int wt, int n_low);
 int resident_ctas(int variant);
 // fine_tail: the job's last tiles are fine-chunked (TailPlan), which allows longer items.
 int auto_chunk_for(int variant, long long n, int n_tiles, bool fine_tail);
 int auto_chunk(const rad_ctx* c, int variant, long long n, int n_tiles);
 // Capacity for n particles, n_chunks coarse chunks and fine_floats floats of
 // fine-tile partial sums (TailPlan::fine_floats).
-rad_status ensure_capacity(rad_ctx* c, long long n, int n_chunks, long long fine_floats = 0);
+rad_status ensure_capacity(rad_ctx* c, long long n, int n_chunks, long long fine_floats = 0,
+                           long long low_floats = 0);
+// How a call of n particles is cut into work items.
+struct CallPlan {
+  int ck = 0, n_chunks = 0;
+  int most_chunks = 0;  // over the low band's alternatives too
+  TailPlan tail;
+  unsigned low_ok = 0;  // the alternatives that pay for this call (bits)
+  LowCall low[kLowSets] = {};
+  long long hi_items = 0, low_items = 0, low_floats = 0;
+  // items of the bin tiles (run: chunks per item), the most over the alternatives
+  long long items(const JobStatic& js, int run) const;
+  void fill(JobCall& K, const JobStatic& js, int run) const;
+};
+CallPlan plan_call(const rad_ctx* c, const JobStatic& js, int variant, long long n);
 rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const double* beta,
                               const double* bdot, const double* w, double t, double dt);
 rad_status upload_static(rad_ctx* c);

@@ -89,13 +89,14 @@ __device__ __forceinline__ void tma_load_1d(void* dst, const void* src, uint32_t
       : "memory");
 }
 
-// Job of a global work item (jobs ordered by item_begin), by a whole warp: each
-// lane counts the jobs of its share that begin at or before the item
-// (independent loads, one round trip).
-__device__ __forceinline__ int find_job_warp(const LaunchArgs& a, long long item) {
+// Job of a global work item (jobs ordered by item_begin; low: of a low-band item,
+// by low_begin), by a whole warp: each lane counts the jobs of its share that
+// begin at or before the item (independent loads, one round trip).
+__device__ __forceinline__ int find_job_warp(const LaunchArgs& a, long long item, bool low = false) {
   if (a.n_jobs == 1) return 0;
   int n = 0;
-  for (int i = threadIdx.x & 31; i < a.n_jobs; i += 32) n += a.jc[i].item_begin <= item;
+  for (int i = threadIdx.x & 31; i < a.n_jobs; i += 32)
+    n += (low ? a.jc[i].low_begin : a.jc[i].item_begin) <= item;
   return __reduce_add_sync(0xffffffffu, n) - 1;
 }
 

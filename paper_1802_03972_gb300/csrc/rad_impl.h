@@ -73,9 +73,11 @@ constexpr int kSortBlock = 2048;
 // A context's counter block (unsigned long long words, zero between calls: the
 // last block of the accumulate kernel to leave zeroes it):
 // [0], [1] the accumulate kernel's work-item counters for ordinary and wide
-// calls, [2] the call's wide flag (an int), [3] the count of blocks that have left.
-constexpr int kCounterWords = 4;
+// calls, [2] the call's wide flag and whether some job takes the low band (two
+// ints), [3] the count of blocks that have left, [4] the low band's item counter.
+constexpr int kCounterWords = 5;
 constexpr int kCounterExit = 3;
+constexpr int kCounterLow = 4;
 constexpr int kSortBuckets = 4096;
 constexpr int kGroup = 256;
 static_assert(kGroup == kChunkAlign, "a work item holds whole sorted groups");
@@ -93,6 +95,55 @@ struct TileSeg {
   int tile0, o0, wt, nt, tiles_om;
 };
 constexpr int kMaxSegs = 4;  // one per tile width: a block's 8, 4, 2 and 1 warps per direction
+
+// The low band of a frequency grid.  A cell of particles whose retarded times lie
+// within +-H of its centre has sums S(omega) that are band-limited in omega: the
+// cell's sums at kLowNodes evenly spaced frequencies (nodes, dnu apart) give
+// all of the grid's bins up to omega_s = 2 pi kLowReach dnu, dnu = 1 / (2
+// kLowOversample H), by interpolation with kLowTaps taps to 2.3e-8 of the
+// neighbouring sums (a window exp(beta (sqrt(1 - (2u/taps)^2) - 1)), as in
+// non-uniform FFTs with an exponential-of-semicircle kernel: Barnett, Magland and
+// af Klinteberg, SIAM J. Sci. Comput. 41 (2019) C479; beta and the
+// particle-side factor's polynomial fitted here, by quadrature).  A logarithmic
+// grid spends hundreds of bins there.  Evaluating 64 nodes per (particle,
+// direction) instead of, say, 256 bins makes the same sums in a quarter of the
+// sin/cos, the bound of this path.  The particles of such a call are sorted
+// into cells of width h along the grid's mean direction (the wide calls' sort).
+constexpr int kLowNodes = 64;
+constexpr int kLowTaps = 10;
+constexpr int kLowReach = kLowNodes - 1 - kLowTaps;  // node 0 is frequency -kLowTaps/2 dnu
+constexpr double kLowOversample = 1.75;
+constexpr double kLowBeta = 21.5;
+constexpr int kLowWt = 12;            // floats per bin of the interpolation table: taps, first node, unused
+constexpr int kLowSets = 16;          // alternatives of one grid (bins in the band, H)
+constexpr long long kLowMin = 16384;  // particles of a call from which the low band is considered
+constexpr int kLowCellMin = 64;       // ... and on average per cell
+constexpr int kLowMaxCells = 4000;
+constexpr int kLowItemsPerCta = 4;    // the band's work items per resident block
+constexpr int kLowChunkMin = 512;
+// A context's status allocation: the status word, the call's extents, its plan.
+constexpr int kStatusExt = 2, kStatusPlan = 8, kStatusWords = 16;
+
+// One alternative: the js lowest bins from nodes, the others in bin tiles.
+struct LowSet {
+  int js, n_tiles, n_seg;
+  float H;               // half-range of a cell's retarded times, s
+  float hi_cost;         // of the other bins' tiles, in full tiles
+  TileSeg seg[kMaxSegs];
+  const float* nodes;    // [kOmTab][kLowNodes], as om_tab
+  const float* wts;      // [js][kLowWt]
+};
+// What a call does (written by the scan kernel): the alternative taken (-1:
+// none) and its cells, of width h from s0 along the axis, centred on c1, c2
+// across it (seconds).
+struct LowPlan {
+  int set, cells;
+  float s0, h, c1, c2;
+};
+// A call's chunks in an alternative: of its bin tiles and of the low band.
+struct LowCall {
+  int ck_hi, n_hi, ck_lo, n_lo;
+};
 
 // Per-job data that does not change between calls.
 struct JobStatic {
@@ -134,6 +185,16 @@ struct JobStatic {
   int* sort_counts;               // [ceil(n_cap / kSortBlock)][kSortBuckets]
   int* bucket_base;               // [kSortBuckets] first sorted position of each bucket
   double* gref;                   // [ceil(n_cap / kGroup)][3] group reference - call reference, m
+  // low band (n_low = 0: never): alternatives, the one with the cheapest bins first
+  int n_low;
+  const LowSet* low;
+  double fr1[3], fr2[3];          // transverse frame of the sort axis
+  float cone1, cone2;             // largest |n . fr1|, |n . fr2| of the grid
+  int* ext;                       // [6] a call's smallest / largest coordinate along fr1, fr2, axis (ordered ints)
+  LowPlan* plan;
+  float* rec_s;                   // [n_cap][20] records in cell order
+  float* partials_l;              // low_cap floats: the low bands' chunk sums, [chunk][8][n_dir][js]
+  long long low_cap;
 };
 
 // Per-call data of one job.
@@ -151,6 +212,9 @@ struct JobCall {
   int block_begin;       // first pre-pass block of this job
   int sort_block_begin;  // first sort-histogram block of this job
   unsigned red_begin;    // first block of this job in the tile reduction
+  unsigned low_ok;       // the low band's alternatives the call may take (bits)
+  LowCall low[kLowSets];
+  long long low_begin;   // first low-band item of this job
   // Fine-chunked last tiles (TailPlan), level 0 then level 1 in tile order
   // (level 1 the job's last tail_tiles[1] tiles): tail_tiles[l] tiles with
   // chunks of ck_f[l] (n_chunks_f[l] per tile)
@@ -236,6 +300,7 @@ struct LaunchArgs {
   int n_jobs;
   int use_inline;        // 1: single job, call passed by value below
   long long n_items;
+  long long n_items_low; // low-band work items (0: none possible)
   // the counter block (kCounterWords), zero before the launch
   unsigned long long* item_counter;
   JobCall inline_call;
@@ -243,7 +308,8 @@ struct LaunchArgs {
   // summed over the accumulate CTAs' lifetimes.
   unsigned long long* prof_clk;
   // Set (non-zero) by the pre-pass when some job's call is wide; null when no
-  // job can be (the wide-call kernels are then not launched).
+  // job can be (the wide-call kernels are then not launched).  The int after it:
+  // some job takes the low band (set by the scan kernel).
   int* any_wide;
 };
 
@@ -311,11 +377,14 @@ constexpr int kWideLaunches = 4;
 // Sort axis and bucket width of a job (host, at creation).
 void wide_geometry(const double* unit_dirs, int n_dir, float tau_fast, double axis[3],
                    double* cone_sin, double* bucket_w);
+// Transverse frame of the sort axis and the grid's reach along it (low band).
+void low_geometry(const double* unit_dirs, int n_dir, JobStatic& js);
 // Launches the accumulate kernel, and the reduction of its partial sums into the
 // states (blocks: reduce_blocks summed over the jobs).
 cudaError_t launch_accumulate(int variant, const LaunchArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_reduce(const LaunchArgs& a, long long blocks, cudaStream_t s);
-int reduce_blocks(const JobStatic& js);
+// (the most over the job's low-band alternatives, a host copy of js.low)
+int reduce_blocks(const JobStatic& js, const LowSet* low);
 int accumulate_blocks_per_sm(int variant);
 // Per-device caches of launch properties cover device ordinals below this.
 constexpr int kMaxDevices = 64;

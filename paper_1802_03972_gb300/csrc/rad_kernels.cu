@@ -10,6 +10,7 @@
 // (FP64 before rounding), w dt and sqrt(w) dt.  FP64 is used here once per
 // particle, never per (particle, direction, frequency).
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stdint.h>
 
@@ -78,6 +79,79 @@ __device__ __forceinline__ void store_record(float* dst_rec, const float v[kRecF
     dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
 }
 
+// ---- low band (see LowSet)
+// Integers in the order of the floats.
+__device__ __forceinline__ int ordered(float x) {
+  const int i = __float_as_int(x);
+  return i < 0 ? i ^ 0x7fffffff : i;
+}
+__device__ __forceinline__ float from_ordered(int i) { return __int_as_float(i < 0 ? i ^ 0x7fffffff : i); }
+
+// Coordinate of a record along a frame axis (seconds).  Explicit roundings: the
+// extents, the histogram and the scatter must agree bit for bit.
+__device__ __forceinline__ float frame_coord(const double ax[3], const float* v) {
+  return __fmaf_rn((float)ax[0], v[0], __fmaf_rn((float)ax[1], v[1], __fmul_rn((float)ax[2], v[2])));
+}
+
+// A block's share of the call's extents along the frame (256 threads).
+__device__ __forceinline__ void call_extents(const JobStatic& J, const float* v, bool live) {
+  __shared__ int s_ext[6];
+  if (threadIdx.x < 6) s_ext[threadIdx.x] = threadIdx.x & 1 ? INT_MIN : INT_MAX;
+  __syncthreads();
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int o = live ? ordered(frame_coord(a == 0 ? J.fr1 : (a == 1 ? J.fr2 : J.axis), v)) : 0;
+    const int lo = __reduce_min_sync(0xffffffffu, live ? o : INT_MAX);
+    const int hi = __reduce_max_sync(0xffffffffu, live ? o : INT_MIN);
+    if ((threadIdx.x & 31) == 0) {
+      atomicMin(&s_ext[2 * a], lo);
+      atomicMax(&s_ext[2 * a + 1], hi);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 6) {
+    if (threadIdx.x & 1) atomicMax(&J.ext[threadIdx.x], s_ext[threadIdx.x]);
+    else atomicMin(&J.ext[threadIdx.x], s_ext[threadIdx.x]);
+  }
+}
+
+// The call's plan: the first alternative whose cells are wide enough.  A cell's
+// retarded times reach, from its centre, at most the grid's largest transverse
+// share of the bunch's half-widths plus half the cell's width.
+__device__ __forceinline__ LowPlan low_plan(const JobStatic& J, const JobCall& K) {
+  LowPlan p = {-1, 0, 0.0f, 0.0f, 0.0f, 0.0f};
+  if (!K.low_ok || (J.wide_flag != nullptr && *J.wide_flag != 0)) return p;
+  float lo[3], hi[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (J.ext[2 * a] > J.ext[2 * a + 1]) return p;  // no valid particle
+    lo[a] = from_ordered(J.ext[2 * a]);
+    hi[a] = from_ordered(J.ext[2 * a + 1]);
+  }
+  const float side = __fmaf_rn(J.cone1, __fmul_rn(0.5f, __fsub_rn(hi[0], lo[0])),
+                               __fmul_rn(J.cone2, __fmul_rn(0.5f, __fsub_rn(hi[1], lo[1]))));
+  for (int s = 0; s < J.n_low; ++s) {
+    if (!(K.low_ok >> s & 1u)) continue;
+    const float h = __fmul_rn(2.0f, __fsub_rn(__fmul_rn(0.998f, J.low[s].H), __fmul_rn(1.001f, side)));
+    if (!(h > 0.0f)) continue;
+    const float cells = __fadd_rn(__fdiv_rn(__fsub_rn(hi[2], lo[2]), h), 1.0f);
+    if (!(cells < (float)kLowMaxCells) || !(cells * kLowCellMin <= (float)K.n)) continue;
+    p.set = s;
+    p.cells = min((int)cells + 1, kLowMaxCells);
+    p.s0 = lo[2];
+    p.h = h;
+    p.c1 = __fmul_rn(0.5f, __fadd_rn(lo[0], hi[0]));
+    p.c2 = __fmul_rn(0.5f, __fadd_rn(lo[1], hi[1]));
+    return p;
+  }
+  return p;
+}
+
+__device__ __forceinline__ int low_cell(const JobStatic& J, const LowPlan& p, const float* v) {
+  const float q = floorf(__fdiv_rn(__fsub_rn(frame_coord(J.axis, v), p.s0), p.h));
+  return max(0, min(p.cells - 1, (int)q));
+}
+
 __global__ void __launch_bounds__(256) prepass_kernel(const __grid_constant__ LaunchArgs a) {
   dev::pdl_trigger();
   const int j = dev::find_job_block(a, blockIdx.x);
@@ -94,9 +168,10 @@ __global__ void __launch_bounds__(256) prepass_kernel(const __grid_constant__ La
     J.ref[2] = rr[2];
     J.ref[3] = K.t;
   }
-  if (k >= n) return;
   float v[kRecFields];
-  const bool valid = make_record(J, K, k, rr, v);
+  const bool valid = k < n && make_record(J, K, k, rr, v);
+  if (K.low_ok) call_extents(J, v, valid && !J.skip);
+  if (k >= n) return;
   if (!valid) atomicOr(J.status, ST_BAD_PARTICLE);
   // A particle that some direction of the grid may see beyond the fast phase
   // range makes the call wide (one atomic per warp that has one).  The bound
@@ -143,6 +218,8 @@ __device__ __forceinline__ int sort_bucket(const JobStatic& J, const JobCall& K,
   return min(kSortBuckets - 1, (int)floor(q + kHalf));
 }
 
+constexpr int kFewBuckets = 512;
+
 // Job of a sort-histogram block (jobs ordered by sort_block_begin).
 __device__ __forceinline__ int find_job_sort_block(const LaunchArgs& a, int block) {
   if (a.n_jobs == 1) return 0;
@@ -155,41 +232,101 @@ __device__ __forceinline__ int find_job_sort_block(const LaunchArgs& a, int bloc
   return lo;
 }
 
+// The bucket of particle k: along the sort axis (wide calls), or its cell (low
+// band; from the pre-pass's record).
+struct Buckets {
+  LowPlan plan;
+  int n;  // buckets in use (0: the call is not sorted)
+};
+__device__ __forceinline__ int bucket_of(const JobStatic& J, const JobCall& K, const Buckets& b, long long k) {
+  return b.plan.set >= 0 ? low_cell(J, b.plan, J.rec + (size_t)k * kRecFields) : sort_bucket(J, K, k);
+}
+
 // Per kSortBlock particles: bucket counts.
-__global__ void __launch_bounds__(256) wide_hist_kernel(const __grid_constant__ LaunchArgs a) {
+constexpr int kHistThreads = 1024;
+__global__ void __launch_bounds__(kHistThreads) wide_hist_kernel(const __grid_constant__ LaunchArgs a) {
   dev::pdl_trigger();
   dev::pdl_wait();
   const int j = find_job_sort_block(a, blockIdx.x);
   const JobStatic& J = a.js[j];
-  if (!call_is_wide(J)) return;
-  const JobCall K = a.use_inline ? a.inline_call : a.jc[j];
+  const JobCall& K = a.use_inline ? a.inline_call : a.jc[j];
+  Buckets B;
+  B.plan = low_plan(J, K);
+  B.n = call_is_wide(J) ? kSortBuckets : B.plan.cells;
+  if (B.n == 0) return;
   __shared__ int hist[kSortBuckets];
-  for (int b = threadIdx.x; b < kSortBuckets; b += blockDim.x) hist[b] = 0;
+  for (int b = threadIdx.x; b < B.n; b += blockDim.x) hist[b] = 0;
   __syncthreads();
   const long long blk = blockIdx.x - K.sort_block_begin;
   const long long k0 = blk * kSortBlock;
   for (int i = threadIdx.x; i < kSortBlock; i += blockDim.x)
-    if (k0 + i < K.n) atomicAdd(&hist[sort_bucket(J, K, k0 + i)], 1);
+    if (k0 + i < K.n) atomicAdd(&hist[bucket_of(J, K, B, k0 + i)], 1);
   __syncthreads();
   int* out = J.sort_counts + (size_t)blk * kSortBuckets;
-  for (int b = threadIdx.x; b < kSortBuckets; b += blockDim.x) out[b] = hist[b];
+  for (int b = threadIdx.x; b < B.n; b += blockDim.x) out[b] = hist[b];
 }
 
 // One block per job: per bucket, the prefix of the counts over the histogram
-// blocks (in place), and the first sorted position of every bucket.
+// blocks (in place), and the first sorted position of every bucket.  Also settles
+// the call's low-band plan for the kernels after it, and clears the extents
+// for the next call.
 __global__ void __launch_bounds__(1024) wide_scan_kernel(const __grid_constant__ LaunchArgs a) {
   dev::pdl_trigger();
   dev::pdl_wait();
   const JobStatic& J = a.js[blockIdx.x];
-  if (!call_is_wide(J)) return;
-  const JobCall K = a.use_inline ? a.inline_call : a.jc[blockIdx.x];
+  const JobCall& K = a.use_inline ? a.inline_call : a.jc[blockIdx.x];
+  __shared__ LowPlan s_plan;
+  if (K.low_ok) {
+    if (threadIdx.x == 0) {
+      s_plan = low_plan(J, K);
+      *J.plan = s_plan;
+      if (s_plan.set >= 0) atomicOr(a.any_wide + 1, 1);
+      for (int e = 0; e < 6; ++e) J.ext[e] = e & 1 ? INT_MIN : INT_MAX;
+    }
+  } else if (threadIdx.x == 0) {
+    s_plan.cells = 0;
+  }
+  __syncthreads();
+  const int n_b = call_is_wide(J) ? kSortBuckets : s_plan.cells;
+  if (n_b == 0) return;
   __shared__ int tot[kSortBuckets];
   __shared__ int wsum[32];
   const int nblk = (int)((K.n + kSortBlock - 1) / kSortBlock);
-  for (int b = threadIdx.x; b < kSortBuckets; b += 1024) {
+  // few buckets (cells): a warp per bucket, its lanes over the blocks
+  const bool few = n_b <= kFewBuckets;
+  if (few) {
+    for (int b = threadIdx.x; b < kSortBuckets; b += 1024) tot[b] = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int b = threadIdx.x >> 5; b < n_b; b += 32) {
+      int run = 0;
+      int* c = J.sort_counts + b;
+      for (int blk0 = 0; blk0 < nblk; blk0 += 128) {
+        int v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int blk = blk0 + 32 * u + lane;
+          v[u] = blk < nblk ? c[(size_t)blk * kSortBuckets] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int blk = blk0 + 32 * u + lane;
+          int x = v[u];
+          for (int off = 1; off < 32; off <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, off);
+            if (lane >= off) x += y;
+          }
+          if (blk < nblk) c[(size_t)blk * kSortBuckets] = run + x - v[u];
+          run += __shfl_sync(0xffffffffu, x, 31);
+        }
+      }
+      if (lane == 0) tot[b] = run;
+    }
+  }
+  for (int b = few ? kSortBuckets : threadIdx.x; b < kSortBuckets; b += 1024) {
     int run = 0;
     int* c = J.sort_counts + b;
-    int blk = 0;
+    int blk = b < n_b ? 0 : nblk;
     // eight independent loads in flight per step, then their prefix
     for (; blk + 8 <= nblk; blk += 8) {
       int v[8];
@@ -238,55 +375,102 @@ __global__ void __launch_bounds__(1024) wide_scan_kernel(const __grid_constant__
 
 // Per kSortBlock particles: the sorted position of every particle, stable
 // (particles of one bucket keep their order), so the order is a function of
-// the input alone.  The block computes the buckets into shared memory, then
-// one warp hands out the positions in particle order.
-__global__ void __launch_bounds__(256) wide_scatter_kernel(const __grid_constant__ LaunchArgs a) {
+// the input alone.  The block computes the buckets into shared memory; then, with
+// few buckets (cells), kRankWarps warps hand out the positions of an equal share
+// of the particles each, in particle order, after counting the shares (the sort
+// of 1e5 particles took 25 us here with one); with many, one warp does all.
+constexpr int kScatterThreads = 512, kRankWarps = 8;
+__global__ void __launch_bounds__(kScatterThreads) wide_scatter_kernel(const __grid_constant__ LaunchArgs a) {
   dev::pdl_trigger();
   dev::pdl_wait();
   const int j = find_job_sort_block(a, blockIdx.x);
   const JobStatic& J = a.js[j];
-  if (!call_is_wide(J)) return;
-  const JobCall K = a.use_inline ? a.inline_call : a.jc[j];
+  const JobCall& K = a.use_inline ? a.inline_call : a.jc[j];
+  Buckets B;
+  B.plan.set = -1;
+  B.plan.cells = 0;
+  if (K.low_ok) B.plan = *J.plan;
+  B.n = call_is_wide(J) ? kSortBuckets : B.plan.cells;
+  if (B.n == 0) return;
+  // next position of every bucket; with few buckets, of every warp's share
   __shared__ int cnt[kSortBuckets];
   __shared__ int bkt[kSortBlock];
+  static_assert(kRankWarps * kFewBuckets <= kSortBuckets, "the shares' counters");
+  const bool few = B.n <= kFewBuckets;
+  const int warps = few ? kRankWarps : 1, share = kSortBlock / warps;
   const long long blk = blockIdx.x - K.sort_block_begin;
   const long long k0 = blk * kSortBlock;
   const int* pre = J.sort_counts + (size_t)blk * kSortBuckets;
-  for (int b = threadIdx.x; b < kSortBuckets; b += blockDim.x) cnt[b] = J.bucket_base[b] + pre[b];
   for (int i = threadIdx.x; i < kSortBlock; i += blockDim.x)
-    bkt[i] = k0 + i < K.n ? sort_bucket(J, K, k0 + i) : -1;
+    bkt[i] = k0 + i < K.n ? bucket_of(J, K, B, k0 + i) : -1;
+  if (few) {
+    for (int i = threadIdx.x; i < kRankWarps * kFewBuckets; i += blockDim.x) cnt[i] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < kSortBlock; i += blockDim.x)
+      if (bkt[i] >= 0) atomicAdd(&cnt[(i / share) * kFewBuckets + bkt[i]], 1);
+    __syncthreads();
+  }
+  for (int b = threadIdx.x; b < B.n; b += blockDim.x) {
+    int at = J.bucket_base[b] + pre[b];
+    if (!few) cnt[b] = at;
+    for (int w = 0; few && w < kRankWarps; ++w) {
+      const int v = cnt[w * kFewBuckets + b];
+      cnt[w * kFewBuckets + b] = at;
+      at += v;
+    }
+  }
   __syncthreads();
-  if (threadIdx.x >= 32) return;
-  const int lane = threadIdx.x;
+  const int warp = threadIdx.x >> 5;
+  if (warp >= warps) return;
+  const int lane = threadIdx.x & 31;
+  int* next = cnt + warp * kFewBuckets;
   const unsigned below = (1u << lane) - 1u;
-  for (int it = 0; it < kSortBlock / 32; ++it) {
-    const long long k = k0 + it * 32 + lane;
+  for (int it = 0; it < share / 32; ++it) {
+    const int i = warp * share + it * 32 + lane;
+    const long long k = k0 + i;
     const bool in = k < K.n;
-    const int b = bkt[it * 32 + lane];
+    const int b = bkt[i];
     const unsigned peers = __match_any_sync(0xffffffffu, b);
-    const int pos = in ? cnt[b] + __popc(peers & below) : 0;
+    const int pos = in ? next[b] + __popc(peers & below) : 0;
     __syncwarp();
     if (in) {
       // positions are in [0, n) by construction; an inconsistency is reported
       // (the context then fails) instead of written
       if (pos >= 0 && pos < K.n) J.perm[pos] = (int)k;
       else atomicOr(J.status, ST_BOUNDS);
-      if (lane == 31 - __clz(peers)) cnt[b] += __popc(peers);
+      if (lane == 31 - __clz(peers)) next[b] += __popc(peers);
     }
     __syncwarp();
   }
 }
 
-// Records in sorted order, positions relative to the first particle of each
-// kGroup-particle group (its reference point); the group references relative
-// to the call's reference go to gref.
+// Wide calls: records in sorted order, positions relative to the first particle of
+// each kGroup-particle group (its reference point); the group references
+// relative to the call's reference go to gref.  Low band: the pre-pass's records
+// in cell order.
 __global__ void __launch_bounds__(256) wide_records_kernel(const __grid_constant__ LaunchArgs a) {
   dev::pdl_trigger();
   dev::pdl_wait();
   const int j = dev::find_job_block(a, blockIdx.x);
   const JobStatic& J = a.js[j];
-  if (!call_is_wide(J)) return;
-  const JobCall K = a.use_inline ? a.inline_call : a.jc[j];
+  const JobCall& K = a.use_inline ? a.inline_call : a.jc[j];
+  if (!call_is_wide(J)) {
+    if (!K.low_ok || J.plan->set < 0) return;
+    // five threads per record, 16 bytes each
+    constexpr int kQ = kRecFields / 4;
+    const long long b0 = (long long)(blockIdx.x - K.block_begin) * 256;
+    const int count = (int)min(256LL, K.n - b0);
+    for (int i = threadIdx.x; i < count * kQ; i += 256) {
+      const long long p = b0 + i / kQ;
+      int k = J.perm[p];
+      if (k < 0 || k >= K.n) {  // never, for a consistent sort
+        atomicOr(J.status, ST_BOUNDS);
+        k = 0;
+      }
+      reinterpret_cast<float4*>(J.rec_s)[p * kQ + i % kQ] = reinterpret_cast<const float4*>(J.rec)[(size_t)k * kQ + i % kQ];
+    }
+    return;
+  }
   static_assert(kGroup == 256, "one block per group");
   const long long p0 = (long long)(blockIdx.x - K.block_begin) * kGroup;
   const long long p = p0 + threadIdx.x;
@@ -658,9 +842,9 @@ cudaError_t launch_prepass(const LaunchArgs& a, int total_blocks, cudaStream_t s
 
 cudaError_t launch_wide(const LaunchArgs& a, int sort_blocks, int prepass_blocks, cudaStream_t s) {
   if (sort_blocks <= 0 || prepass_blocks <= 0) return cudaSuccess;
-  cudaError_t e = launch_pdl(wide_hist_kernel, sort_blocks, 256, 0, s, a);
+  cudaError_t e = launch_pdl(wide_hist_kernel, sort_blocks, kHistThreads, 0, s, a);
   if (e == cudaSuccess) e = launch_pdl(wide_scan_kernel, a.n_jobs, 1024, 0, s, a);
-  if (e == cudaSuccess) e = launch_pdl(wide_scatter_kernel, sort_blocks, 256, 0, s, a);
+  if (e == cudaSuccess) e = launch_pdl(wide_scatter_kernel, sort_blocks, kScatterThreads, 0, s, a);
   if (e == cudaSuccess) e = launch_pdl(wide_records_kernel, prepass_blocks, 256, 0, s, a);
   count_launches(kWideLaunches);
   return e;
@@ -685,6 +869,29 @@ void wide_geometry(const double* nd, int n_dir, float tau_fast, double axis[3], 
   // A group of sorted particles spans about two buckets along the axis: an
   // eighth of the fast range keeps it well inside.
   *bucket_w = (double)tau_fast * kC / 8.0;
+}
+
+void low_geometry(const double* nd, int n_dir, JobStatic& js) {
+  const double* n = js.axis;
+  int ax = 0;
+  if (fabs(n[1]) < fabs(n[ax])) ax = 1;
+  if (fabs(n[2]) < fabs(n[ax])) ax = 2;
+  double len = 0.0;
+  for (int i = 0; i < 3; ++i) {
+    js.fr1[i] = (i == ax) - n[ax] * n[i];
+    len += js.fr1[i] * js.fr1[i];
+  }
+  for (int i = 0; i < 3; ++i) js.fr1[i] /= sqrt(len);
+  for (int i = 0; i < 3; ++i)
+    js.fr2[i] = n[(i + 1) % 3] * js.fr1[(i + 2) % 3] - n[(i + 2) % 3] * js.fr1[(i + 1) % 3];
+  double c1 = 0.0, c2 = 0.0;
+  for (int d = 0; d < n_dir; ++d) {
+    const double* q = nd + 3 * (size_t)d;
+    c1 = std::max(c1, fabs(q[0] * js.fr1[0] + q[1] * js.fr1[1] + q[2] * js.fr1[2]));
+    c2 = std::max(c2, fabs(q[0] * js.fr2[0] + q[1] * js.fr2[1] + q[2] * js.fr2[2]));
+  }
+  js.cone1 = (float)c1;
+  js.cone2 = (float)c2;
 }
 
 cudaError_t launch_readout(const float* state, int mixed, const double* state64, int n_omega,

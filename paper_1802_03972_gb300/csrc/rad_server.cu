@@ -94,9 +94,15 @@ size_t estimate_footprint(const rad_job_desc& d) {
   const size_t grid = (size_t)resident_ctas(kDefaultVariant);
   const size_t tiles_per_nb = std::max<size_t>(1, nb / bins_per_tile);
   const size_t fine = 32 * bins_per_tile * (6 * grid + 12) + 40 * partials / tiles_per_nb;
+  // The low band's chunk sums (kLowItemsPerCta items per block, or chunks of
+  // kLowChunkMin, of 8 directions x up to n_omega bins) and its sorted records.
+  const size_t low = d.max_particles < kLowMin ? 0
+                         : 32 * 8 * (size_t)d.n_omega *
+                                   ((size_t)kLowItemsPerCta * grid + (size_t)(d.n_dir + 7) / 8) +
+                               80 * (size_t)d.max_particles;
   // Records (80 B per particle), the sort buffers of wide calls (13 B) and the
   // queued steps' staging slots (80 B each).
-  return nb * (64 + 24) + partials + fine +
+  return nb * (64 + 24) + partials + fine + low +
          (size_t)d.max_particles * (80 + 13 + 80 * (size_t)d.max_queued) +
          (size_t)d.n_omega * 48 + (size_t)d.n_dir * 72 + (1 << 16) + 4 * (size_t)kSortBuckets;
 }

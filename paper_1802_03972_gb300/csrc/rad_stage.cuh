@@ -223,5 +223,55 @@ __device__ __forceinline__ void tc_block(float2 pA, float2 pB, uint32_t b0, uint
            __float_as_uint(sbL.y), b0, b1);
 }
 
+// Variant 9's record of particle kk of a direction: dtau hi [kk]; the cross-term B
+// row [kk][8] as four pairs (terms c, c + 4), pair c of particle p at position
+// c ^ 2 ((p >> 2) & 1); the amplitudes' hi/lo parts [kk][12], 8 used.  The
+// swizzle and the 12-word stride keep the stores and the loop's loads free of
+// bank conflicts.
+__device__ __forceinline__ void store_record_xt(float th, float tl, const float a[4], int kk, float* xth,
+                                                float* xrt, float* xam) {
+  xth[kk] = th;
+  uint32_t thh, thl, tlh, tll;
+  split_tf32(th, thh, thl);
+  split_tf32(tl, tlh, tll);
+  float4* rp = reinterpret_cast<float4*>(xrt + (size_t)kk * 8);
+  const int sw = (kk >> 2) & 1;  // pairs 0, 1 and 2, 3 swap places
+  rp[sw] = make_float4(__uint_as_float(thh), __uint_as_float(tll), __uint_as_float(thl),
+                       __uint_as_float(tlh));
+  rp[sw ^ 1] = make_float4(__uint_as_float(thh), __uint_as_float(thl), __uint_as_float(tlh),
+                           __uint_as_float(tll));
+  const uint32_t h0 = tf32_hi(a[0]), h1 = tf32_hi(a[1]), h2 = tf32_hi(a[2]), h3 = tf32_hi(a[3]);
+  float4* ap = reinterpret_cast<float4*>(xam + (size_t)kk * 12);
+  ap[0] = make_float4(__uint_as_float(h0), __uint_as_float(h1), __uint_as_float(h2), __uint_as_float(h3));
+  ap[1] = make_float4(a[0] - __uint_as_float(h0), a[1] - __uint_as_float(h1),
+                      a[2] - __uint_as_float(h2), a[3] - __uint_as_float(h3));
+}
+
+// Variant 9's 8-particle step at kk over a warp's NB frequency blocks (lane (r, c) of
+// the fragments; xr_off: its cross-term pair within particle kk + r's row).
+// The main product's k = c and k = c + 4 are particles kk + 2c and kk + 2c + 1
+// (the columns of the cross-term result this lane holds).
+template <int NB>
+__device__ __forceinline__ void xt_step(const float* xtw, const float* xrw, const float* xaw, int kk, int r,
+                                        int c, int xr_off, const float2 (&omr)[NB], const float2 (&omr8)[NB],
+                                        const uint32_t (&xa)[NB][4], float (&dre)[NB][4], float (&dim)[NB][4]) {
+  const float2 th2 = *reinterpret_cast<const float2*>(xtw + kk + 2 * c);
+  const uint2 rt = *reinterpret_cast<const uint2*>(xrw + (size_t)(kk + r) * 8 + xr_off);
+  const uint32_t b0 = __float_as_uint(xaw[(kk + 2 * c) * 12 + r]);
+  const uint32_t b1 = __float_as_uint(xaw[(kk + 2 * c + 1) * 12 + r]);
+  // cr: rows r, r + 8 x particles kk + 2c, kk + 2c + 1.  All blocks' products
+  // first: one block's wait covers the next (0.1-1.3 % of a call).
+  float cr[NB][4];
+#pragma unroll
+  for (int b = 0; b < NB; ++b)
+    mma_tf32_zero(cr[b], xa[b][0], xa[b][1], xa[b][2], xa[b][3], rt.x, rt.y);
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    const float2 p0 = phase2x(omr[b], th2, make_float2(cr[b][0], cr[b][1]));
+    const float2 p8 = phase2x(omr8[b], th2, make_float2(cr[b][2], cr[b][3]));
+    tc_block(make_float2(p0.x, p8.x), make_float2(p0.y, p8.y), b0, b1, dre[b], dim[b]);
+  }
+}
+
 }  // namespace dev
 }  // namespace radimpl

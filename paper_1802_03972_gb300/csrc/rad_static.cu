@@ -171,7 +171,7 @@ extern "C" rad_status rad_accumulate_static(const double* omega, int32_t n_omega
   js.n_omega = n_omega;
   js.n_dir = n_dir;
   js.n_bins = n_omega * n_dir;
-  fill_tiles(js, variant, default_omega_tile(variant, n_omega));
+  fill_tiles(js, variant, default_omega_tile(variant, n_omega), 0);
   if (js.n_tiles > kMaxTiles) return RAD_EINVAL;
   int ck = auto_chunk_for(variant, n, js.n_tiles, false);  // (no fine-chunked tail here)
   int n_chunks = (int)((n + ck - 1) / ck);
@@ -219,7 +219,7 @@ extern "C" rad_status rad_accumulate_static(const double* omega, int32_t n_omega
   if (launch_prepass(a, (int)((n + 255) / 256), s) != cudaSuccess) return RAD_ECUDA;
   const long long grid = std::min<long long>(a.n_items, resident_ctas(variant));
   if (launch_accumulate(variant, a, (int)grid, s) != cudaSuccess) return RAD_ECUDA;
-  if (launch_reduce(a, reduce_blocks(js), s) != cudaSuccess) return RAD_ECUDA;
+  if (launch_reduce(a, reduce_blocks(js, nullptr), s) != cudaSuccess) return RAD_ECUDA;
   return RAD_OK;
 }
 
