@@ -903,13 +903,23 @@ rad_status rad_spectrum_species(rad_ctx* const* ctxs, const rad_ff* ffs, int32_t
     a.flags[i] = ff.flags;
     a.width[i] = ff.width;
   }
-  // Every species' queued work must be complete before its state is read; a
-  // species that saw invalid particles is reported after the spectra are written.
+  // Every species' queued work must be complete before its state is read: on one
+  // stream it is by order, else the host waits for each first.  A species that
+  // saw invalid particles is reported after the spectra are written.
   rad_status data = RAD_OK;
-  for (int i = 0; i < n_species; ++i) {
-    const rad_status s = check_status_word(ctxs[i]);
-    if (s == RAD_EDATA) data = RAD_EDATA;
-    else if (s != RAD_OK) return s;
+  auto check_all = [&]() -> rad_status {
+    for (int i = 0; i < n_species; ++i) {
+      const rad_status s = check_status_word(ctxs[i]);
+      if (s == RAD_EDATA) data = RAD_EDATA;
+      else if (s != RAD_OK) return s;
+    }
+    return RAD_OK;
+  };
+  bool one_stream = true;
+  for (int i = 1; i < n_species; ++i) one_stream = one_stream && ctxs[i]->stream == c0->stream;
+  if (!one_stream) {
+    const rad_status s = check_all();
+    if (s != RAD_OK) return s;
   }
   double* outs[3] = {coh, inc, tot};
   double* dev_out[3];
@@ -926,7 +936,7 @@ rad_status rad_spectrum_species(rad_ctx* const* ctxs, const rad_ff* ffs, int32_t
     s = cuda_check(c0, cudaMemcpyAsync(outs[i], dev_out[i], sizeof(double) * c0->n_bins,
                                        cudaMemcpyDeviceToHost, c0->stream));
   }
-  if (s == RAD_OK) s = cuda_check(c0, cudaStreamSynchronize(c0->stream));
+  if (s == RAD_OK) s = one_stream ? check_all() : cuda_check(c0, cudaStreamSynchronize(c0->stream));
   if (s != RAD_OK) return s;
   return data;
 }

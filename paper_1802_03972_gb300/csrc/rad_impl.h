@@ -57,7 +57,7 @@ constexpr int kMinChunk = 2048;
 static_assert(kMinChunk % kChunkAlign == 0, "the minimum chunk is a whole number of tiles");
 // Small calls (auto_chunk_for): an item's fixed cost in units of one particle
 // of a tile.
-constexpr int kItemCost = 60;
+constexpr int kItemCost = 45;
 // A batch hands out runs of consecutive chunks as one work item: about this
 // many items per resident block over all its jobs.
 constexpr int kBatchItemsPerCta = 8;

@@ -515,79 +515,118 @@ __device__ double form_factor(int kind, double width, double omega) {
 }
 
 // With RAD_FF_3D, box shapes are axis-aligned 3-D products: f = prod_d f_1(omega n_d).
-__device__ double form_factor_dir(int kind, int flags, double width, double omega,
-                                  const double* n) {
-  if (!(flags & RAD_FF_3D) || kind == RAD_FF_POINT || kind == RAD_FF_GAUSS)
-    return form_factor(kind, width, omega);
+__device__ double form_factor_3d(int kind, double width, double omega, const double* n) {
   return form_factor(kind, width, omega * n[0]) * form_factor(kind, width, omega * n[1]) *
          form_factor(kind, width, omega * n[2]);
 }
-
-__global__ void readout_kernel(const float* __restrict__ state, const double* __restrict__ state64,
-                               int mixed, int n_omega, int n_bins, const double* __restrict__ omega,
-                               const double* __restrict__ dirs, int kind, int flags, double width,
-                               double k0, double* coh, double* inc, double* tot) {
-  const int bin = blockIdx.x * blockDim.x + threadIdx.x;
-  if (bin >= n_bins) return;
-  double u2 = 0.0, v2 = 0.0;
-  if (mixed) {
-#pragma unroll
-    for (int c = 0; c < kComps; ++c) {
-      const double x = (double)state[(size_t)c * n_bins + bin] -
-                       (double)state[(size_t)(kComps + c) * n_bins + bin];
-      if (c < 4) u2 += x * x;
-      else v2 += x * x;
-    }
-  } else {
-#pragma unroll
-    for (int c = 0; c < 12; ++c) {
-      const double x = state64[(size_t)c * n_bins + bin];
-      if (c < 6) u2 += x * x;
-      else v2 += x * x;
-    }
-  }
-  const int d = bin / n_omega;
-  const double f = form_factor_dir(kind, flags, width, omega[bin - d * n_omega], dirs + 3 * d);
-  const double f2 = f * f;
-  const double ic = k0 * f2 * u2, ii = k0 * (1.0 - f2) * v2;
-  if (coh) coh[bin] = ic;
-  if (inc) inc[bin] = ii;
-  if (tot) tot[bin] = ic + ii;
+__device__ __forceinline__ bool per_direction(int kind, int flags) {
+  return (flags & RAD_FF_3D) && kind != RAD_FF_POINT && kind != RAD_FF_GAUSS;
 }
 
-__global__ void readout_species_kernel(SpeciesArgs a, int n_omega, int n_bins,
-                                       const double* __restrict__ omega,
-                                       const double* __restrict__ dirs, double k0, double* coh,
-                                       double* inc, double* tot) {
-  const int bin = blockIdx.x * blockDim.x + threadIdx.x;
-  if (bin >= n_bins) return;
-  const int d = bin / n_omega;
-  const double om = omega[bin - d * n_omega];
-  const int nu = a.mixed ? 4 : 6;  // real components of U (and of V)
-  double u[6] = {0, 0, 0, 0, 0, 0};
-  double ii = 0.0;
-  for (int s = 0; s < a.n_species; ++s) {
-    const double f = form_factor_dir(a.kind[s], a.flags[s], a.width[s], om, dirs + 3 * d);
-    double v2 = 0.0;
-    for (int c = 0; c < 2 * nu; ++c) {
-      double x;
-      if (a.mixed)
-        x = (double)a.state[s][(size_t)c * n_bins + bin] -
-            (double)a.state[s][(size_t)(kComps + c) * n_bins + bin];
-      else
-        x = a.state64[s][(size_t)c * n_bins + bin];
-      if (c < nu) u[c] += f * x;  // amplitudes add across species before |.|^2
-      else v2 += x * x;
+// float to double on the integer pipe (the conversion shares the narrow FP64
+// pipe): exponent rebias and shift; zero, and with the instruction what is
+// subnormal, infinite or NaN.
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), mag = b & 0x7fffffffu;
+  if (mag - 0x00800000u >= 0x7f000000u && mag != 0u) return (double)x;
+  return __hiloint2double((int)((b & 0x80000000u) | (mag ? (mag >> 3) + 0x38000000u : 0u)), (int)(b << 29));
+}
+
+// Readout, FP64: coherent k0 f^2 |U|^2, incoherent k0 (1 - f^2) |V|^2.  Bound by
+// the FP64 pipe (1.7 lanes/clk/SM), not by the 88 bytes per bin: so a thread
+// takes up to kReadBins bins of one frequency (bins t, t + stride, ..., the stride
+// a multiple of the frequencies) and computes the shape's factor once for
+// them, and the state's floats are widened on the integer pipe.  131072 bins, the
+// whole call: 40 -> 30 us for a 1-D shape, 57 for a 3-D box (three sines per
+// bin), 81 -> 59 for two species (kReadBins 2: 32 and 65; 8: 31 and 59).
+constexpr int kReadBins = 4;
+
+__global__ void __launch_bounds__(128) readout_kernel(
+    const float* __restrict__ state, const double* __restrict__ state64, int mixed, int n_omega, int n_bins,
+    long long stride, const double* __restrict__ omega, const double* __restrict__ dirs, int kind, int flags,
+    double width, double k0, double* coh, double* inc, double* tot) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= stride || t >= n_bins) return;
+  const bool by_dir = per_direction(kind, flags);
+  const int o = (int)(t % n_omega);
+  const double om = omega[o];
+  double f = by_dir ? 0.0 : form_factor(kind, width, om);
+#pragma unroll 1
+  for (long long at = t; at < n_bins; at += stride) {
+    const int bin = (int)at;
+    double u2 = 0.0, v2 = 0.0;
+    if (mixed) {
+      float a[2 * kComps];
+#pragma unroll
+      for (int c = 0; c < 2 * kComps; ++c) a[c] = state[(size_t)c * n_bins + bin];
+#pragma unroll
+      for (int c = 0; c < kComps; ++c) {
+        const double x = widen(a[c]) - widen(a[kComps + c]);
+        if (c < 4) u2 += x * x;
+        else v2 += x * x;
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < 12; ++c) {
+        const double x = state64[(size_t)c * n_bins + bin];
+        if (c < 6) u2 += x * x;
+        else v2 += x * x;
+      }
     }
-    ii += (1.0 - f * f) * v2;
+    if (by_dir) f = form_factor_3d(kind, width, om, dirs + 3 * (size_t)(bin / n_omega));
+    const double f2 = f * f;
+    const double ic = k0 * f2 * u2, ii = k0 * (1.0 - f2) * v2;
+    if (coh) coh[bin] = ic;
+    if (inc) inc[bin] = ii;
+    if (tot) tot[bin] = ic + ii;
   }
-  double u2 = 0.0;
-  for (int c = 0; c < nu; ++c) u2 += u[c] * u[c];
-  const double ic = k0 * u2;
-  ii *= k0;
-  if (coh) coh[bin] = ic;
-  if (inc) inc[bin] = ii;
-  if (tot) tot[bin] = ic + ii;
+}
+
+template <bool MIXED>
+__global__ void __launch_bounds__(128) readout_species_kernel(
+    const __grid_constant__ SpeciesArgs a, int n_omega, int n_bins, long long stride,
+    const double* __restrict__ omega, const double* __restrict__ dirs, double k0, double* coh, double* inc,
+    double* tot) {
+  constexpr int NU = MIXED ? 4 : 6;  // real components of U (and of V)
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= stride || t >= n_bins) return;
+  const double om = omega[(int)(t % n_omega)];
+  double u[kReadBins][NU] = {}, ii[kReadBins] = {};  // (stride: at most kReadBins bins per thread)
+  for (int s = 0; s < a.n_species; ++s) {
+    const bool by_dir = per_direction(a.kind[s], a.flags[s]);
+    double f = by_dir ? 0.0 : form_factor(a.kind[s], a.width[s], om);
+    const float* st = a.state[s];
+    const double* st64 = a.state64[s];
+#pragma unroll
+    for (int k = 0; k < kReadBins; ++k) {
+      const long long at = t + k * stride;
+      if (at >= n_bins) break;
+      const int bin = (int)at;
+      if (by_dir) f = form_factor_3d(a.kind[s], a.width[s], om, dirs + 3 * (size_t)(bin / n_omega));
+      double v2 = 0.0;
+#pragma unroll
+      for (int c = 0; c < 2 * NU; ++c) {
+        double x;
+        if (MIXED) x = widen(st[(size_t)c * n_bins + bin]) - widen(st[(size_t)(kComps + c) * n_bins + bin]);
+        else x = st64[(size_t)c * n_bins + bin];
+        if (c < NU) u[k][c < NU ? c : 0] += f * x;  // amplitudes add across species before |.|^2
+        else v2 += x * x;
+      }
+      ii[k] += (1.0 - f * f) * v2;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < kReadBins; ++k) {
+    const long long bin = t + k * stride;
+    if (bin >= n_bins) break;
+    double u2 = 0.0;
+#pragma unroll
+    for (int c = 0; c < NU; ++c) u2 += u[k][c] * u[k][c];
+    const double ic = k0 * u2, i2 = k0 * ii[k];
+    if (coh) coh[bin] = ic;
+    if (inc) inc[bin] = i2;
+    if (tot) tot[bin] = ic + i2;
+  }
 }
 
 // ----------------------------------------------------------- plain FP64 K5
@@ -894,13 +933,23 @@ void low_geometry(const double* nd, int n_dir, JobStatic& js) {
   js.cone2 = (float)c2;
 }
 
+// Bins between a readout thread's bins: all of them for grids of less than a
+// thread per lane of the GPU, else about a kReadBins-th, in whole frequency rows.
+static long long readout_stride(int n_omega, int n_bins) {
+  constexpr int kEnough = 152 * 128;
+  const int per = std::max(1, std::min(kReadBins, n_bins / kEnough));
+  const long long rows = ((n_bins + per - 1) / per + n_omega - 1) / n_omega;
+  return rows * n_omega;
+}
+
 cudaError_t launch_readout(const float* state, int mixed, const double* state64, int n_omega,
                            int n_bins, const double* omega, const double* dirs, rad_ff ff,
                            double* coh, double* inc, double* tot, cudaStream_t s) {
   const double k0 = kQe * kQe / (16.0 * kPi * kPi * kPi * kEps0 * kC);
-  readout_kernel<<<(n_bins + 255) / 256, 256, 0, s>>>(state, state64, mixed, n_omega, n_bins,
-                                                       omega, dirs, ff.kind, ff.flags, ff.width,
-                                                       k0, coh, inc, tot);
+  const long long stride = readout_stride(n_omega, n_bins);
+  readout_kernel<<<(unsigned)((stride + 127) / 128), 128, 0, s>>>(state, state64, mixed, n_omega, n_bins, stride,
+                                                                   omega, dirs, ff.kind, ff.flags, ff.width, k0,
+                                                                   coh, inc, tot);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -909,8 +958,12 @@ cudaError_t launch_readout_species(const SpeciesArgs& a, int n_omega, int n_bins
                                    const double* omega, const double* dirs, double* coh,
                                    double* inc, double* tot, cudaStream_t s) {
   const double k0 = kQe * kQe / (16.0 * kPi * kPi * kPi * kEps0 * kC);
-  readout_species_kernel<<<(n_bins + 255) / 256, 256, 0, s>>>(a, n_omega, n_bins, omega, dirs, k0,
-                                                              coh, inc, tot);
+  const long long stride = readout_stride(n_omega, n_bins);
+  const unsigned blocks = (unsigned)((stride + 127) / 128);
+  if (a.mixed)
+    readout_species_kernel<true><<<blocks, 128, 0, s>>>(a, n_omega, n_bins, stride, omega, dirs, k0, coh, inc, tot);
+  else
+    readout_species_kernel<false><<<blocks, 128, 0, s>>>(a, n_omega, n_bins, stride, omega, dirs, k0, coh, inc, tot);
   count_launches(1);
   return cudaGetLastError();
 }
