@@ -347,20 +347,24 @@ inline bool variant_tensor_core(int v) { return v == 3 || v == 4 || v == 7 || v 
 
 #ifdef __CUDACC__
 // Launches a kernel of a call's chain with programmatic dependent launch (see
-// pdl_trigger): its set-up overlaps the kernel before it.
+// pdl_trigger): its set-up overlaps the kernel before it.  cluster: blocks per
+// cluster (0: none).
 template <class Kernel, class Args>
 inline cudaError_t launch_pdl(Kernel k, long long grid, int threads, size_t smem, cudaStream_t s,
-                              const Args& a) {
+                              const Args& a, int cluster = 0) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute at = {};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute at[2] = {};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cluster;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 0 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, k, a);
 }
 #endif
@@ -371,7 +375,8 @@ cudaError_t launch_prepass(const LaunchArgs& a, int total_blocks, cudaStream_t s
 // The wide-call kernels (histogram, scan, scatter, sorted records), launched
 // after the pre-pass; each returns at once for jobs whose call is not wide.
 // sort_blocks / prepass_blocks: the calls' ceil(n / kSortBlock) and
-// ceil(n / 256) summed over the jobs.  Adds 4 to the launch count.
+// ceil(n / 256) summed over the jobs.  Adds 4 to the launch count, or 1 for a
+// single small call, whose sort is one kernel.
 cudaError_t launch_wide(const LaunchArgs& a, int sort_blocks, int prepass_blocks, cudaStream_t s);
 constexpr int kWideLaunches = 4;
 // Sort axis and bucket width of a job (host, at creation).
