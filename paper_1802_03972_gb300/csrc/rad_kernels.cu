@@ -154,6 +154,7 @@ __device__ __forceinline__ int low_cell(const JobStatic& J, const LowPlan& p, co
 
 __global__ void __launch_bounds__(256) prepass_kernel(const __grid_constant__ LaunchArgs a) {
   dev::pdl_trigger();
+  dev::pdl_wait();  // (of the stream's last kernel: a call's chain may follow another's)
   const int j = dev::find_job_block(a, blockIdx.x);
   const JobStatic& J = a.js[j];
   const JobCall K = a.use_inline ? a.inline_call : a.jc[j];
@@ -923,9 +924,8 @@ void count_launches(int n) { g_launches.fetch_add(n); }
 
 cudaError_t launch_prepass(const LaunchArgs& a, int total_blocks, cudaStream_t s) {
   if (total_blocks <= 0) return cudaSuccess;
-  prepass_kernel<<<total_blocks, 256, 0, s>>>(a);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_pdl(prepass_kernel, total_blocks, 256, 0, s, a);
 }
 
 cudaError_t launch_wide(const LaunchArgs& a, int sort_blocks, int prepass_blocks, cudaStream_t s) {
