@@ -287,7 +287,7 @@ int auto_chunk_for(int variant, long long n, int n_tiles, bool fine_tail) {
   ck = (ck + kChunkAlign - 1) / kChunkAlign * kChunkAlign;
   if (ck >= kMinChunk) return (int)std::min(ck, 1LL << 30);
   long long best = 0, best_cost = 0;
-  for (long long c = kSmallestChunk; c <= kMinChunk; c += c < kChunkAlign ? c : kChunkAlign) {
+  for (long long c = n <= kGroup ? kTinyChunk : kSmallestChunk; c <= kMinChunk; c += c < kChunkAlign ? c : kChunkAlign) {
     const long long per_tile = (n + c - 1) / c, waves = (per_tile * n_tiles + resident - 1) / resident;
     if (c < kChunkAlign && waves > 1) continue;
     const long long cost = waves * (std::min(c, n) + kItemCost);

@@ -33,7 +33,13 @@ constexpr int kOmTab = 3;
 // (small calls): no shared-memory tile (threads / directions-per-tile particles
 // at most) then crosses a 256-particle group of a wide call.
 constexpr int kChunkAlign = 256;
-constexpr int kSmallestChunk = 32;
+// 8 steps of 1777 particles, 96 x 25 bins, take 347 us with chunks of 256 or
+// more, 275 with 128, 265 with 32; a batch of 40 jobs of 500-3000 particles
+// (8 rounds) 4.9, 5.0 and 5.3 ms: every chunk writes its sums.
+constexpr int kSmallestChunk = 128;
+// ... and 32 for calls of at most one sorted group, whose items are few in any
+// launch (16 helix steps of 64 particles: 307 us with 64-particle chunks, 287 with 32).
+constexpr int kTinyChunk = 32;
 // Levels of fine-chunked last tiles (TailPlan).
 constexpr int kTailLevels = 2;
 // Automatic chunking aims at this many (coarse) work items per resident
@@ -59,8 +65,10 @@ static_assert(kMinChunk % kChunkAlign == 0, "the minimum chunk is a whole number
 // of a tile.
 constexpr int kItemCost = 45;
 // A batch hands out runs of consecutive chunks as one work item: about this
-// many items per resident block over all its jobs.
-constexpr int kBatchItemsPerCta = 8;
+// many items per resident block over all its jobs (64 jobs of up to 1e6 particles:
+// 1.85e12 updates/s with 5, 1.94 with 8, 1.98 with 12, 2.04 with 20; 64 jobs of
+// 1e3-1e4 particles 1.23, 1.26, 1.27, 1.27).
+constexpr int kBatchItemsPerCta = 20;
 
 // Wide calls (particles farther than half the fast phase range from the
 // call's reference point): a stable bucket sort along the grid's mean

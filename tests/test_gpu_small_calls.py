@@ -1,4 +1,4 @@
-"""Small calls: chunks below 256 particles, one chunk per tile, tiles of many chunks, grids that are no multiple of four
+"""Small calls: chunks of 128 particles, one chunk per tile, tiles of many chunks, grids that are no multiple of four
 frequencies (the tile reduction's scalar path), ragged tiles and directions; alone, batched and replayed from a graph."""
 import numpy as np
 import pytest
@@ -17,7 +17,7 @@ from paper_1802_03972_gb300 import build as _build  # noqa: E402
 _build.build()
 from paper_1802_03972_gb300 import rad  # noqa: E402
 
-# (particles, frequencies, directions): one particle; one tile of 32-particle chunks; many chunks of one tile; a
+# (particles, frequencies, directions): one particle; one chunk; many chunks of one tile; a
 # frequency count that is no multiple of 4; one frequency; a tile's last directions and frequencies outside the grid
 SIZES = [(1, 1, 1), (33, 64, 1), (5000, 64, 3), (300, 99, 5), (777, 1, 37), (2049, 130, 9), (20000, 257, 2)]
 
