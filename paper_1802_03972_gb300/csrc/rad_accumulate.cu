@@ -841,9 +841,10 @@ __device__ __forceinline__ LowTile low_tile(long long pos, long long cell_end, i
 
 // Particle-side factor of the interpolation, 1 / (the window's Fourier transform
 // at x / (2 kLowOversample), x = tau / H): a polynomial in x^2 fitted to
-// quadratures of the transform (relative error 1e-7 in FP32 on |x| <= 1).
+// quadratures of the transform (relative error 1e-7 in FP32 on |x| <= 1).  Only
+// records of invalid particles, of zero weight, lie outside: kept finite.
 __device__ __forceinline__ float low_factor(float x) {
-  const float y = x * x;
+  const float y = fminf(x * x, 1.0f);
   float p = 0.00316812399f;
   p = fmaf(p, y, -0.00347217099f);
   p = fmaf(p, y, 0.0177691517f);

@@ -204,15 +204,16 @@ void fill_tiles(JobStatic& js, int variant, int wt, int n_low) {
 // numbers of bins js that pay when taken from nodes (the remaining tiles and
 // the nodes, kLowCost of a full tile per direction group, below 0.92 of the full
 // tiling), cheapest first, a factor of two apart in H at least.  Tables: per
-// alternative the nodes' frequency table and the interpolation weights, appended
-// to `tab`; L.nodes and L.wts hold their offsets until they are uploaded.
+// alternative the nodes' frequency table and the interpolation weights, after
+// the om_tab of `tab` floats; L.nodes and L.wts are byte offsets until the
+// allocation is there, and launch_low_tables fills them.
 constexpr double kLowCost = 1.3;
 // Particles of a tile per resident block that the low band has to save: the sort and the
 // waves of smaller launches (about 200 us).  20000 particles, 512 x 64 bins
 // would take 475 us with it, 450 without; 40000, 1000 x 32 865 and 815; 1e5,
 // 512 x 256 4930 and 6790; 1e6, 1024 x 256 77.4 and 132.2 ms.
 constexpr double kLowFixed = 2500.0;
-int low_alternatives(const JobStatic& js, const double* omega, std::vector<float>& tab, LowSet* low, double* full) {
+int low_alternatives(const JobStatic& js, const double* omega, size_t& tab, LowSet* low, double* full) {
   for (int i = 1; i < js.n_omega; ++i)
     if (!(omega[i] > omega[i - 1])) return 0;
   struct Cand { int js; double cost; };
@@ -238,29 +239,12 @@ int low_alternatives(const JobStatic& js, const double* omega, std::vector<float
     L.js = q.js;
     L.hi_cost = (float)(make_segments(kDefaultVariant, js.n_omega, js.n_dir, q.js, L.seg, L.n_seg, L.n_tiles));
     L.H = (float)H;
-    L.nodes = reinterpret_cast<const float*>(tab.size());
-    for (int part = 0; part < kOmTab; ++part)
-      for (int i = 0; i < kLowNodes; ++i) {
-        const double nu = (i - kLowTaps / 2) * dnu;
-        const float hi = (float)nu;
-        tab.push_back(part == 0 ? hi : (float)(kTwoPi * (part == 1 ? (double)hi : nu - (double)hi)));
-      }
-    while (tab.size() & 3) tab.push_back(0.0f);  // (read 16 bytes at a time)
-    L.wts = reinterpret_cast<const float*>(tab.size());
-    for (int i = 0; i < q.js; ++i) {
-      const double s = omega[i] / kTwoPi / dnu;  // in node spacings, from frequency 0
-      const int base = (int)std::min(floor(s), (double)kLowReach);
-      // taps at base - kLowTaps/2 + 1 .. base + kLowTaps/2; node 0 is -kLowTaps/2
-      for (int t = 0; t < kLowTaps; ++t) {
-        const double u = (s - (base - kLowTaps / 2 + 1 + t)) / (0.5 * kLowTaps);
-        tab.push_back(fabs(u) < 1.0 ? (float)exp(kLowBeta * (sqrt(1.0 - u * u) - 1.0)) : 0.0f);
-      }
-      float index;
-      const int first = base + 1;
-      memcpy(&index, &first, sizeof(float));
-      tab.push_back(index);
-      tab.push_back(0.0f);
-    }
+    tab = (tab + 3) & ~(size_t)3;  // (read 16 bytes at a time)
+    L.dnu = dnu;
+    L.nodes = reinterpret_cast<float*>(tab * sizeof(float));
+    tab += kOmTab * kLowNodes;
+    L.wts = reinterpret_cast<float*>(tab * sizeof(float));
+    tab += (size_t)kLowWt * q.js;
   }
   return n;
 }
@@ -678,7 +662,8 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
   js.tau_fast = (float)(2097152.0 / std::max(om_hi_max, 1e-300));  // 2^21 turns
   wide_geometry(nd.data(), n_dir, js.tau_fast, js.axis, &js.cone_sin, &js.bucket_w);
   low_geometry(nd.data(), n_dir, js);
-  if (prec == RAD_PREC_MIXED && !literal) c->n_low = low_alternatives(js, omega, om_tab, c->low, &c->low_full);
+  size_t tab_floats = om_tab.size();
+  if (prec == RAD_PREC_MIXED && !literal) c->n_low = low_alternatives(js, omega, tab_floats, c->low, &c->low_full);
   fill_tiles(js, c->tile.variant, c->tile.omega_tile, c->n_low);
 
   rad_status s = RAD_OK;
@@ -688,7 +673,7 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
   };
   chk(dmalloc(&c->d_omega, n_omega));
   chk(dmalloc(&c->d_om_turns, n_omega));
-  chk(dmalloc(&c->d_om_tab, om_tab.size()));
+  chk(dmalloc(&c->d_om_tab, tab_floats));
   chk(dmalloc(&c->d_dirs, nd.size()));
   chk(dmalloc(&c->d_dir_tab, dir_tab.size()));
   chk(dmalloc(&c->d_ref, 4));
@@ -716,8 +701,8 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
   // the low band's alternatives go after the status words
   js.low = reinterpret_cast<const LowSet*>(c->d_status + kStatusWords);
   for (int i = 0; i < c->n_low; ++i) {
-    c->low[i].nodes = c->d_om_tab + reinterpret_cast<size_t>(c->low[i].nodes);
-    c->low[i].wts = c->d_om_tab + reinterpret_cast<size_t>(c->low[i].wts);
+    c->low[i].nodes = c->d_om_tab + reinterpret_cast<size_t>(c->low[i].nodes) / sizeof(float);
+    c->low[i].wts = c->d_om_tab + reinterpret_cast<size_t>(c->low[i].wts) / sizeof(float);
   }
   if (s == RAD_OK) {
     chk(cudaMemcpy(c->d_omega, omega, sizeof(double) * n_omega, cudaMemcpyHostToDevice));
@@ -768,6 +753,7 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
     fill_tiles(js, c->tile.variant, c->tile.omega_tile, 0);
   }
   if (s == RAD_OK) chk(cudaMemcpy(c->d_js, &js, sizeof(JobStatic), cudaMemcpyHostToDevice));
+  if (s == RAD_OK && c->n_low > 0) chk(launch_low_tables(js, c->n_low, c->stream));
   if (s != RAD_OK) {
     rad_destroy(c);
     return s;

@@ -138,8 +138,9 @@ struct LowSet {
   float H;               // half-range of a cell's retarded times, s
   float hi_cost;         // of the other bins' tiles, in full tiles
   TileSeg seg[kMaxSegs];
-  const float* nodes;    // [kOmTab][kLowNodes], as om_tab
-  const float* wts;      // [js][kLowWt]
+  double dnu;            // node spacing, turns/s
+  float* nodes;          // [kOmTab][kLowNodes], as om_tab
+  float* wts;            // [js][kLowWt]
 };
 // What a call does (written by the scan kernel): the alternative taken (-1:
 // none) and its cells, of width h from s0 along the axis, centred on c1, c2
@@ -390,6 +391,8 @@ constexpr int kWideLaunches = 4;
 // Sort axis and bucket width of a job (host, at creation).
 void wide_geometry(const double* unit_dirs, int n_dir, float tau_fast, double axis[3],
                    double* cone_sin, double* bucket_w);
+// Fills the tables of the context's n alternatives.
+cudaError_t launch_low_tables(const JobStatic& js, int n, cudaStream_t s);
 // Transverse frame of the sort axis and the grid's reach along it (low band).
 void low_geometry(const double* unit_dirs, int n_dir, JobStatic& js);
 // Launches the accumulate kernel, and the reduction of its partial sums into the

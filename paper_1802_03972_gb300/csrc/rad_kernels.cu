@@ -549,6 +549,34 @@ __global__ void __launch_bounds__(1024) wide_small_kernel(const __grid_constant_
     wide_record(J, K, p / kGroup * kGroup, p);
 }
 
+// An alternative's tables (LowSet): the nodes' frequency factors, and per bin of the
+// band its taps' weights (of the window) and first node.
+__global__ void __launch_bounds__(128) low_tables_kernel(const LowSet* __restrict__ sets,
+                                                         const double* __restrict__ om_turns) {
+  const LowSet& L = sets[blockIdx.y];
+  constexpr double k2Pi = 6.283185307179586476925286766559;
+  if (blockIdx.x == 0 && threadIdx.x < kLowNodes) {
+    const int i = threadIdx.x;
+    const double nu = (i - kLowTaps / 2) * L.dnu;
+    const float hi = __double2float_rn(nu);
+    L.nodes[i] = hi;
+    L.nodes[kLowNodes + i] = __double2float_rn(k2Pi * (double)hi);
+    L.nodes[2 * kLowNodes + i] = __double2float_rn(k2Pi * (nu - (double)hi));
+  }
+  const int j = blockIdx.x * 128 + threadIdx.x;
+  if (j >= L.js) return;
+  const double s = om_turns[j] / L.dnu;  // in node spacings, from frequency 0
+  const int base = min((int)floor(s), kLowReach);
+  float* w = L.wts + (size_t)j * kLowWt;
+  // taps at base - kLowTaps/2 + 1 .. base + kLowTaps/2; node 0 is -kLowTaps/2
+  for (int t = 0; t < kLowTaps; ++t) {
+    const double u = (s - (base - kLowTaps / 2 + 1 + t)) / (0.5 * kLowTaps);
+    w[t] = fabs(u) < 1.0 ? __double2float_rn(exp(kLowBeta * (sqrt(1.0 - u * u) - 1.0))) : 0.0f;
+  }
+  w[kLowTaps] = __int_as_float(base + 1);
+  w[kLowTaps + 1] = 0.0f;
+}
+
 // ------------------------------------------------------------------ readout
 __device__ double sinc(double x) { return x == 0.0 ? 1.0 : sin(x) / x; }
 
@@ -984,6 +1012,12 @@ void low_geometry(const double* nd, int n_dir, JobStatic& js) {
   }
   js.cone1 = (float)c1;
   js.cone2 = (float)c2;
+}
+
+cudaError_t launch_low_tables(const JobStatic& js, int n, cudaStream_t s) {
+  low_tables_kernel<<<dim3((unsigned)((js.n_omega + 127) / 128), (unsigned)n), 128, 0, s>>>(js.low, js.om_turns);
+  count_launches(1);
+  return cudaGetLastError();
 }
 
 // Bins between a readout thread's bins: all of them for grids of less than a

@@ -67,16 +67,21 @@ def test_low_band_far_from_the_origin_and_off_axis():
     check(wl, arrays)
 
 
-def test_low_band_with_invalid_particles():
+@pytest.mark.parametrize("first", [False, True])
+def test_low_band_with_invalid_particles(first):
+    """Invalid particles at the end, or first (the call's reference is then the origin, a millimetre from the bunch)."""
     wl = workload(150000, 512, 8, 8)
     good = wl.step(0)
+    if first:
+        good.r = good.r.reshape(3, -1) + np.array([[1e-3], [2e-3], [-1e-3]])
     ctx = rad.Context(wl.omega, wl.dirs, wl.ff_kind, wl.ff_width)
     ref = rad.Context(wl.omega, wl.dirs, wl.ff_kind, wl.ff_width)
     ref.accumulate(*[to_dev(a) for a in (good.r, good.beta, good.beta_dot, good.w)], 0.0, 1e-16)
-    pad = lambda v, bad: np.concatenate([v.reshape(3, -1), np.array(bad, dtype=float).T], axis=1)  # noqa: E731
+    order = (lambda v, b: [b, v]) if first else (lambda v, b: [v, b])
+    pad = lambda v, bad: np.concatenate(order(v.reshape(3, -1), np.array(bad, dtype=float).T), axis=1)  # noqa: E731
     ctx.accumulate(to_dev(pad(good.r, [[np.nan, 0, 0], [0, 1.0, 0], [0, 0, np.inf]])),
                    to_dev(pad(good.beta, [[0, 0, .5], [0, 0, 1.5], [0, 0, .5]])),
-                   to_dev(pad(good.beta_dot, [[1e13, 0, 0]] * 3)), to_dev(np.concatenate([good.w, [10.0, 10.0, 10.0]])),
+                   to_dev(pad(good.beta_dot, [[1e13, 0, 0]] * 3)), to_dev(np.concatenate(order(good.w, [10.0, 10.0, 10.0]))),
                    0.0, 1e-16)
     with pytest.raises(rad.RadError) as ei:
         ctx.spectrum()
