@@ -668,10 +668,11 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
             }
           }
         };
-        // A full tile of one direction takes the loop with its trip count known at
-        // compile time (measured ~1 % faster); ragged and multi-direction tiles
-        // the runtime bound.
+        // Full tiles of one and two directions take the loop with its trip count
+        // known at compile time (LWFA step, two directions: 4880 -> 4726 us);
+        // ragged and narrower tiles the runtime bound.
         if (kn8 == THREADS) fast_loop(THREADS);
+        else if (kn8 == THREADS / 2) fast_loop(THREADS / 2);
         else fast_loop(kn8);
       } else {
         if (threadIdx.x == 0) atomicOr(J.status, ST_SLOW_PHASE);
@@ -819,7 +820,7 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
 // adds them to the chunk's sums.  Bound: MUFU, as the direct bins, for 64
 // frequencies instead of js; the interpolation is 10 taps x 8 sums per bin and
 // cell.  LWFA step (1e5 particles, 512 x 256 bins, 256 bins from nodes): 6.79 ->
-// 4.93 ms; 1e6 particles, 1024 x 256 bins (512 from nodes) 132.2 -> 77.4 ms.
+// 4.73 ms; 1e6 particles, 1024 x 256 bins (512 from nodes) 132.2 -> 76.4 ms.
 constexpr int kLowTile = 128;
 constexpr int kLowDirs = 8;
 
@@ -1097,7 +1098,11 @@ __device__ __forceinline__ void settle_plan(BlockState& b) {
   b.K.ck = C.ck_hi;
   b.K.n_chunks = C.n_hi;
   b.K.run = 1;
-  for (int l = 0; l < kTailLevels; ++l) b.K.tail_tiles[l] = 0;
+  for (int l = 0; l < kTailLevels; ++l) {
+    b.K.tail_tiles[l] = C.tail_tiles[l];
+    b.K.ck_f[l] = C.ck_f[l];
+    b.K.n_chunks_f[l] = C.n_chunks_f[l];
+  }
 }
 
 // Claims the pass's next item (thread 0's counter; a block's first item is its
@@ -1148,8 +1153,14 @@ __device__ __forceinline__ bool run_items(const LaunchArgs& a, BlockState& b, un
     if (b.any_wide && (b.J.wide_flag != nullptr && *b.J.wide_flag != 0) != WIDE) continue;  // the other pass's
     // Tile-major order: one tile's chunks run close together in time.
     const long long local = item - b.K.item_begin;
-    // (a call with the low band may have fewer items than its share of the range)
-    if (XT && b.plan.set >= 0 && local >= (long long)b.J.n_tiles * b.K.n_chunks) continue;
+    // (the range holds the most items over the call's alternatives)
+    if (XT && b.K.low_ok) {
+      const int t0 = b.K.tail_tiles[0], t1 = b.K.tail_tiles[1];
+      const int per_tile = (b.K.n_chunks + b.K.run - 1) / b.K.run;
+      if (local >= (long long)(b.J.n_tiles - t0 - t1) * per_tile + (long long)t0 * b.K.n_chunks_f[0] +
+                       (long long)t1 * b.K.n_chunks_f[1])
+        continue;
+    }
     const ItemRef it = decode_item<TC>(b.J, b.K, local);
     if (threadIdx.x == 0) {
       b.it.it = it;
@@ -1219,14 +1230,18 @@ __global__ void __launch_bounds__(THREADS, MINB) accumulate_kernel(const __grid_
     s_ns0 = global_ns();
   }
   uint32_t phase = 0u;
-  bool ok = run_items<THREADS, W, TC, LIT, PASSES, false, XT>(a, b, smem, &bar, phase);
+  // The low bands first: the bin tiles' fine-chunked last items end the launch
+  // (with the bands' items last the SMs were active for 96.1 % of it).
+  bool ok = true;
   if constexpr (XT) {
-    if (ok && b.any_low) {
+    __syncthreads();
+    if (b.any_low) {
+      ok = run_low<THREADS>(a, b, smem, bars_low);
       __syncthreads();
       if (threadIdx.x == 0) b.item = -1;
-      ok = run_low<THREADS>(a, b, smem, bars_low);
     }
   }
+  if (ok) ok = run_items<THREADS, W, TC, LIT, PASSES, false, XT>(a, b, smem, &bar, phase);
   if (ok && b.any_wide) {
     __syncthreads();
     if (threadIdx.x == 0) b.item = -1;

@@ -209,10 +209,10 @@ void fill_tiles(JobStatic& js, int variant, int wt, int n_low) {
 // allocation is there, and launch_low_tables fills them.
 constexpr double kLowCost = 1.3;
 // Particles of a tile per resident block that the low band has to save: the sort and the
-// waves of smaller launches (about 200 us).  20000 particles, 512 x 64 bins
-// would take 475 us with it, 450 without; 40000, 1000 x 32 865 and 815; 1e5,
-// 512 x 256 4930 and 6790; 1e6, 1024 x 256 77.4 and 132.2 ms.
-constexpr double kLowFixed = 2500.0;
+// waves of smaller launches (about 100 us).  With 600, 17000 particles, 1000 x
+// 16 bins (two steps) take 483 us instead of 454; with 2500, 25000 particles,
+// 400 x 100 bins 820 instead of 637, and 60000, 330 x 81 1274 instead of 1117.
+constexpr double kLowFixed = 1200.0;
 int low_alternatives(const JobStatic& js, const double* omega, size_t& tab, LowSet* low, double* full) {
   for (int i = 1; i < js.n_omega; ++i)
     if (!(omega[i] > omega[i - 1])) return 0;
@@ -391,10 +391,10 @@ CallPlan plan_call(const rad_ctx* c, const JobStatic& js, int variant, long long
   p.tail = tail_plan(variant_tensor_core(variant) && !js.literal, n, js.n_tiles, p.ck, p.n_chunks,
                      resident_ctas(variant));
   p.most_chunks = p.n_chunks;
+  p.fine_floats = p.tail.fine_floats(js.bpt);
   // The low band (automatic chunks, calls that are sorted when wide): per
-  // alternative, the other bins' tiles chunked as a job of their own (without the
-  // fine tail: the low band's items follow), and about kLowItemsPerCta items per
-  // resident block of the band.
+  // alternative, the other bins' tiles chunked as a job of their own, and about
+  // kLowItemsPerCta items per resident block of the band.
   if (js.n_low == 0 || c->tile.chunk != 0 || js.wide_flag == nullptr || n < kLowMin || n >= (1LL << 31))
     return p;
   const long long dirs8 = (js.n_dir + 7) / 8;
@@ -414,7 +414,10 @@ CallPlan plan_call(const rad_ctx* c, const JobStatic& js, int variant, long long
     if (saved < kLowFixed * resident_ctas(variant)) continue;
     p.low_ok |= 1u << s;
     p.most_chunks = std::max(p.most_chunks, C.n_hi);
-    p.hi_items = std::max(p.hi_items, (long long)L.n_tiles * C.n_hi);
+    const TailPlan tail = tail_plan(true, n, L.n_tiles, C.ck_hi, C.n_hi, resident_ctas(variant));
+    set_tail(C, tail);
+    p.fine_floats = std::max(p.fine_floats, tail.fine_floats(js.bpt));
+    p.hi_items = std::max(p.hi_items, tail.items(L.n_tiles, C.n_hi));
     p.low_items = std::max(p.low_items, dirs8 * C.n_lo);
     p.low_floats = std::max(p.low_floats, (long long)C.n_lo * kComps * js.n_dir * L.js);
   }
@@ -497,7 +500,7 @@ rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const do
   }
   const int variant = c->tile.variant;
   const CallPlan plan = plan_call(c, c->h_js, variant, n);
-  rad_status s = ensure_capacity(c, n, plan.most_chunks, plan.tail.fine_floats(c->h_js.bpt), plan.low_floats);
+  rad_status s = ensure_capacity(c, n, plan.most_chunks, plan.fine_floats, plan.low_floats);
   if (s != RAD_OK) return s;
   LaunchArgs a;
   memset(&a, 0, sizeof(a));

@@ -119,7 +119,7 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
     // chunked as the job alone would be (results equal bit for bit)
     const CallPlan call = plan_call(c, js, variant, steps[i].n);
     const int nch = call.most_chunks;
-    const long long fine = call.tail.fine_floats(js.bpt);
+    const long long fine = call.fine_floats;
     if (steps[i].n > c->h_js.n_cap || nch > c->h_js.chunk_cap || fine > c->h_js.fine_cap ||
         call.low_floats > c->h_js.low_cap) {
       if (!drained) {

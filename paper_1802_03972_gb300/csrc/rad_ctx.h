@@ -98,6 +98,7 @@ struct CallPlan {
   unsigned low_ok = 0;  // the alternatives that pay for this call (bits)
   LowCall low[kLowSets] = {};
   long long hi_items = 0, low_items = 0, low_floats = 0;
+  long long fine_floats = 0;  // of partials_f
   // items of the bin tiles (run: chunks per item), the most over the alternatives
   long long items(const JobStatic& js, int run) const;
   void fill(JobCall& K, const JobStatic& js, int run) const;

@@ -127,7 +127,7 @@ constexpr int kLowSets = 16;          // alternatives of one grid (bins in the b
 constexpr long long kLowMin = 16384;  // particles of a call from which the low band is considered
 constexpr int kLowCellMin = 64;       // ... and on average per cell
 constexpr int kLowMaxCells = 4000;
-constexpr int kLowItemsPerCta = 4;    // the band's work items per resident block
+constexpr int kLowItemsPerCta = 2;    // the band's work items per resident block
 constexpr int kLowChunkMin = 512;
 // A context's status allocation: the status word, the call's extents, its plan.
 constexpr int kStatusExt = 2, kStatusPlan = 8, kStatusWords = 16;
@@ -149,9 +149,11 @@ struct LowPlan {
   int set, cells;
   float s0, h, c1, c2;
 };
-// A call's chunks in an alternative: of its bin tiles and of the low band.
+// A call's chunks in an alternative: of its bin tiles, with their fine-chunked
+// last tiles (TailPlan), and of the low band.
 struct LowCall {
   int ck_hi, n_hi, ck_lo, n_lo;
+  int tail_tiles[kTailLevels], ck_f[kTailLevels], n_chunks_f[kTailLevels];
 };
 
 // Per-job data that does not change between calls.
@@ -295,7 +297,8 @@ inline TailPlan tail_plan(bool tensor_core, long long n, int n_tiles, int ck, in
   return t;
 }
 // The plan's fields of a call.
-inline void set_tail(JobCall& K, const TailPlan& t) {
+template <class Call>
+inline void set_tail(Call& K, const TailPlan& t) {
   for (int l = 0; l < kTailLevels; ++l) {
     K.tail_tiles[l] = t.lv[l].tiles;
     K.ck_f[l] = t.lv[l].ck;
