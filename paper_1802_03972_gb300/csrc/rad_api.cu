@@ -408,10 +408,13 @@ CallPlan plan_call(const rad_ctx* c, const JobStatic& js, int variant, long long
     C.ck_lo = (int)ck;
     C.n_lo = (int)((n + ck - 1) / ck);
     // What it saves, in particles of a tile: the bins' tiles against the nodes and
-    // an interpolation per direction and piece of a cell (about 64 cells).
-    const double saved = (c->low_full - L.hi_cost) * (double)n -
-                         (double)dirs8 * (kLowCost * (double)n + (C.n_lo + 64) * (64 + 0.5 * L.js));
-    if (saved < kLowFixed * resident_ctas(variant)) continue;
+    // an interpolation per direction and piece of a cell.  The cells' number is
+    // the device's: it may use three quarters of what is saved.
+    const double piece = (double)dirs8 * (64 + L.js);
+    const double saved = (c->low_full - L.hi_cost) * (double)n - (double)dirs8 * kLowCost * (double)n -
+                         C.n_lo * piece - kLowFixed * resident_ctas(variant);
+    C.max_cells = (int)std::min(0.75 * saved / piece, (double)kLowMaxCells);
+    if (C.max_cells < 8) continue;
     p.low_ok |= 1u << s;
     p.most_chunks = std::max(p.most_chunks, C.n_hi);
     const TailPlan tail = tail_plan(true, n, L.n_tiles, C.ck_hi, C.n_hi, resident_ctas(variant));

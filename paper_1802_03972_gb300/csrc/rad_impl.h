@@ -153,6 +153,7 @@ struct LowPlan {
 // last tiles (TailPlan), and of the low band.
 struct LowCall {
   int ck_hi, n_hi, ck_lo, n_lo;
+  int max_cells;  // more would cost more than the band saves
   int tail_tiles[kTailLevels], ck_f[kTailLevels], n_chunks_f[kTailLevels];
 };
 

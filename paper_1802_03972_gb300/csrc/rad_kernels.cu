@@ -135,7 +135,7 @@ __device__ __forceinline__ LowPlan low_plan(const JobStatic& J, const JobCall& K
     const float h = __fmul_rn(2.0f, __fsub_rn(__fmul_rn(0.998f, J.low[s].H), __fmul_rn(1.001f, side)));
     if (!(h > 0.0f)) continue;
     const float cells = __fadd_rn(__fdiv_rn(__fsub_rn(hi[2], lo[2]), h), 1.0f);
-    if (!(cells < (float)kLowMaxCells) || !(cells * kLowCellMin <= (float)K.n)) continue;
+    if (!(cells < (float)K.low[s].max_cells) || !(cells * kLowCellMin <= (float)K.n)) continue;
     p.set = s;
     p.cells = min((int)cells + 1, kLowMaxCells);
     p.s0 = lo[2];
