@@ -50,6 +50,12 @@ rad_status rad_selftest_stage1(rad_ctx* ctx, int64_t n, const double* r, const d
 rad_status rad_selftest_phase(rad_ctx* ctx, int32_t n_tau, const float* th, const float* tl,
                               float* fast, float* wide);
 
+/* rad_selftest_fail_alloc - the nth (from 1) of the context's next device buffer
+ * allocations for its calls' work (records, sort buffers, partial sums) fails as
+ * cudaMalloc does without memory, once; 0: none.  Allocates nothing itself.
+ * Errors: RAD_EINVAL for a NULL context or nth < 0. */
+rad_status rad_selftest_fail_alloc(rad_ctx* ctx, int32_t nth);
+
 #ifdef __cplusplus
 }
 #endif

@@ -63,7 +63,21 @@ template <class T>
 cudaError_t dmalloc(T** p, size_t count) {
   *p = nullptr;
   if (count == 0) return cudaSuccess;
-  return cudaMalloc((void**)p, count * sizeof(T));
+  const cudaError_t e = cudaMalloc((void**)p, count * sizeof(T));
+  if (e != cudaSuccess) cudaGetLastError();  // (else the next launch's check would report it again)
+  return e;
+}
+
+// A buffer named in the context's job table.  The device's copy of the table is
+// stale from here on, until upload_static has succeeded: a call that fails
+// between the two (RAD_ENOMEM leaves the context usable) must not leave the
+// next one, which may need no new buffer, with pointers to freed memory.
+template <class T>
+rad_status alloc_buffer(rad_ctx* c, T** p, size_t count) {
+  c->js_stale = true;
+  *p = nullptr;
+  if (c->fail_alloc > 0 && --c->fail_alloc == 0) return cuda_check(c, cudaErrorMemoryAllocation);
+  return cuda_check(c, dmalloc(p, count));
 }
 
 }  // namespace
@@ -291,12 +305,13 @@ int auto_chunk(const rad_ctx* c, int variant, long long n, int n_tiles) {
 
 rad_status upload_static(rad_ctx* c) {
   c->generation++;
-  return cuda_check(c, cudaMemcpyAsync(c->d_js, &c->h_js, sizeof(JobStatic),
-                                       cudaMemcpyHostToDevice, c->stream));
+  const rad_status s = cuda_check(c, cudaMemcpyAsync(c->d_js, &c->h_js, sizeof(JobStatic),
+                                                     cudaMemcpyHostToDevice, c->stream));
+  if (s == RAD_OK) c->js_stale = false;
+  return s;
 }
 
 rad_status ensure_capacity(rad_ctx* c, long long n, int n_chunks, long long fine_floats, long long low_floats) {
-  bool changed = false;
   if (n > c->h_js.n_cap) {
     long long cap = std::max(n, c->h_js.n_cap * 3 / 2);
     cap = (cap + 255) / 256 * 256;
@@ -309,24 +324,22 @@ rad_status ensure_capacity(rad_ctx* c, long long n, int n_chunks, long long fine
     js.perm = js.sort_counts = js.bucket_base = nullptr;
     js.gref = nullptr;
     // the record buffer, and the sort buffers of wide calls (12 B per particle)
-    rad_status s = cuda_check(c, dmalloc(&js.rec, (size_t)cap * kRecFields));
+    rad_status s = alloc_buffer(c, &js.rec, (size_t)cap * kRecFields);
     if (s == RAD_OK && js.wide_flag) {
-      s = cuda_check(c, dmalloc(&js.perm, (size_t)cap));
+      s = alloc_buffer(c, &js.perm, (size_t)cap);
       if (s == RAD_OK)
-        s = cuda_check(c, dmalloc(&js.sort_counts,
-                                  (size_t)((cap + kSortBlock - 1) / kSortBlock) * kSortBuckets));
-      if (s == RAD_OK) s = cuda_check(c, dmalloc(&js.bucket_base, (size_t)kSortBuckets));
-      if (s == RAD_OK) s = cuda_check(c, dmalloc(&js.gref, (size_t)3 * ((cap + kGroup - 1) / kGroup)));
+        s = alloc_buffer(c, &js.sort_counts, (size_t)((cap + kSortBlock - 1) / kSortBlock) * kSortBuckets);
+      if (s == RAD_OK) s = alloc_buffer(c, &js.bucket_base, (size_t)kSortBuckets);
+      if (s == RAD_OK) s = alloc_buffer(c, &js.gref, (size_t)3 * ((cap + kGroup - 1) / kGroup));
       // (a context that may take the low band, at any tile set later)
       if (s == RAD_OK && c->n_low > 0 && cap >= kLowMin)
-        s = cuda_check(c, dmalloc(&js.rec_s, (size_t)cap * kRecFields));
+        s = alloc_buffer(c, &js.rec_s, (size_t)cap * kRecFields);
     }
     if (s != RAD_OK) {
       js.n_cap = 0;
       return s;
     }
     js.n_cap = cap;
-    changed = true;
   }
   if (n_chunks > c->h_js.chunk_cap) {
     const int cap = std::max(n_chunks, c->h_js.chunk_cap * 3 / 2);
@@ -335,21 +348,20 @@ rad_status ensure_capacity(rad_ctx* c, long long n, int n_chunks, long long fine
       cudaFree(c->h_js.partials);
       c->h_js.partials = nullptr;
     }
-    rad_status s = cuda_check(c, dmalloc(&c->h_js.partials, (size_t)cap * kComps * c->n_bins));
+    rad_status s = alloc_buffer(c, &c->h_js.partials, (size_t)cap * kComps * c->n_bins);
     if (s != RAD_OK) {
       c->h_js.chunk_cap = 0;
       return s;
     }
     if (c->h_js.literal) {
       if (c->h_js.partials_p) cudaFree(c->h_js.partials_p);
-      s = cuda_check(c, dmalloc(&c->h_js.partials_p, (size_t)cap * 4 * c->n_bins));
+      s = alloc_buffer(c, &c->h_js.partials_p, (size_t)cap * 4 * c->n_bins);
       if (s != RAD_OK) {
         c->h_js.chunk_cap = 0;
         return s;
       }
     }
     c->h_js.chunk_cap = cap;
-    changed = true;
   }
   if (fine_floats > c->h_js.fine_cap) {
     const long long cap = std::max(fine_floats, c->h_js.fine_cap * 3 / 2);
@@ -358,13 +370,12 @@ rad_status ensure_capacity(rad_ctx* c, long long n, int n_chunks, long long fine
       cudaFree(c->h_js.partials_f);
       c->h_js.partials_f = nullptr;
     }
-    rad_status s = cuda_check(c, dmalloc(&c->h_js.partials_f, (size_t)cap));
+    rad_status s = alloc_buffer(c, &c->h_js.partials_f, (size_t)cap);
     if (s != RAD_OK) {
       c->h_js.fine_cap = 0;
       return s;
     }
     c->h_js.fine_cap = cap;
-    changed = true;
   }
   if (low_floats > c->h_js.low_cap) {
     const long long cap = std::max(low_floats, c->h_js.low_cap * 3 / 2);
@@ -373,15 +384,14 @@ rad_status ensure_capacity(rad_ctx* c, long long n, int n_chunks, long long fine
       cudaFree(c->h_js.partials_l);
       c->h_js.partials_l = nullptr;
     }
-    rad_status s = cuda_check(c, dmalloc(&c->h_js.partials_l, (size_t)cap));
+    rad_status s = alloc_buffer(c, &c->h_js.partials_l, (size_t)cap);
     if (s != RAD_OK) {
       c->h_js.low_cap = 0;
       return s;
     }
     c->h_js.low_cap = cap;
-    changed = true;
   }
-  return changed ? upload_static(c) : RAD_OK;
+  return c->js_stale ? upload_static(c) : RAD_OK;
 }
 
 CallPlan plan_call(const rad_ctx* c, const JobStatic& js, int variant, long long n) {

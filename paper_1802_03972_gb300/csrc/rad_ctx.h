@@ -56,6 +56,8 @@ struct rad_ctx {
   double low_full = 0.0;         // cost of the full tiling, in full tiles
   radimpl::LowSet low[radimpl::kLowSets]{};
   long long generation = 0;      // bumped whenever d_js changes
+  bool js_stale = false;         // h_js names buffers that d_js does not (yet)
+  int fail_alloc = 0;            // test support: the so-many-th buffer allocation from now fails
   uint64_t grid_hash = 0;        // FNV-1a of the frequencies and unit directions
   int device = -1;               // the CUDA device current at rad_create
   rad_status last_err = RAD_OK;

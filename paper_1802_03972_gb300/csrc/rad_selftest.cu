@@ -100,6 +100,12 @@ rad_status rad_selftest_wait(int64_t limit_ns, int32_t* timed_out, double* waite
   return RAD_OK;
 }
 
+rad_status rad_selftest_fail_alloc(rad_ctx* c, int32_t nth) {
+  if (!c || nth < 0) return RAD_EINVAL;
+  c->fail_alloc = nth;
+  return RAD_OK;
+}
+
 rad_status rad_selftest_stage1(rad_ctx* c, int64_t n, const double* r, const double* beta,
                                const double* beta_dot, const double* w, double t, double dt,
                                int32_t dir, float* out, float* basis) {

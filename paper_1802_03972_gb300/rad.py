@@ -37,7 +37,7 @@ EXPORTS = [
     "rad_probe_peaks", "rad_probe_tensor", "rad_probe_loop", "rad_profile_enable", "rad_profile_read", "rad_profile_clock", "rad_accumulate_static",
     "rad_static_status",
     "rad_spectrum_literal", "rad_push_step", "rad_push_flush",
-    "rad_selftest_wait", "rad_selftest_stage1", "rad_selftest_phase",
+    "rad_selftest_wait", "rad_selftest_stage1", "rad_selftest_phase", "rad_selftest_fail_alloc",
 ]
 FF_LITERAL = 2  # rad_ff.flags at creation: also accumulate the paper's literal sum
 # Round policies of the serving loop (rad_server_set_policy).
@@ -137,6 +137,7 @@ def load(path: str = LIB_PATH):
         "rad_selftest_wait": (st, [i64, ctypes.POINTER(i32), ctypes.POINTER(dbl)]),
         "rad_selftest_stage1": (st, [vp, i64, vp, vp, vp, vp, dbl, dbl, i32, vp, vp]),
         "rad_selftest_phase": (st, [vp, i32, vp, vp, vp, vp]),
+        "rad_selftest_fail_alloc": (st, [vp, i32]),
         "rad_accumulate_static": (st, [vp, i32, vp, i32, i64, vp, vp, vp, vp, dbl, dbl, vp, vp]),
         "rad_static_status": (st, [vp]),
         "rad_spectrum_literal": (st, [vp, vp]),
@@ -384,6 +385,10 @@ class Context:
                                              float(t), float(dt), int(direction), out.ctypes.data,
                                              basis.ctypes.data), "rad_selftest_stage1")
         return out, basis.reshape(2, 3)
+
+    def selftest_fail_alloc(self, nth: int) -> None:
+        """rad_selftest_fail_alloc: the nth next buffer allocation of this context's calls fails, once."""
+        _check(self._lib.rad_selftest_fail_alloc(self._h, int(nth)), "rad_selftest_fail_alloc")
 
     def selftest_phase(self, th, tl):
         """rad_selftest_phase: (fast, wide) phases in radians, [n_omega][len(th)]."""

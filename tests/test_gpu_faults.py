@@ -143,3 +143,28 @@ def test_bounded_wait_gives_up_and_the_context_keeps_working():
     gpu_run(wl, range(2, 4), ctx=ctx)
     ref = spectra_grid(oracle_run(wl, range(4)), wl)
     assert_parity(ctx.spectrum()[2], ref["tot"])
+
+
+@pytest.mark.parametrize("used_before", [False, True])
+@pytest.mark.parametrize("nth", range(1, 10))
+def test_a_call_after_one_that_ran_out_of_memory(nth, used_before):
+    """The nth buffer allocation of a large call fails; a smaller call, which may need no new buffer, then gives a fresh
+    context's results bit for bit, and so does the large call when it is made again."""
+    large = inputs.Workload("large", inputs.omega_log(1e14, 1e20, 512), inputs.dirs_grid(0.01, 8, 8),
+                            inputs.BetatronBunch(150000, seed=61), 4, 1e-16, inputs.FF_GAUSS, 0.1e-6)
+    small = inputs.Workload("small", large.omega, large.dirs, inputs.BetatronBunch(3000, seed=62), 4, 1e-16,
+                            inputs.FF_GAUSS, 0.1e-6)
+    ctx = rad.Context(large.omega, large.dirs, large.ff_kind, large.ff_width)
+    if used_before:
+        gpu_run(small, [0], ctx=ctx)
+    ctx.selftest_fail_alloc(nth)
+    try:
+        gpu_run(large, [0], ctx=ctx)
+    except rad.RadError as e:
+        assert e.status == rad.RAD_ENOMEM
+    ctx.selftest_fail_alloc(0)
+    for wl in (small, large, small):
+        ctx.reset()
+        gpu_run(wl, [1], ctx=ctx)
+        for x, y in zip(ctx.spectrum(), gpu_run(wl, [1]).spectrum()):
+            np.testing.assert_array_equal(x, y)
