@@ -1212,9 +1212,12 @@ __global__ void __launch_bounds__(THREADS, MINB) accumulate_kernel(const __grid_
     mbar_init(&bars_low[1], 1);
     mbar_fence_init();
   }
-  // A single job's tables do not depend on the kernels before this one.
-  if (a.n_jobs == 1) load_job<THREADS>(b, a, 0);
+  // A single job's tables, before the wait where no kernel writes them.  (The
+  // allocation-free entry's set-up kernel does: the pre-pass triggers before its own
+  // wait, so this kernel can be running before those writes are visible to it.)
+  if (a.n_jobs == 1 && !a.js_from_kernel) load_job<THREADS>(b, a, 0);
   pdl_wait();
+  if (a.n_jobs == 1 && a.js_from_kernel) load_job<THREADS>(b, a, 0);
   // Whether any job of the launch is wide is final by now; without, the first
   // pass takes every item without looking at the jobs' flags.
   if (a.n_jobs == 1) __syncthreads();
@@ -1298,7 +1301,7 @@ __global__ void __launch_bounds__(kRedThreads) reduce_kernel(const __grid_consta
   __shared__ float2 rot[kRedBins];
   pdl_trigger();
   if (a.n_jobs == 1) {
-    load_job<kRedThreads>(b, a, 0);
+    if (!a.js_from_kernel) load_job<kRedThreads>(b, a, 0);  // (as accumulate_kernel)
   } else {
     if (threadIdx.x < 32) {
       int n = 0;
@@ -1310,6 +1313,7 @@ __global__ void __launch_bounds__(kRedThreads) reduce_kernel(const __grid_consta
     load_job<kRedThreads>(b, a, b.job);
   }
   pdl_wait();
+  if (a.n_jobs == 1 && a.js_from_kernel) load_job<kRedThreads>(b, a, 0);
   __syncthreads();
   if (threadIdx.x == 0) settle_plan(b);
   __syncthreads();

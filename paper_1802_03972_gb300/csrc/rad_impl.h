@@ -312,6 +312,10 @@ struct LaunchArgs {
   const JobCall* jc;     // device [n_jobs] (unused when use_inline)
   int n_jobs;
   int use_inline;        // 1: single job, call passed by value below
+  // 1: js is written by a kernel of the same chain (the allocation-free entry's
+  // set-up), so it may be read only after pdl_wait; 0: by a copy that is complete
+  // before the chain's first kernel starts
+  int js_from_kernel;
   long long n_items;
   long long n_items_low; // low-band work items (0: none possible)
   // the counter block (kCounterWords), zero before the launch

@@ -203,6 +203,7 @@ extern "C" rad_status rad_accumulate_static(const double* omega, int32_t n_omega
   a.js = reinterpret_cast<const JobStatic*>(base + kOffJob);
   a.n_jobs = 1;
   a.use_inline = 1;
+  a.js_from_kernel = 1;
   a.n_items = (long long)js.n_tiles * n_chunks;
   a.item_counter = reinterpret_cast<unsigned long long*>(base + kOffCounter);
   JobCall& K = a.inline_call;

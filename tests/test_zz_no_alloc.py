@@ -157,3 +157,30 @@ def test_static_entry_rejects_sizes_beyond_its_limits():
     many = torch.ones(rad.STATIC_MAX_OMEGA + 1, dtype=torch.float64, device="cuda")
     with pytest.raises(rad.RadError):
         rad.accumulate_static(many, dirs_d, big[:3], big[:3], big[:3], w[:1], 0.0, 1e-16, state)
+
+
+def test_calls_on_alternating_grids_and_states_without_a_wait_between():
+    """Calls on two grids of different tilings, each with accumulators of its own, enqueued back to back on one stream:
+    every call's kernels use the job table that its own set-up kernel wrote, so each state equals, bit for bit, that of
+    the same calls made one by one."""
+    wls = [inputs.lwfa_bunch(n_particles=700, n_omega=40, n_side=3, seed=82),
+           inputs.lwfa_bunch(n_particles=3000, n_omega=300, n_side=5, seed=83)]
+    sets = [device_inputs(wl, range(4)) for wl in wls]
+
+    def zeros():
+        return [torch.zeros(16 * wl.omega.shape[0] * wl.dirs.shape[0], dtype=torch.float32, device="cuda") for wl in wls]
+    alone, mixed = zeros(), zeros()
+    for k, (om, dirs, data) in enumerate(sets):
+        for _ in range(5):
+            for dev, t, dt in data:
+                rad.accumulate_static(om, dirs, *dev, t, dt, alone[k])
+                torch.cuda.synchronize()
+    for _ in range(5):
+        for s in range(4):
+            for k, (om, dirs, data) in enumerate(sets):
+                dev, t, dt = data[s]
+                rad.accumulate_static(om, dirs, *dev, t, dt, mixed[k])
+    torch.cuda.synchronize()
+    assert rad.static_status() == rad.RAD_OK
+    for a, b in zip(alone, mixed):
+        assert torch.equal(a, b) and bool(torch.any(a != 0))
