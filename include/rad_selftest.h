@@ -56,6 +56,12 @@ rad_status rad_selftest_phase(rad_ctx* ctx, int32_t n_tau, const float* th, cons
  * Errors: RAD_EINVAL for a NULL context or nth < 0. */
 rad_status rad_selftest_fail_alloc(rad_ctx* ctx, int32_t nth);
 
+/* rad_selftest_memory - *bytes (host) = device bytes the context holds in its tables,
+ * accumulators, records, sort buffers and partial sums (not the copies of
+ * host arrays, in-situ steps or profiling counters).  Mixed-precision contexts only.
+ * Errors: RAD_EINVAL. */
+rad_status rad_selftest_memory(const rad_ctx* ctx, int64_t* bytes);
+
 #ifdef __cplusplus
 }
 #endif

@@ -156,7 +156,11 @@ __device__ __forceinline__ ItemRef decode_item(const JobStatic& J, const JobCall
 
 // Where an item's partial sums live: component comp of chunk ch at
 // base[ch * chunk_stride + comp * comp_stride + bin offset].  Coarse tiles:
-// J.partials [chunk][comp][n_bins], the offset the bin; fine tiles: their
+// J.partials [chunk][comp][bin], the bins those of the tiled frequencies (all, or
+// the ones above the low band: rows of n_omega - o_part per direction, so an
+// alternative with few tiles and many chunks needs no room for the band's bins:
+// a context of 4096 x 256 bins with 3e5 particles holds 0.81 GB instead of
+// 3.23); fine tiles: their
 // level's region of J.partials_f, [chunk][comp][level tiles][NT WT], level 1's
 // after level 0's, the offset the bin's index within the tile.  room: the
 // floats from the start of the item's buffer or region.
@@ -170,8 +174,8 @@ __device__ __forceinline__ PartMap part_map(const JobStatic& J, const JobCall& K
   PartMap m;
   if (it.fine < 0) {
     m.base = J.partials;
-    m.comp_stride = (size_t)J.n_bins;
-    m.room = (long long)J.chunk_cap * kComps * J.n_bins;
+    m.comp_stride = (size_t)J.n_dir * (J.n_omega - J.o_part);
+    m.room = J.part_cap;
   } else {
     const long long tb = (long long)g.NT * g.WT;
     const bool l1 = it.tile >= J.n_tiles - K.tail_tiles[1];
@@ -193,8 +197,7 @@ __device__ __forceinline__ void kahan_add(float* sum, float* cmp, float x) {
 
 // Whether an item's chunks fit the partial-sum buffer it writes.
 __device__ __forceinline__ bool part_fits(const JobStatic& J, const ItemRef& it, const PartMap& m) {
-  return it.fine < 0 ? it.n_chunks <= J.chunk_cap
-                     : m.room >= (long long)it.n_chunks * (long long)m.chunk_stride;
+  return m.room >= (long long)it.n_chunks * (long long)m.chunk_stride;
 }
 
 __device__ __forceinline__ float sqrt_approx(float x) {
@@ -441,7 +444,7 @@ __device__ __forceinline__ bool process_item_fma(const JobStatic& J, const JobCa
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           const int o = om_first + 2 * p + e;
-          if (o < n_om && bounds_ok(chunk < J.chunk_cap && si.it.fine < 0, J.status)) {
+          if (o < n_om && bounds_ok((chunk + 1) * (long long)(kComps * cs) <= J.part_cap && si.it.fine < 0, J.status)) {
 #pragma unroll
             for (int c = 0; c < kComps; ++c)
               part[(size_t)c * cs + off + 2 * p + e] = e ? acc2[p][c].y : acc2[p][c].x;
@@ -776,7 +779,7 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
       const PartMap pm = part_map(J, K, si.it, g);
       float* part = pm.base + (size_t)chunk * pm.chunk_stride;
       const size_t cs = pm.comp_stride;
-      const size_t off = si.it.fine < 0 ? (size_t)my_d * n_om + o_warp0
+      const size_t off = si.it.fine < 0 ? (size_t)my_d * (n_om - J.o_part) + (o_warp0 - J.o_part)
                                         : (size_t)my_dl * g.WT + (o_warp0 - g.o0);
       float* q = part + off + r + (size_t)(4 * c) * cs;
       const int left = n_om - o_warp0 - r;  // rows past the grid are not written
@@ -1092,6 +1095,7 @@ __device__ __forceinline__ void settle_plan(BlockState& b) {
   b.low = b.J.low[b.plan.set];
   const LowSet& L = b.low;
   const LowCall& C = b.K.low[b.plan.set];
+  b.J.o_part = L.js;
   b.J.n_tiles = L.n_tiles;
   b.J.n_seg = L.n_seg;
   for (int i = 0; i < kMaxSegs; ++i) b.J.seg[i] = L.seg[i];
@@ -1345,8 +1349,8 @@ __global__ void __launch_bounds__(kRedThreads) reduce_kernel(const __grid_consta
     const int i = s * kRedBins + 4 * q, ti = s * kRedBins + rt;
     d = g.d0 + (i >> sh), o = g.o0 + (i & (g.WT - 1));
     rd = g.d0 + (ti >> sh), ro = g.o0 + (ti & (g.WT - 1));
-    off = it.fine < 0 ? (size_t)d * n_om + o : (size_t)i;
-    part4 = it.fine >= 0 || om4;
+    off = it.fine < 0 ? (size_t)d * (n_om - J.o_part) + (o - J.o_part) : (size_t)i;
+    part4 = it.fine >= 0 || om4;  // (o_part is a multiple of 64)
   } else {
     // the low band's bins, direction by direction
     const long long f = (local - hi_blocks) * kRedBins;

@@ -311,7 +311,7 @@ rad_status upload_static(rad_ctx* c) {
   return s;
 }
 
-rad_status ensure_capacity(rad_ctx* c, long long n, int n_chunks, long long fine_floats, long long low_floats) {
+rad_status ensure_capacity(rad_ctx* c, long long n, long long part_floats, long long fine_floats, long long low_floats) {
   if (n > c->h_js.n_cap) {
     long long cap = std::max(n, c->h_js.n_cap * 3 / 2);
     cap = (cap + 255) / 256 * 256;
@@ -341,27 +341,27 @@ rad_status ensure_capacity(rad_ctx* c, long long n, int n_chunks, long long fine
     }
     js.n_cap = cap;
   }
-  if (n_chunks > c->h_js.chunk_cap) {
-    const int cap = std::max(n_chunks, c->h_js.chunk_cap * 3 / 2);
+  if (part_floats > c->h_js.part_cap) {
+    const long long cap = std::max(part_floats, c->h_js.part_cap * 3 / 2);
     if (c->h_js.partials) {
       cudaStreamSynchronize(c->stream);
       cudaFree(c->h_js.partials);
       c->h_js.partials = nullptr;
     }
-    rad_status s = alloc_buffer(c, &c->h_js.partials, (size_t)cap * kComps * c->n_bins);
+    rad_status s = alloc_buffer(c, &c->h_js.partials, (size_t)cap);
     if (s != RAD_OK) {
-      c->h_js.chunk_cap = 0;
+      c->h_js.part_cap = 0;
       return s;
     }
     if (c->h_js.literal) {
       if (c->h_js.partials_p) cudaFree(c->h_js.partials_p);
-      s = alloc_buffer(c, &c->h_js.partials_p, (size_t)cap * 4 * c->n_bins);
+      s = alloc_buffer(c, &c->h_js.partials_p, (size_t)cap / 2);
       if (s != RAD_OK) {
-        c->h_js.chunk_cap = 0;
+        c->h_js.part_cap = 0;
         return s;
       }
     }
-    c->h_js.chunk_cap = cap;
+    c->h_js.part_cap = cap;
   }
   if (fine_floats > c->h_js.fine_cap) {
     const long long cap = std::max(fine_floats, c->h_js.fine_cap * 3 / 2);
@@ -394,13 +394,28 @@ rad_status ensure_capacity(rad_ctx* c, long long n, int n_chunks, long long fine
   return c->js_stale ? upload_static(c) : RAD_OK;
 }
 
+size_t context_bytes(const rad_ctx* c, const JobStatic& js) {
+  const size_t nb = c->n_bins, n = (size_t)js.n_cap;
+  size_t b = 2 * sizeof(double) * c->n_omega + sizeof(float) * c->tab_floats +
+             (3 * sizeof(double) + kDirTab * sizeof(float)) * (size_t)c->n_dir + 4 * sizeof(double) +
+             kStatusWords * sizeof(int) + sizeof(c->low) + kCounterWords * sizeof(unsigned long long) +
+             sizeof(JobStatic) + (3 * sizeof(double) + 2 * kComps * sizeof(float)) * nb;
+  if (js.literal) b += 8 * sizeof(float) * nb + sizeof(float) * c->n_omega + sizeof(float) * (size_t)(js.part_cap / 2);
+  b += sizeof(float) * kRecFields * n;
+  if (n > 0)
+    b += sizeof(int) * (n + (n + kSortBlock - 1) / kSortBlock * kSortBuckets + kSortBuckets) +
+         3 * sizeof(double) * ((n + kGroup - 1) / kGroup);
+  if (js.rec_s) b += sizeof(float) * kRecFields * n;
+  return b + sizeof(float) * (size_t)(js.part_cap + js.fine_cap + js.low_cap);
+}
+
 CallPlan plan_call(const rad_ctx* c, const JobStatic& js, int variant, long long n) {
   CallPlan p;
   p.ck = auto_chunk(c, variant, n, js.n_tiles);
   p.n_chunks = (int)((n + p.ck - 1) / p.ck);
   p.tail = tail_plan(variant_tensor_core(variant) && !js.literal, n, js.n_tiles, p.ck, p.n_chunks,
                      resident_ctas(variant));
-  p.most_chunks = p.n_chunks;
+  p.part_floats = (long long)p.n_chunks * kComps * js.n_bins;
   p.fine_floats = p.tail.fine_floats(js.bpt);
   // The low band (automatic chunks, calls that are sorted when wide): per
   // alternative, the other bins' tiles chunked as a job of their own, and about
@@ -426,7 +441,7 @@ CallPlan plan_call(const rad_ctx* c, const JobStatic& js, int variant, long long
     C.max_cells = (int)std::min(0.75 * saved / piece, (double)kLowMaxCells);
     if (C.max_cells < 8) continue;
     p.low_ok |= 1u << s;
-    p.most_chunks = std::max(p.most_chunks, C.n_hi);
+    p.part_floats = std::max(p.part_floats, (long long)C.n_hi * kComps * js.n_dir * (js.n_omega - L.js));
     const TailPlan tail = tail_plan(true, n, L.n_tiles, C.ck_hi, C.n_hi, resident_ctas(variant));
     set_tail(C, tail);
     p.fine_floats = std::max(p.fine_floats, tail.fine_floats(js.bpt));
@@ -513,7 +528,7 @@ rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const do
   }
   const int variant = c->tile.variant;
   const CallPlan plan = plan_call(c, c->h_js, variant, n);
-  rad_status s = ensure_capacity(c, n, plan.most_chunks, plan.fine_floats, plan.low_floats);
+  rad_status s = ensure_capacity(c, n, plan.part_floats, plan.fine_floats, plan.low_floats);
   if (s != RAD_OK) return s;
   LaunchArgs a;
   memset(&a, 0, sizeof(a));
@@ -689,6 +704,7 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
   };
   chk(dmalloc(&c->d_omega, n_omega));
   chk(dmalloc(&c->d_om_turns, n_omega));
+  c->tab_floats = tab_floats;
   chk(dmalloc(&c->d_om_tab, tab_floats));
   chk(dmalloc(&c->d_dirs, nd.size()));
   chk(dmalloc(&c->d_dir_tab, dir_tab.size()));

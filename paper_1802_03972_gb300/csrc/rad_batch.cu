@@ -118,21 +118,19 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
       fill_tiles(js, variant, default_omega_tile(variant, c->n_omega), c->n_low);
     // chunked as the job alone would be (results equal bit for bit)
     const CallPlan call = plan_call(c, js, variant, steps[i].n);
-    const int nch = call.most_chunks;
-    const long long fine = call.fine_floats;
-    if (steps[i].n > c->h_js.n_cap || nch > c->h_js.chunk_cap || fine > c->h_js.fine_cap ||
-        call.low_floats > c->h_js.low_cap) {
+    if (steps[i].n > c->h_js.n_cap || call.part_floats > c->h_js.part_cap ||
+        call.fine_floats > c->h_js.fine_cap || call.low_floats > c->h_js.low_cap) {
       if (!drained) {
         if (cudaStreamSynchronize(work) != cudaSuccess) return RAD_ECUDA;
         drained = true;
       }
-      rad_status s = ensure_capacity(c, steps[i].n, nch, fine, call.low_floats);
+      rad_status s = ensure_capacity(c, steps[i].n, call.part_floats, call.fine_floats, call.low_floats);
       if (s != RAD_OK) return s;
       if (cudaStreamSynchronize(c->stream) != cudaSuccess) return RAD_ECUDA;
       js.rec = c->h_js.rec;
       js.n_cap = c->h_js.n_cap;
       js.partials = c->h_js.partials;
-      js.chunk_cap = c->h_js.chunk_cap;
+      js.part_cap = c->h_js.part_cap;
       js.partials_f = c->h_js.partials_f;
       js.fine_cap = c->h_js.fine_cap;
       js.perm = c->h_js.perm;

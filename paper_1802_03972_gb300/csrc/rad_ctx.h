@@ -56,6 +56,7 @@ struct rad_ctx {
   double low_full = 0.0;         // cost of the full tiling, in full tiles
   radimpl::LowSet low[radimpl::kLowSets]{};
   long long generation = 0;      // bumped whenever d_js changes
+  size_t tab_floats = 0;         // of d_om_tab: om_tab, then the low band's tables
   bool js_stale = false;         // h_js names buffers that d_js does not (yet)
   int fail_alloc = 0;            // test support: the so-many-th buffer allocation from now fails
   uint64_t grid_hash = 0;        // FNV-1a of the frequencies and unit directions
@@ -88,19 +89,22 @@ int resident_ctas(int variant);
 // fine_tail: the job's last tiles are fine-chunked (TailPlan), which allows longer items.
 int auto_chunk_for(int variant, long long n, int n_tiles, bool fine_tail);
 int auto_chunk(const rad_ctx* c, int variant, long long n, int n_tiles);
-// Capacity for n particles, n_chunks coarse chunks and fine_floats floats of
-// fine-tile partial sums (TailPlan::fine_floats).
-rad_status ensure_capacity(rad_ctx* c, long long n, int n_chunks, long long fine_floats = 0,
+// Device bytes of a MIXED context with these buffer capacities (js): its tables and
+// accumulators, and its calls' records, sort buffers and partial sums.
+size_t context_bytes(const rad_ctx* c, const JobStatic& js);
+// Capacity for n particles and for so many floats of the coarse tiles', the fine
+// tiles' (TailPlan::fine_floats) and the low band's partial sums.
+rad_status ensure_capacity(rad_ctx* c, long long n, long long part_floats, long long fine_floats = 0,
                            long long low_floats = 0);
 // How a call of n particles is cut into work items.
 struct CallPlan {
   int ck = 0, n_chunks = 0;
-  int most_chunks = 0;  // over the low band's alternatives too
   TailPlan tail;
   unsigned low_ok = 0;  // the alternatives that pay for this call (bits)
   LowCall low[kLowSets] = {};
-  long long hi_items = 0, low_items = 0, low_floats = 0;
-  long long fine_floats = 0;  // of partials_f
+  long long hi_items = 0, low_items = 0;
+  // of partials, partials_f and partials_l, the most over the alternatives
+  long long part_floats = 0, fine_floats = 0, low_floats = 0;
   // items of the bin tiles (run: chunks per item), the most over the alternatives
   long long items(const JobStatic& js, int run) const;
   void fill(JobCall& K, const JobStatic& js, int run) const;

@@ -164,7 +164,8 @@ struct JobStatic {
   int bpt, n_tiles, n_seg;
   TileSeg seg[kMaxSegs];
   float tau_fast;                 // |delta tau| bound of the fast phase path, s
-  int chunk_cap;                  // capacity of partials, in chunks
+  int o_part;                     // first frequency of partials' rows (0; a call that takes the low band: its js)
+  long long part_cap;             // capacity of partials, in floats
   long long n_cap;                // capacity of rec, in particles
   const float* om_tab;
   const double* om_turns;
@@ -172,7 +173,7 @@ struct JobStatic {
   const float* dir_tab;
   const double* dirs;
   float* state;
-  float* partials;                // [chunk_cap][kComps][n_bins]
+  float* partials;                // per call [n_chunks][kComps][n_dir][n_omega - o_part]
   // the fine-chunked last tiles of a call (see TailPlan): per level l,
   // [n_chunks_f[l]][kComps][tail_tiles[l]][nt * wt], level 1 after level 0;
   // fine_cap floats
@@ -186,7 +187,7 @@ struct JobStatic {
   int skip;                       // 1: the grid is invalid, every particle weighs zero
   const float* f2_tab;            // [n_omega] f(omega)^2 of the creation shape
   float* state_p;                 // [8][n_bins]: P.e1, P.e2 re/im sums, then compensations
-  float* partials_p;              // [chunk_cap][4][n_bins]
+  float* partials_p;              // [n_chunks][4][n_bins], in part_cap / 2 floats
   // wide calls (null wide_flag: never; the tiles of a spread call then take
   // the FP64 phase path)
   int* wide_flag;                 // per call: 1 if the call is wide (set by the pre-pass)

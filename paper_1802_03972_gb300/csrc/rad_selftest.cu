@@ -106,6 +106,12 @@ rad_status rad_selftest_fail_alloc(rad_ctx* c, int32_t nth) {
   return RAD_OK;
 }
 
+rad_status rad_selftest_memory(const rad_ctx* c, int64_t* bytes) {
+  if (!c || !bytes || c->prec != RAD_PREC_MIXED) return RAD_EINVAL;
+  *bytes = (int64_t)context_bytes(c, c->h_js);
+  return RAD_OK;
+}
+
 rad_status rad_selftest_stage1(rad_ctx* c, int64_t n, const double* r, const double* beta,
                                const double* beta_dot, const double* w, double t, double dt,
                                int32_t dir, float* out, float* basis) {
@@ -114,7 +120,7 @@ rad_status rad_selftest_stage1(rad_ctx* c, int64_t n, const double* r, const dou
   if (check_device(c) != RAD_OK) return RAD_EINVAL;
   if (c->prec != RAD_PREC_MIXED || n < 1 || n > (1 << 20) || dir < 0 || dir >= c->n_dir)
     return RAD_EINVAL;
-  rad_status s = ensure_capacity(c, n, 1);
+  rad_status s = ensure_capacity(c, n, (long long)kComps * c->n_bins);
   if (s != RAD_OK) return s;
   LaunchArgs a;
   memset(&a, 0, sizeof(a));

@@ -181,7 +181,7 @@ extern "C" rad_status rad_accumulate_static(const double* omega, int32_t n_omega
     ck = (int)((c2 + kChunkAlign - 1) / kChunkAlign * kChunkAlign);
     n_chunks = (int)((n + ck - 1) / ck);
   }
-  js.chunk_cap = max_chunks;
+  js.part_cap = (long long)kMaxChunks * kComps * RAD_STATIC_MAX_BINS;
   js.n_cap = RAD_STATIC_MAX_PARTICLES;
   js.om_tab = reinterpret_cast<const float*>(base + kOffOmTab);
   js.om_turns = reinterpret_cast<const double*>(base + kOffOmTurns);

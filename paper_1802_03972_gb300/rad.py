@@ -38,6 +38,7 @@ EXPORTS = [
     "rad_static_status",
     "rad_spectrum_literal", "rad_push_step", "rad_push_flush",
     "rad_selftest_wait", "rad_selftest_stage1", "rad_selftest_phase", "rad_selftest_fail_alloc",
+    "rad_selftest_memory",
 ]
 FF_LITERAL = 2  # rad_ff.flags at creation: also accumulate the paper's literal sum
 # Round policies of the serving loop (rad_server_set_policy).
@@ -138,6 +139,7 @@ def load(path: str = LIB_PATH):
         "rad_selftest_stage1": (st, [vp, i64, vp, vp, vp, vp, dbl, dbl, i32, vp, vp]),
         "rad_selftest_phase": (st, [vp, i32, vp, vp, vp, vp]),
         "rad_selftest_fail_alloc": (st, [vp, i32]),
+        "rad_selftest_memory": (st, [vp, ctypes.POINTER(i64)]),
         "rad_accumulate_static": (st, [vp, i32, vp, i32, i64, vp, vp, vp, vp, dbl, dbl, vp, vp]),
         "rad_static_status": (st, [vp]),
         "rad_spectrum_literal": (st, [vp, vp]),
@@ -389,6 +391,12 @@ class Context:
     def selftest_fail_alloc(self, nth: int) -> None:
         """rad_selftest_fail_alloc: the nth next buffer allocation of this context's calls fails, once."""
         _check(self._lib.rad_selftest_fail_alloc(self._h, int(nth)), "rad_selftest_fail_alloc")
+
+    def selftest_memory(self) -> int:
+        """rad_selftest_memory: device bytes of the context's tables, accumulators and call buffers."""
+        b = ctypes.c_int64()
+        _check(self._lib.rad_selftest_memory(self._h, ctypes.byref(b)), "rad_selftest_memory")
+        return b.value
 
     def selftest_phase(self, th, tl):
         """rad_selftest_phase: (fast, wide) phases in radians, [n_omega][len(th)]."""
