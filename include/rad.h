@@ -145,7 +145,10 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
  * on the device along the grid's mean direction and given one reference point
  * per 256 particles; its results are as deterministic as any other call's.
  * The context keeps ~92 bytes of device memory per macro-particle of the
- * largest call (records and sort buffers).
+ * largest call (records and sort buffers), the calls' partial sums and, for large
+ * calls on ascending grids that may take their lowest frequencies from nodes
+ * (the low band), another 80 bytes per macro-particle and the band's sums.  Where
+ * the band's buffers do not fit the device, calls go without it until rad_reset.
  * Errors: RAD_EINVAL, RAD_ENOMEM, RAD_ECUDA, RAD_ESTATE. */
 rad_status rad_accumulate(rad_ctx* ctx, int64_t n, const double* r, const double* beta,
                           const double* beta_dot, const double* w, double t, double dt);
@@ -200,7 +203,8 @@ rad_status rad_spectrum_species(rad_ctx* const* ctxs, const rad_ff* ffs, int32_t
 /* rad_sync - wait for the context's queued work; report RAD_EDATA / errors. */
 rad_status rad_sync(rad_ctx* ctx);
 
-/* rad_reset - zero the accumulators (keeps grids and buffers). */
+/* rad_reset - zero the accumulators (keeps grids and buffers).  Calls may take
+ * the low band again (rad_accumulate) where memory ran short for it before. */
 rad_status rad_reset(rad_ctx* ctx);
 
 /* rad_destroy - free everything (synchronises the stream first). NULL is ok. */

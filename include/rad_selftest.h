@@ -51,10 +51,11 @@ rad_status rad_selftest_phase(rad_ctx* ctx, int32_t n_tau, const float* th, cons
                               float* fast, float* wide);
 
 /* rad_selftest_fail_alloc - the nth (from 1) of the context's next device buffer
- * allocations for its calls' work (records, sort buffers, partial sums) fails as
- * cudaMalloc does without memory, once; 0: none.  Allocates nothing itself.
- * Errors: RAD_EINVAL for a NULL context or nth < 0. */
-rad_status rad_selftest_fail_alloc(rad_ctx* ctx, int32_t nth);
+ * allocations for its calls' work (records, sort buffers, partial sums), and the
+ * times - 1 after it, fail as cudaMalloc does without memory; nth = 0: none.
+ * Allocates nothing itself.  Errors: RAD_EINVAL for a NULL context, nth < 0 or
+ * times < 1. */
+rad_status rad_selftest_fail_alloc(rad_ctx* ctx, int32_t nth, int32_t times);
 
 /* rad_selftest_memory - *bytes (host) = device bytes the context holds in its tables,
  * accumulators, records, sort buffers and partial sums (not the copies of

@@ -888,7 +888,7 @@ __device__ __forceinline__ bool process_item_low(const JobStatic& J, const JobCa
 
   for (int t = lane; t < 12; t += 32) sdir[warp * 12 + t] = __ldg(J.dir_tab + (size_t)t * J.n_dir + my_d);
   auto issue = [&](const LowTile& t, int buf) {
-    if (!bounds_ok(t.pos + t.kn <= J.n_cap, J.status)) return;
+    if (!bounds_ok(t.pos + t.kn <= J.rec_s_cap, J.status)) return;
     tma_load_1d(raw + (size_t)buf * kLowTile * kRecFields, J.rec_s + (size_t)t.pos * kRecFields,
                 (uint32_t)t.kn * kRecFields * sizeof(float), &bars[buf]);
   };

@@ -76,7 +76,10 @@ template <class T>
 rad_status alloc_buffer(rad_ctx* c, T** p, size_t count) {
   c->js_stale = true;
   *p = nullptr;
-  if (c->fail_alloc > 0 && --c->fail_alloc == 0) return cuda_check(c, cudaErrorMemoryAllocation);
+  if (c->fail_alloc > 0 && --c->fail_alloc == 0) {
+    if (--c->fail_times > 0) c->fail_alloc = 1;
+    return cuda_check(c, cudaErrorMemoryAllocation);
+  }
   return cuda_check(c, dmalloc(p, count));
 }
 
@@ -317,10 +320,10 @@ rad_status ensure_capacity(rad_ctx* c, long long n, long long part_floats, long 
     cap = (cap + 255) / 256 * 256;
     JobStatic& js = c->h_js;
     if (js.rec) cudaStreamSynchronize(c->stream);
-    void* old[] = {js.rec, js.perm, js.sort_counts, js.bucket_base, js.gref, js.rec_s};
+    void* old[] = {js.rec, js.perm, js.sort_counts, js.bucket_base, js.gref};
     for (void* p : old)
       if (p) cudaFree(p);
-    js.rec = js.rec_s = nullptr;
+    js.rec = nullptr;
     js.perm = js.sort_counts = js.bucket_base = nullptr;
     js.gref = nullptr;
     // the record buffer, and the sort buffers of wide calls (12 B per particle)
@@ -331,9 +334,6 @@ rad_status ensure_capacity(rad_ctx* c, long long n, long long part_floats, long 
         s = alloc_buffer(c, &js.sort_counts, (size_t)((cap + kSortBlock - 1) / kSortBlock) * kSortBuckets);
       if (s == RAD_OK) s = alloc_buffer(c, &js.bucket_base, (size_t)kSortBuckets);
       if (s == RAD_OK) s = alloc_buffer(c, &js.gref, (size_t)3 * ((cap + kGroup - 1) / kGroup));
-      // (a context that may take the low band, at any tile set later)
-      if (s == RAD_OK && c->n_low > 0 && cap >= kLowMin)
-        s = alloc_buffer(c, &js.rec_s, (size_t)cap * kRecFields);
     }
     if (s != RAD_OK) {
       js.n_cap = 0;
@@ -377,6 +377,18 @@ rad_status ensure_capacity(rad_ctx* c, long long n, long long part_floats, long 
     }
     c->h_js.fine_cap = cap;
   }
+  if (low_floats > 0 && n > c->h_js.rec_s_cap) {
+    // records in cell order, for the calls that may take the low band
+    const long long cap = c->h_js.n_cap;
+    if (c->h_js.rec_s) {
+      cudaStreamSynchronize(c->stream);
+      cudaFree(c->h_js.rec_s);
+    }
+    c->h_js.rec_s_cap = 0;
+    rad_status s = alloc_buffer(c, &c->h_js.rec_s, (size_t)cap * kRecFields);
+    if (s != RAD_OK) return s;
+    c->h_js.rec_s_cap = cap;
+  }
   if (low_floats > c->h_js.low_cap) {
     const long long cap = std::max(low_floats, c->h_js.low_cap * 3 / 2);
     if (c->h_js.partials_l) {
@@ -405,7 +417,7 @@ size_t context_bytes(const rad_ctx* c, const JobStatic& js) {
   if (n > 0)
     b += sizeof(int) * (n + (n + kSortBlock - 1) / kSortBlock * kSortBuckets + kSortBuckets) +
          3 * sizeof(double) * ((n + kGroup - 1) / kGroup);
-  if (js.rec_s) b += sizeof(float) * kRecFields * n;
+  b += sizeof(float) * kRecFields * (size_t)js.rec_s_cap;
   return b + sizeof(float) * (size_t)(js.part_cap + js.fine_cap + js.low_cap);
 }
 
@@ -420,7 +432,7 @@ CallPlan plan_call(const rad_ctx* c, const JobStatic& js, int variant, long long
   // The low band (automatic chunks, calls that are sorted when wide): per
   // alternative, the other bins' tiles chunked as a job of their own, and about
   // kLowItemsPerCta items per resident block of the band.
-  if (js.n_low == 0 || c->tile.chunk != 0 || js.wide_flag == nullptr || n < kLowMin || n >= (1LL << 31))
+  if (js.n_low == 0 || c->low_nomem || c->tile.chunk != 0 || js.wide_flag == nullptr || n < kLowMin || n >= (1LL << 31))
     return p;
   const long long dirs8 = (js.n_dir + 7) / 8;
   for (int s = 0; s < js.n_low; ++s) {
@@ -450,6 +462,26 @@ CallPlan plan_call(const rad_ctx* c, const JobStatic& js, int variant, long long
     p.low_floats = std::max(p.low_floats, (long long)C.n_lo * kComps * js.n_dir * L.js);
   }
   return p;
+}
+
+rad_status reserve_call(rad_ctx* c, const JobStatic& js, int variant, long long n, CallPlan& plan) {
+  const rad_status last = c->last_err;
+  plan = plan_call(c, js, variant, n);
+  rad_status s = ensure_capacity(c, n, plan.part_floats, plan.fine_floats, plan.low_floats);
+  if (s != RAD_ENOMEM || plan.low_ok == 0) return s;
+  rad_log(1, "no device memory for the low band's buffers: bin tiles until the context is reset");
+  c->low_nomem = true;
+  JobStatic& h = c->h_js;
+  cudaStreamSynchronize(c->stream);
+  cudaFree(h.rec_s);
+  cudaFree(h.partials_l);
+  h.rec_s = h.partials_l = nullptr;
+  h.rec_s_cap = h.low_cap = 0;
+  c->js_stale = true;
+  plan = plan_call(c, js, variant, n);
+  s = ensure_capacity(c, n, plan.part_floats, plan.fine_floats, plan.low_floats);
+  if (s == RAD_OK) c->last_err = last;
+  return s;
 }
 
 long long CallPlan::items(const JobStatic& js, int run) const {
@@ -527,8 +559,8 @@ rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const do
                                      c->f64_chunks, c->h_js.status, c->stream));
   }
   const int variant = c->tile.variant;
-  const CallPlan plan = plan_call(c, c->h_js, variant, n);
-  rad_status s = ensure_capacity(c, n, plan.part_floats, plan.fine_floats, plan.low_floats);
+  CallPlan plan;
+  rad_status s = reserve_call(c, c->h_js, variant, n, plan);
   if (s != RAD_OK) return s;
   LaunchArgs a;
   memset(&a, 0, sizeof(a));
@@ -978,6 +1010,7 @@ rad_status rad_reset(rad_ctx* c) {
     if (s != RAD_OK) return s;
   }
   s = cuda_check(c, cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream));
+  c->low_nomem = false;
   if (s == RAD_OK) c->last_err = RAD_OK;
   return s;
 }

@@ -117,14 +117,15 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
     if (c->tile.variant != variant)
       fill_tiles(js, variant, default_omega_tile(variant, c->n_omega), c->n_low);
     // chunked as the job alone would be (results equal bit for bit)
-    const CallPlan call = plan_call(c, js, variant, steps[i].n);
+    CallPlan call = plan_call(c, js, variant, steps[i].n);
     if (steps[i].n > c->h_js.n_cap || call.part_floats > c->h_js.part_cap ||
-        call.fine_floats > c->h_js.fine_cap || call.low_floats > c->h_js.low_cap) {
+        call.fine_floats > c->h_js.fine_cap || call.low_floats > c->h_js.low_cap ||
+        (call.low_floats > 0 && steps[i].n > c->h_js.rec_s_cap)) {
       if (!drained) {
         if (cudaStreamSynchronize(work) != cudaSuccess) return RAD_ECUDA;
         drained = true;
       }
-      rad_status s = ensure_capacity(c, steps[i].n, call.part_floats, call.fine_floats, call.low_floats);
+      rad_status s = reserve_call(c, js, variant, steps[i].n, call);
       if (s != RAD_OK) return s;
       if (cudaStreamSynchronize(c->stream) != cudaSuccess) return RAD_ECUDA;
       js.rec = c->h_js.rec;
@@ -138,6 +139,7 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
       js.bucket_base = c->h_js.bucket_base;
       js.gref = c->h_js.gref;
       js.rec_s = c->h_js.rec_s;
+      js.rec_s_cap = c->h_js.rec_s_cap;
       js.partials_l = c->h_js.partials_l;
       js.low_cap = c->h_js.low_cap;
     }

@@ -57,8 +57,12 @@ struct rad_ctx {
   radimpl::LowSet low[radimpl::kLowSets]{};
   long long generation = 0;      // bumped whenever d_js changes
   size_t tab_floats = 0;         // of d_om_tab: om_tab, then the low band's tables
+  // Some call's low-band buffers did not fit the device: calls take the bin tiles, as
+  // they do without the band, until rad_reset.
+  bool low_nomem = false;
   bool js_stale = false;         // h_js names buffers that d_js does not (yet)
-  int fail_alloc = 0;            // test support: the so-many-th buffer allocation from now fails
+  int fail_alloc = 0;            // test support: the so-many-th buffer allocation from now fails ...
+  int fail_times = 0;            // ... and this many in all
   uint64_t grid_hash = 0;        // FNV-1a of the frequencies and unit directions
   int device = -1;               // the CUDA device current at rad_create
   rad_status last_err = RAD_OK;
@@ -110,6 +114,9 @@ struct CallPlan {
   void fill(JobCall& K, const JobStatic& js, int run) const;
 };
 CallPlan plan_call(const rad_ctx* c, const JobStatic& js, int variant, long long n);
+// Plans a call and makes room for it.  The low band is taken only where its buffers
+// fit: without memory for them the call is planned again without it.
+rad_status reserve_call(rad_ctx* c, const JobStatic& js, int variant, long long n, CallPlan& plan);
 rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const double* beta,
                               const double* bdot, const double* w, double t, double dt);
 rad_status upload_static(rad_ctx* c);

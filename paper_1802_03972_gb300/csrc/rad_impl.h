@@ -205,7 +205,8 @@ struct JobStatic {
   float cone1, cone2;             // largest |n . fr1|, |n . fr2| of the grid
   int* ext;                       // [6] a call's smallest / largest coordinate along fr1, fr2, axis (ordered ints)
   LowPlan* plan;
-  float* rec_s;                   // [n_cap][20] records in cell order
+  float* rec_s;                   // [rec_s_cap][20] records in cell order
+  long long rec_s_cap;
   float* partials_l;              // low_cap floats: the low bands' chunk sums, [chunk][8][n_dir][js]
   long long low_cap;
 };

@@ -100,9 +100,10 @@ rad_status rad_selftest_wait(int64_t limit_ns, int32_t* timed_out, double* waite
   return RAD_OK;
 }
 
-rad_status rad_selftest_fail_alloc(rad_ctx* c, int32_t nth) {
-  if (!c || nth < 0) return RAD_EINVAL;
+rad_status rad_selftest_fail_alloc(rad_ctx* c, int32_t nth, int32_t times) {
+  if (!c || nth < 0 || times < 1) return RAD_EINVAL;
   c->fail_alloc = nth;
+  c->fail_times = times;
   return RAD_OK;
 }
 

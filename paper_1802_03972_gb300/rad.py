@@ -138,7 +138,7 @@ def load(path: str = LIB_PATH):
         "rad_selftest_wait": (st, [i64, ctypes.POINTER(i32), ctypes.POINTER(dbl)]),
         "rad_selftest_stage1": (st, [vp, i64, vp, vp, vp, vp, dbl, dbl, i32, vp, vp]),
         "rad_selftest_phase": (st, [vp, i32, vp, vp, vp, vp]),
-        "rad_selftest_fail_alloc": (st, [vp, i32]),
+        "rad_selftest_fail_alloc": (st, [vp, i32, i32]),
         "rad_selftest_memory": (st, [vp, ctypes.POINTER(i64)]),
         "rad_accumulate_static": (st, [vp, i32, vp, i32, i64, vp, vp, vp, vp, dbl, dbl, vp, vp]),
         "rad_static_status": (st, [vp]),
@@ -388,9 +388,9 @@ class Context:
                                              basis.ctypes.data), "rad_selftest_stage1")
         return out, basis.reshape(2, 3)
 
-    def selftest_fail_alloc(self, nth: int) -> None:
-        """rad_selftest_fail_alloc: the nth next buffer allocation of this context's calls fails, once."""
-        _check(self._lib.rad_selftest_fail_alloc(self._h, int(nth)), "rad_selftest_fail_alloc")
+    def selftest_fail_alloc(self, nth: int, times: int = 1) -> None:
+        """rad_selftest_fail_alloc: the nth next buffer allocation of this context's calls and the times - 1 after it fail."""
+        _check(self._lib.rad_selftest_fail_alloc(self._h, int(nth), int(times)), "rad_selftest_fail_alloc")
 
     def selftest_memory(self) -> int:
         """rad_selftest_memory: device bytes of the context's tables, accumulators and call buffers."""

@@ -168,3 +168,60 @@ def test_a_call_after_one_that_ran_out_of_memory(nth, used_before):
         gpu_run(wl, [1], ctx=ctx)
         for x, y in zip(ctx.spectrum(), gpu_run(wl, [1]).spectrum()):
             np.testing.assert_array_equal(x, y)
+
+
+def band_workload(n, seed=61):
+    return inputs.Workload("band", inputs.omega_log(1e14, 1e20, 512), inputs.dirs_grid(0.01, 8, 8),
+                           inputs.BetatronBunch(n, seed=seed), 4, 1e-16, inputs.FF_GAUSS, 0.1e-6)
+
+
+@pytest.mark.parametrize("batched", [False, True])
+@pytest.mark.parametrize("nth", range(1, 10))
+def test_a_call_whose_low_band_does_not_fit_takes_the_bin_tiles(nth, batched):
+    """The nth buffer allocation of a call that could take the low band fails: the call runs without the band, as it does
+    on a grid that has none (the frequencies listed the other way round), and reports nothing."""
+    wl = band_workload(150000)
+    down = band_workload(150000)
+    down.omega = wl.omega[::-1].copy()
+    want = [s[:, ::-1] for s in gpu_run(down, range(2)).spectrum()]
+    ctx = rad.Context(wl.omega, wl.dirs, wl.ff_kind, wl.ff_width)
+    other = rad.Context(wl.omega[:64], wl.dirs, wl.ff_kind, wl.ff_width)
+    batch, keep = rad.Batch([other, ctx]) if batched else None, []
+    ctx.selftest_fail_alloc(nth)
+    for s in range(2):
+        st = wl.step(s)
+        keep.append([to_dev(a) for a in (st.r, st.beta, st.beta_dot, st.w)])
+        if batched:
+            batch.accumulate([rad.make_step(0, *keep[-1], st.t, st.dt), rad.make_step(st.n, *keep[-1], st.t, st.dt)])
+        else:
+            ctx.accumulate(*keep[-1], st.t, st.dt)
+    if batched:
+        batch.sync()
+    for x, y in zip(ctx.spectrum(), want):  # (the same sums; the frequencies sit in other lanes and tiles)
+        np.testing.assert_allclose(np.linalg.norm(x - y, axis=1), 0.0, atol=2e-6 * np.linalg.norm(y, axis=1).max())
+    ctx.reset()
+    gpu_run(wl, range(2), ctx=ctx)
+    for x, y in zip(ctx.spectrum(), gpu_run(wl, range(2)).spectrum()):  # (with the band again)
+        np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("nth", range(1, 10))
+def test_a_call_after_one_that_stayed_out_of_memory(nth):
+    """No memory for the bin tiles either: the call is refused, and a smaller one afterwards runs on the buffers it has."""
+    large, small = band_workload(150000), band_workload(3000, seed=62)
+    ctx = rad.Context(large.omega, large.dirs, large.ff_kind, large.ff_width)
+    gpu_run(small, [0], ctx=ctx)
+    ctx.selftest_fail_alloc(nth, 100)
+    refused = False
+    try:
+        gpu_run(large, [0], ctx=ctx)
+    except rad.RadError as e:
+        refused = e.status == rad.RAD_ENOMEM
+    # the ninth buffer of this call is the band's, and so is the eighth: the tiles have theirs
+    assert refused == (nth <= 7)
+    ctx.selftest_fail_alloc(0)
+    for wl in (small, large):
+        ctx.reset()
+        gpu_run(wl, [1], ctx=ctx)
+        for x, y in zip(ctx.spectrum(), gpu_run(wl, [1]).spectrum()):
+            np.testing.assert_array_equal(x, y)
