@@ -312,7 +312,9 @@ typedef struct {
 } rad_server_stats;
 
 /* hbm_budget: device bytes the admitted jobs may hold in total; max_slots:
- * jobs admitted at once. */
+ * jobs admitted at once.  A job's bytes are counted from its grids, max_particles
+ * and max_queued at submission, and its buffers grow no further; one that fits the
+ * budget only without the low band (rad_accumulate) runs without it. */
 rad_status rad_server_create(size_t hbm_budget, int32_t max_slots, void* stream,
                              rad_server** out);
 /* Round policy of the scheduler.  Each round runs one pending step from each

@@ -63,6 +63,12 @@ rad_status rad_selftest_fail_alloc(rad_ctx* ctx, int32_t nth, int32_t times);
  * Errors: RAD_EINVAL. */
 rad_status rad_selftest_memory(const rad_ctx* ctx, int64_t* bytes);
 
+/* rad_selftest_limit - holds the context, as the server does a job's, to calls of at
+ * most max_particles: its buffers then grow no further than those calls need.
+ * *bytes (host) = rad_selftest_memory's figure when they have.  For contexts with
+ * the default tile.  Errors: RAD_EINVAL. */
+rad_status rad_selftest_limit(rad_ctx* ctx, int64_t max_particles, int64_t* bytes);
+
 #ifdef __cplusplus
 }
 #endif

@@ -278,8 +278,7 @@ int resident_ctas(int variant) {
 // Chunks below kChunkAlign only while one wave holds them.  Depends only on the
 // job's shape, n and the device, so a job is chunked the same way alone and in a
 // batch.
-int auto_chunk_for(int variant, long long n, int n_tiles, bool fine_tail) {
-  const long long resident = resident_ctas(variant);
+static int chunk_for(long long resident, long long n, int n_tiles, bool fine_tail) {
   const long long target = (long long)(fine_tail ? kItemsPerCta : kItemsPerCtaUniform) * resident;
   long long chunks = (target + n_tiles - 1) / n_tiles;
   const long long max_chunks = (n + kChunkAlign - 1) / kChunkAlign;
@@ -301,6 +300,10 @@ int auto_chunk_for(int variant, long long n, int n_tiles, bool fine_tail) {
   return (int)best;
 }
 
+int auto_chunk_for(int variant, long long n, int n_tiles, bool fine_tail) {
+  return chunk_for(resident_ctas(variant), n, n_tiles, fine_tail);
+}
+
 int auto_chunk(const rad_ctx* c, int variant, long long n, int n_tiles) {
   if (c->tile.chunk > 0) return c->tile.chunk;
   return auto_chunk_for(variant, n, n_tiles, variant_tensor_core(variant) && !c->h_js.literal);
@@ -314,9 +317,27 @@ rad_status upload_static(rad_ctx* c) {
   return s;
 }
 
+// Cells that a call of n particles may have in an alternative of the low band, its
+// particles in n_lo chunks.  What it saves, in particles of a tile: the bins' tiles
+// against the nodes and an interpolation per direction and piece of a cell.  The
+// cells' number is the device's: it may use three quarters of what is saved.
+constexpr int kLowCellsMin = 8;  // fewer: not taken
+static int low_cells(const rad_ctx* c, const LowSet& L, long long n, long long dirs8, int n_lo, long long resident) {
+  const double piece = (double)dirs8 * (64 + L.js);
+  const double saved = (c->low_full - L.hi_cost) * (double)n - (double)dirs8 * kLowCost * (double)n -
+                       n_lo * piece - kLowFixed * resident;
+  return (int)std::min(0.75 * saved / piece, (double)kLowMaxCells);
+}
+
+// Capacity for `need`, half as much again as there was when it grows, within the limit (0: none).
+static long long grown(long long need, long long have, long long limit) {
+  const long long cap = std::max(need, have * 3 / 2);
+  return limit > 0 ? std::max(need, std::min(cap, limit)) : cap;
+}
+
 rad_status ensure_capacity(rad_ctx* c, long long n, long long part_floats, long long fine_floats, long long low_floats) {
   if (n > c->h_js.n_cap) {
-    long long cap = std::max(n, c->h_js.n_cap * 3 / 2);
+    long long cap = grown(n, c->h_js.n_cap, c->limit.n);
     cap = (cap + 255) / 256 * 256;
     JobStatic& js = c->h_js;
     if (js.rec) cudaStreamSynchronize(c->stream);
@@ -342,7 +363,7 @@ rad_status ensure_capacity(rad_ctx* c, long long n, long long part_floats, long 
     js.n_cap = cap;
   }
   if (part_floats > c->h_js.part_cap) {
-    const long long cap = std::max(part_floats, c->h_js.part_cap * 3 / 2);
+    const long long cap = grown(part_floats, c->h_js.part_cap, c->limit.part);
     if (c->h_js.partials) {
       cudaStreamSynchronize(c->stream);
       cudaFree(c->h_js.partials);
@@ -364,7 +385,7 @@ rad_status ensure_capacity(rad_ctx* c, long long n, long long part_floats, long 
     c->h_js.part_cap = cap;
   }
   if (fine_floats > c->h_js.fine_cap) {
-    const long long cap = std::max(fine_floats, c->h_js.fine_cap * 3 / 2);
+    const long long cap = grown(fine_floats, c->h_js.fine_cap, c->limit.fine);
     if (c->h_js.partials_f) {
       cudaStreamSynchronize(c->stream);
       cudaFree(c->h_js.partials_f);
@@ -390,7 +411,7 @@ rad_status ensure_capacity(rad_ctx* c, long long n, long long part_floats, long 
     c->h_js.rec_s_cap = cap;
   }
   if (low_floats > c->h_js.low_cap) {
-    const long long cap = std::max(low_floats, c->h_js.low_cap * 3 / 2);
+    const long long cap = grown(low_floats, c->h_js.low_cap, c->limit.low);
     if (c->h_js.partials_l) {
       cudaStreamSynchronize(c->stream);
       cudaFree(c->h_js.partials_l);
@@ -421,6 +442,57 @@ size_t context_bytes(const rad_ctx* c, const JobStatic& js) {
   return b + sizeof(float) * (size_t)(js.part_cap + js.fine_cap + js.low_cap);
 }
 
+CallLimits call_limits(const rad_ctx* c, long long n, bool band) {
+  const JobStatic& js = c->h_js;
+  const long long R = resident_ctas(kDefaultVariant);
+  CallLimits lim;
+  lim.n = (n + kGroup - 1) / kGroup * kGroup;
+  // A tiling's chunks over all sizes up to n: the chunk rule is a function of
+  // ceil(n / 128) (of ceil(n / 32) up to one group) until every chunk has kMinChunk
+  // particles, so those sizes are gone through; past them a tile has at most T
+  // chunks and the fine-chunked tail (TailPlan) at most 4 R + 8 T and R + 32 T
+  // (tile, chunk) pairs in its two levels.
+  auto tiling = [&](int n_tiles, long long bins, long long from) {
+    const long long T = ((long long)kItemsPerCta * R + n_tiles - 1) / n_tiles;
+    long long chunks = 0;
+    for (long long m = from;; m += m < kGroup ? kTinyChunk : kSmallestChunk) {
+      const long long k = std::min(m, n);
+      const int ck = chunk_for(R, k, n_tiles, true);
+      const int nc = (int)((k + ck - 1) / ck);
+      chunks = std::max<long long>(chunks, nc);
+      lim.fine = std::max(lim.fine, tail_plan(true, k, n_tiles, ck, nc, R).fine_floats(js.bpt));
+      if (m >= n) break;
+      if (m > kMinChunk * T) {
+        const long long most = std::max(T, (n >> 30) + 1);
+        chunks = std::max(chunks, most);
+        if (n_tiles >= 4) lim.fine = std::max(lim.fine, (5 * R + 40 * most) * kComps * js.bpt);
+        break;
+      }
+    }
+    lim.part = std::max(lim.part, chunks * kComps * bins);
+  };
+  tiling(js.n_tiles, js.n_bins, kTinyChunk);
+  const long long dirs8 = (js.n_dir + 7) / 8;
+  for (int s = 0; band && n >= kLowMin && s < c->n_low; ++s) {
+    const LowSet& L = c->low[s];
+    if (low_cells(c, L, std::min(n, (1LL << 31) - 1), dirs8, 1, R) < kLowCellsMin) continue;  // at no size up to n
+    tiling(L.n_tiles, (long long)js.n_dir * (js.n_omega - L.js), kLowMin);
+    const long long n_lo = std::min((long long)kLowItemsPerCta * R / dirs8 + 1, (n + kLowChunkMin - 1) / kLowChunkMin);
+    lim.low = std::max(lim.low, n_lo * kComps * js.n_dir * L.js);
+  }
+  return lim;
+}
+
+size_t context_bytes_at(const rad_ctx* c, const CallLimits& limits) {
+  JobStatic js = c->h_js;
+  js.n_cap = limits.n;
+  js.part_cap = limits.part;
+  js.fine_cap = limits.fine;
+  js.low_cap = limits.low;
+  js.rec_s_cap = limits.low > 0 ? limits.n : 0;
+  return context_bytes(c, js);
+}
+
 CallPlan plan_call(const rad_ctx* c, const JobStatic& js, int variant, long long n) {
   CallPlan p;
   p.ck = auto_chunk(c, variant, n, js.n_tiles);
@@ -444,14 +516,8 @@ CallPlan plan_call(const rad_ctx* c, const JobStatic& js, int variant, long long
     ck = std::max<long long>(kLowChunkMin, std::min<long long>(ck, 1LL << 30) / kChunkAlign * kChunkAlign);
     C.ck_lo = (int)ck;
     C.n_lo = (int)((n + ck - 1) / ck);
-    // What it saves, in particles of a tile: the bins' tiles against the nodes and
-    // an interpolation per direction and piece of a cell.  The cells' number is
-    // the device's: it may use three quarters of what is saved.
-    const double piece = (double)dirs8 * (64 + L.js);
-    const double saved = (c->low_full - L.hi_cost) * (double)n - (double)dirs8 * kLowCost * (double)n -
-                         C.n_lo * piece - kLowFixed * resident_ctas(variant);
-    C.max_cells = (int)std::min(0.75 * saved / piece, (double)kLowMaxCells);
-    if (C.max_cells < 8) continue;
+    C.max_cells = low_cells(c, L, n, dirs8, C.n_lo, resident_ctas(variant));
+    if (C.max_cells < kLowCellsMin) continue;
     p.low_ok |= 1u << s;
     p.part_floats = std::max(p.part_floats, (long long)C.n_hi * kComps * js.n_dir * (js.n_omega - L.js));
     const TailPlan tail = tail_plan(true, n, L.n_tiles, C.ck_hi, C.n_hi, resident_ctas(variant));
@@ -495,6 +561,24 @@ void CallPlan::fill(JobCall& K, const JobStatic& js, int run) const {
   set_tail(K, tail);
   K.low_ok = low_ok;
   for (int s = 0; low_ok && s < js.n_low; ++s) K.low[s] = low[s];
+}
+
+void plan_grid(rad_ctx* c, const double* omega, int n_omega, int n_dir, int prec, bool literal) {
+  c->n_omega = n_omega;
+  c->n_dir = n_dir;
+  c->n_bins = n_omega * n_dir;
+  c->prec = prec;
+  c->tile.variant = literal ? kLiteralVariant : kDefaultVariant;
+  c->tile.omega_tile = default_omega_tile(c->tile.variant, n_omega);
+  c->tile.chunk = 0;
+  JobStatic& js = c->h_js;
+  memset(&js, 0, sizeof(js));
+  js.n_omega = n_omega;
+  js.n_dir = n_dir;
+  js.n_bins = c->n_bins;
+  c->tab_floats = (size_t)kOmTab * n_omega;
+  if (prec == RAD_PREC_MIXED && !literal) c->n_low = low_alternatives(js, omega, c->tab_floats, c->low, &c->low_full);
+  fill_tiles(js, c->tile.variant, c->tile.omega_tile, c->n_low);
 }
 
 // Host copy of the amplitude form factor of Table 1 (f(0) = 1), for the
@@ -669,15 +753,9 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
     c->grid_hash = h;
     c->device = current_device();
   }
-  c->n_omega = n_omega;
-  c->n_dir = n_dir;
-  c->n_bins = n_omega * n_dir;
+  plan_grid(c, omega, n_omega, n_dir, prec, literal);
   c->ff = ff;
-  c->prec = prec;
   c->stream = (cudaStream_t)stream;
-  c->tile.variant = kDefaultVariant;
-  c->tile.omega_tile = default_omega_tile(kDefaultVariant, n_omega);
-  c->tile.chunk = 0;
 
   // Frequency table: omega/2pi split hi/lo; (hi, 2pi hi, 2pi lo) floats.
   std::vector<float> om_tab((size_t)kOmTab * n_omega);
@@ -718,16 +796,9 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
   }
 
   JobStatic& js = c->h_js;
-  memset(&js, 0, sizeof(js));
-  js.n_omega = n_omega;
-  js.n_dir = n_dir;
-  js.n_bins = c->n_bins;
   js.tau_fast = (float)(2097152.0 / std::max(om_hi_max, 1e-300));  // 2^21 turns
   wide_geometry(nd.data(), n_dir, js.tau_fast, js.axis, &js.cone_sin, &js.bucket_w);
   low_geometry(nd.data(), n_dir, js);
-  size_t tab_floats = om_tab.size();
-  if (prec == RAD_PREC_MIXED && !literal) c->n_low = low_alternatives(js, omega, tab_floats, c->low, &c->low_full);
-  fill_tiles(js, c->tile.variant, c->tile.omega_tile, c->n_low);
 
   rad_status s = RAD_OK;
   size_t f64_words = 0;  // doubles of an FP64 context's allocation
@@ -736,8 +807,7 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
   };
   chk(dmalloc(&c->d_omega, n_omega));
   chk(dmalloc(&c->d_om_turns, n_omega));
-  c->tab_floats = tab_floats;
-  chk(dmalloc(&c->d_om_tab, tab_floats));
+  chk(dmalloc(&c->d_om_tab, c->tab_floats));
   chk(dmalloc(&c->d_dirs, nd.size()));
   chk(dmalloc(&c->d_dir_tab, dir_tab.size()));
   chk(dmalloc(&c->d_ref, 4));
@@ -811,11 +881,6 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
   js.state_p = c->d_state_p;
   // the wide flag lives in the counter block, zero between calls
   js.wide_flag = c->d_counter ? reinterpret_cast<int*>(c->d_counter + 2) : nullptr;
-  if (literal) {
-    c->tile.variant = kLiteralVariant;
-    c->tile.omega_tile = default_omega_tile(kLiteralVariant, n_omega);
-    fill_tiles(js, c->tile.variant, c->tile.omega_tile, 0);
-  }
   if (s == RAD_OK) chk(cudaMemcpy(c->d_js, &js, sizeof(JobStatic), cudaMemcpyHostToDevice));
   if (s == RAD_OK && c->n_low > 0) chk(launch_low_tables(js, c->n_low, c->stream));
   if (s != RAD_OK) {

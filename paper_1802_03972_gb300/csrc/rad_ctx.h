@@ -10,6 +10,14 @@
 #include "rad.h"
 #include "rad_impl.h"
 
+namespace radimpl {
+// The most that calls of up to n particles need: floats of partials, partials_f and
+// partials_l (low 0: no call may take the low band).
+struct CallLimits {
+  long long n = 0, part = 0, fine = 0, low = 0;
+};
+}  // namespace radimpl
+
 struct rad_ctx {
   int n_omega = 0, n_dir = 0, n_bins = 0;
   rad_ff ff{};
@@ -61,6 +69,7 @@ struct rad_ctx {
   // they do without the band, until rad_reset.
   bool low_nomem = false;
   bool js_stale = false;         // h_js names buffers that d_js does not (yet)
+  radimpl::CallLimits limit;     // n > 0: calls have at most so many particles, and their buffers stay within this
   int fail_alloc = 0;            // test support: the so-many-th buffer allocation from now fails ...
   int fail_times = 0;            // ... and this many in all
   uint64_t grid_hash = 0;        // FNV-1a of the frequencies and unit directions
@@ -114,6 +123,12 @@ struct CallPlan {
   void fill(JobCall& K, const JobStatic& js, int run) const;
 };
 CallPlan plan_call(const rad_ctx* c, const JobStatic& js, int variant, long long n);
+// Sizes, default tile, low-band alternatives and tiles of a context of this grid (host only).
+void plan_grid(rad_ctx* c, const double* omega, int n_omega, int n_dir, int prec, bool literal);
+// With the default tile (band: with the low band, where the grid has alternatives).
+CallLimits call_limits(const rad_ctx* c, long long n, bool band);
+// Bytes of the context when its buffers have grown to the limits.
+size_t context_bytes_at(const rad_ctx* c, const CallLimits& limits);
 // Plans a call and makes room for it.  The low band is taken only where its buffers
 // fit: without memory for them the call is planned again without it.
 rad_status reserve_call(rad_ctx* c, const JobStatic& js, int variant, long long n, CallPlan& plan);

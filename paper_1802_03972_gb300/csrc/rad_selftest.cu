@@ -113,6 +113,13 @@ rad_status rad_selftest_memory(const rad_ctx* c, int64_t* bytes) {
   return RAD_OK;
 }
 
+rad_status rad_selftest_limit(rad_ctx* c, int64_t max_particles, int64_t* bytes) {
+  if (!c || !bytes || c->prec != RAD_PREC_MIXED || max_particles < 1) return RAD_EINVAL;
+  c->limit = call_limits(c, max_particles, true);
+  *bytes = (int64_t)context_bytes_at(c, c->limit);
+  return RAD_OK;
+}
+
 rad_status rad_selftest_stage1(rad_ctx* c, int64_t n, const double* r, const double* beta,
                                const double* beta_dot, const double* w, double t, double dt,
                                int32_t dir, float* out, float* basis) {

@@ -59,6 +59,8 @@ struct Job {
   long long max_particles = 0;
   int max_queued = 1;
   size_t footprint = 0;
+  CallLimits limit;
+  bool band = true;  // its calls may take the low band
   JobState state = JobState::Waiting;
   rad_ctx* ctx = nullptr;
   std::vector<Slot> slots;
@@ -71,40 +73,19 @@ struct Job {
   Clock::time_point t_submit, t_ready;
 };
 
-size_t estimate_footprint(const rad_job_desc& d) {
-  const size_t nb = (size_t)d.n_omega * d.n_dir;
-  // Per-chunk partial sums (32 B per bin and chunk).  Automatic chunking aims
-  // at kItemsPerCta work items per resident block with the fine-chunked tail
-  // and kItemsPerCtaUniform (the larger) without it; with B bins per tile,
-  // chunks x bins <= kItemsPerCtaUniform x resident blocks x B + bins.  There
-  // are also never more chunks than 256-particle groups, except for a small
-  // call's, which fit one wave: chunks x bins <= resident blocks x B.
-  const Variant v = variant_info(kDefaultVariant);
-  const size_t bins_per_tile = (size_t)v.threads * v.w * v.passes;
-  const size_t by_particles =
-      std::max(nb * (size_t)((d.max_particles + kChunkAlign - 1) / kChunkAlign),
-               (size_t)resident_ctas(kDefaultVariant) * bins_per_tile);
-  const size_t by_items = (size_t)kItemsPerCtaUniform * resident_ctas(kDefaultVariant) * bins_per_tile + nb;
-  const size_t partials = 32 * std::min(by_particles, by_items);
-  // The fine-chunked last tiles' partial sums (TailPlan), 32 B per tile bin
-  // and (tile, chunk).  Level 0: L0 <= grid / n_c + 2 tiles of n_0 <= 4 n_c
-  // chunks, L0 n_0 <= 4 grid + 8 n_c; level 1: L1 <= grid / n_1 + 2 tiles of
-  // n_1 <= 4 n_0 <= 16 n_c chunks, L1 n_1 <= grid + 32 n_c.  Together at most
-  // 6 grid + 40 n_c (tile, chunk) pairs, with a few to spare.
-  const size_t grid = (size_t)resident_ctas(kDefaultVariant);
-  const size_t tiles_per_nb = std::max<size_t>(1, nb / bins_per_tile);
-  const size_t fine = 32 * bins_per_tile * (6 * grid + 12) + 40 * partials / tiles_per_nb;
-  // The low band's chunk sums (kLowItemsPerCta items per block, or chunks of
-  // kLowChunkMin, of 8 directions x up to n_omega bins) and its sorted records.
-  const size_t low = d.max_particles < kLowMin ? 0
-                         : 32 * 8 * (size_t)d.n_omega *
-                                   ((size_t)kLowItemsPerCta * grid + (size_t)(d.n_dir + 7) / 8) +
-                               80 * (size_t)d.max_particles;
-  // Records (80 B per particle), the sort buffers of wide calls (13 B) and the
-  // queued steps' staging slots (80 B each).
-  return nb * (64 + 24) + partials + fine + low +
-         (size_t)d.max_particles * (80 + 13 + 80 * (size_t)d.max_queued) +
-         (size_t)d.n_omega * 48 + (size_t)d.n_dir * 72 + (1 << 16) + 4 * (size_t)kSortBuckets;
+// Device bytes a job may come to hold: its context with the buffers of calls of up to
+// max_particles (the context is held to them, rad_ctx::limit) and the queued
+// steps' staging slots (80 B per particle each).  A job that fits the budget only
+// without the low band's buffers goes without it.
+void set_footprint(Job& j, const rad_job_desc& d, size_t budget) {
+  rad_ctx c;
+  plan_grid(&c, d.omega, d.n_omega, d.n_dir, RAD_PREC_MIXED, false);
+  for (const bool band : {true, false}) {
+    j.band = band;
+    j.limit = call_limits(&c, d.max_particles, band);
+    j.footprint = context_bytes_at(&c, j.limit) + (size_t)d.max_particles * 80 * (size_t)d.max_queued;
+    if (j.footprint <= budget || j.limit.low == 0) return;
+  }
 }
 
 }  // namespace
@@ -144,6 +125,8 @@ rad_status rad_server::admit_locked(Job& j) {
                             (int32_t)(j.dirs.size() / 3), j.ff, RAD_PREC_MIXED, compute, &c);
   if (s != RAD_OK) return s;
   j.ctx = c;
+  if (!j.band) c->n_low = c->h_js.n_low = 0;
+  c->limit = j.limit;
   j.slots.resize(j.max_queued);
   for (auto& sl : j.slots) {
     if (cudaMalloc(&sl.d, sizeof(double) * 10 * (size_t)j.max_particles) != cudaSuccess ||
@@ -399,7 +382,7 @@ rad_status rad_job_submit(rad_server* s, const rad_job_desc* d, rad_job_id* id) 
   j->ff = d->ff;
   j->max_particles = d->max_particles;
   j->max_queued = d->max_queued;
-  j->footprint = estimate_footprint(*d);
+  set_footprint(*j, *d, s->budget);
   if (j->footprint > s->budget) return RAD_EINVAL;
   j->t_submit = Clock::now();
   std::lock_guard<std::mutex> lk(s->mu);

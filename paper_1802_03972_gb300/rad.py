@@ -38,7 +38,7 @@ EXPORTS = [
     "rad_static_status",
     "rad_spectrum_literal", "rad_push_step", "rad_push_flush",
     "rad_selftest_wait", "rad_selftest_stage1", "rad_selftest_phase", "rad_selftest_fail_alloc",
-    "rad_selftest_memory",
+    "rad_selftest_memory", "rad_selftest_limit",
 ]
 FF_LITERAL = 2  # rad_ff.flags at creation: also accumulate the paper's literal sum
 # Round policies of the serving loop (rad_server_set_policy).
@@ -140,6 +140,7 @@ def load(path: str = LIB_PATH):
         "rad_selftest_phase": (st, [vp, i32, vp, vp, vp, vp]),
         "rad_selftest_fail_alloc": (st, [vp, i32, i32]),
         "rad_selftest_memory": (st, [vp, ctypes.POINTER(i64)]),
+        "rad_selftest_limit": (st, [vp, i64, ctypes.POINTER(i64)]),
         "rad_accumulate_static": (st, [vp, i32, vp, i32, i64, vp, vp, vp, vp, dbl, dbl, vp, vp]),
         "rad_static_status": (st, [vp]),
         "rad_spectrum_literal": (st, [vp, vp]),
@@ -396,6 +397,12 @@ class Context:
         """rad_selftest_memory: device bytes of the context's tables, accumulators and call buffers."""
         b = ctypes.c_int64()
         _check(self._lib.rad_selftest_memory(self._h, ctypes.byref(b)), "rad_selftest_memory")
+        return b.value
+
+    def selftest_limit(self, max_particles: int) -> int:
+        """rad_selftest_limit: the bytes this context may hold with calls of up to max_particles, and holds it to them."""
+        b = ctypes.c_int64()
+        _check(self._lib.rad_selftest_limit(self._h, int(max_particles), ctypes.byref(b)), "rad_selftest_limit")
         return b.value
 
     def selftest_phase(self, th, tl):
