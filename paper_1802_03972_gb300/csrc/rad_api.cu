@@ -530,6 +530,11 @@ CallPlan plan_call(const rad_ctx* c, const JobStatic& js, int variant, long long
   return p;
 }
 
+double evaluated_share(const rad_ctx* c, int set) {
+  if (set < 0 || set >= c->n_low) return 1.0;
+  return (c->low[set].hi_cost + kLowCost * ((c->n_dir + 7) / 8)) / c->low_full;
+}
+
 rad_status reserve_call(rad_ctx* c, const JobStatic& js, int variant, long long n, CallPlan& plan) {
   const rad_status last = c->last_err;
   plan = plan_call(c, js, variant, n);

@@ -129,6 +129,9 @@ void plan_grid(rad_ctx* c, const double* omega, int n_omega, int n_dir, int prec
 CallLimits call_limits(const rad_ctx* c, long long n, bool band);
 // Bytes of the context when its buffers have grown to the limits.
 size_t context_bytes_at(const rad_ctx* c, const CallLimits& limits);
+// A call's evaluated updates as a share of its particles x bins when it takes
+// alternative `set` of the low band (-1: none): tiles and nodes against all tiles.
+double evaluated_share(const rad_ctx* c, int set);
 // Plans a call and makes room for it.  The low band is taken only where its buffers
 // fit: without memory for them the call is planned again without it.
 rad_status reserve_call(rad_ctx* c, const JobStatic& js, int variant, long long n, CallPlan& plan);

@@ -68,6 +68,7 @@ struct Job {
   bool finished = false;
   bool in_round = false;
   long long served = 0;  // amplitude updates done
+  double share = 1.0;    // of its last step's updates that were evaluated (low band: fewer)
   rad_status err = RAD_OK;
   std::vector<double> coh, inc, tot;
   Clock::time_point t_submit, t_ready;
@@ -88,6 +89,11 @@ void set_footprint(Job& j, const rad_job_desc& d, size_t budget) {
   }
 }
 
+// The work of a job's next step, in evaluated updates, as its last step's were.
+long long step_work(const Job& j) {
+  return (long long)(j.share * (double)(j.queue.front().n * (long long)j.ctx->n_bins));
+}
+
 }  // namespace
 
 struct rad_server {
@@ -98,6 +104,7 @@ struct rad_server {
   cudaStream_t copy = nullptr;
   bool own_compute = false;
   BatchCore core;
+  int* h_sets = nullptr;  // pinned [max_slots]: the low-band alternative each step of a round took
   std::mutex mu;
   std::condition_variable cv_sched, cv_done;
   std::thread worker;
@@ -205,15 +212,16 @@ void rad_server::loop() {
     // Oldest job with bounded backfill: the oldest ready job always gets its
     // step, and other jobs (least served first) join only while the round's
     // work stays within max(round_updates, 17/16 of the head's step).  The head
-    // of the queue then runs at >= 16/17 of its own pace, as under FIFO, which
-    // keeps the tail latency of a FIFO queue, while small jobs progress in the
-    // margin instead of waiting behind large ones.
+    // of the queue then runs at >= 16/17 of its own pace, while small jobs progress
+    // in the margin instead of waiting behind large ones.  Work counts evaluated
+    // updates: a step that takes its lowest frequencies from nodes costs about half
+    // its particles x bins, and a margin counted in those slowed it by an eighth.
     const bool backfill = policy == RAD_SERVE_OLDEST_BACKFILL;
     long long budget = round_updates;
     if (backfill && !ready.empty()) {
       std::stable_sort(ready.begin() + 1, ready.end(),
                        [](const Job* a, const Job* b) { return a->served < b->served; });
-      const long long head = ready[0]->queue.front().n * (long long)ready[0]->ctx->n_bins;
+      const long long head = step_work(*ready[0]);
       budget = std::max(round_updates, head + head / 16);
     }
     if (policy == RAD_SERVE_LEAST_SERVED_AGED) {
@@ -239,7 +247,7 @@ void rad_server::loop() {
     for (Job* jp : ready) {
       Job& j = *jp;
       QueuedStep& q = j.queue.front();
-      const long long work = q.n * (long long)j.ctx->n_bins;
+      const long long work = backfill ? step_work(j) : q.n * (long long)j.ctx->n_bins;
       if (backfill) {
         if (!in_round.empty() && round_work + work > budget) continue;
       } else if (policy != RAD_SERVE_ALL && !in_round.empty() && round_work >= round_updates) {
@@ -278,6 +286,13 @@ void rad_server::loop() {
     if (!ctxs.empty()) {
       TraceRange trace("rad_server round");
       rs = core.run(ctxs.data(), steps.data(), (int)ctxs.size(), false);
+      for (size_t i = 0; i < ctxs.size() && rs == RAD_OK; ++i) {
+        h_sets[i] = -1;
+        const bool may = plan_call(ctxs[i], ctxs[i]->h_js, kDefaultVariant, steps[i].n).low_ok != 0;
+        if (may && cudaMemcpyAsync(&h_sets[i], &ctxs[i]->h_js.plan->set, sizeof(int), cudaMemcpyDeviceToHost,
+                                   compute) != cudaSuccess)
+          rs = RAD_ECUDA;
+      }
       if (rs == RAD_OK && cudaStreamSynchronize(compute) != cudaSuccess) rs = RAD_ECUDA;
     }
     for (Job* j : to_read) {
@@ -302,6 +317,7 @@ void rad_server::loop() {
         } else {
           st.updates += steps[i].n * (long long)j.ctx->n_bins;
           j.served += steps[i].n * (long long)j.ctx->n_bins;
+          j.share = evaluated_share(j.ctx, h_sets[i]);
         }
       }
       if (rs == RAD_ECUDA) fatal = RAD_ECUDA;
@@ -345,6 +361,7 @@ rad_status rad_server_create(size_t hbm_budget, int32_t max_slots, void* stream,
     return RAD_ECUDA;
   }
   rad_status st = s->core.init(max_slots, s->compute);
+  if (st == RAD_OK && cudaMallocHost(&s->h_sets, sizeof(int) * (size_t)max_slots) != cudaSuccess) st = RAD_ENOMEM;
   if (st != RAD_OK) {
     s->core.release();
     cudaStreamDestroy(s->copy);
@@ -538,6 +555,7 @@ void rad_server_destroy(rad_server* s) {
     s->jobs.clear();
   }
   s->core.release();
+  cudaFreeHost(s->h_sets);
   cudaStreamDestroy(s->copy);
   if (s->own_compute) cudaStreamDestroy(s->compute);
   delete s;

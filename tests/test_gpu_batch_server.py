@@ -257,3 +257,29 @@ def test_rad_log_reports_decisions_and_job_events():
     err = p.stderr
     assert "[rad] tune: 64 omega x 4 directions" in err, err[-2000:]
     assert "admitted" in err and "done after" in err, err[-2000:]
+
+
+def test_backfill_margin_counts_evaluated_updates():
+    """The oldest job takes its lowest frequencies from nodes (about 0.6 of its particles x bins are evaluated); a second
+    job's step is worth less than a sixteenth of those, and more than a sixteenth of the evaluated ones, so once the
+    server has seen a step of the first it runs the two in rounds of their own."""
+    omega, dirs = inputs.omega_log(1e14, 1e20, 512), inputs.dirs_grid(0.01, 16, 16)
+    n_large, n_small, n_steps = 100000, 4900, 24
+    large, small = (inputs.Workload("serve", omega, dirs, inputs.BetatronBunch(n, seed=61), n_steps, 1e-16,
+                                    inputs.FF_GAUSS, 0.1e-6) for n in (n_large, n_small))
+    arrs = [dev_steps(wl, 0)[1] for wl in (large, small)]
+    srv = rad.Server(hbm_budget=8 << 30, max_slots=2)
+    srv.set_policy(rad.SERVE_OLDEST_BACKFILL, 1)
+    ids = [srv.submit(omega, dirs, inputs.FF_GAUSS, 0.1e-6, max_particles=wl.n_particles, max_queued=n_steps)
+           for wl in (large, small)]
+    while srv.stats()["active"] < 2:
+        time.sleep(0.001)
+    for j, wl in enumerate((large, small)):
+        for s in range(n_steps):
+            assert srv.feed(ids[j], rad.make_step(wl.n_particles, *arrs[j], s * 1e-16, 1e-16)) == rad.RAD_OK
+        srv.finish(ids[j])
+    for j in ids:
+        srv.result(j, 256, 512, timeout=60)
+    rounds = srv.stats()["rounds"]
+    srv.close()
+    assert rounds >= 2 * n_steps - 3, rounds
