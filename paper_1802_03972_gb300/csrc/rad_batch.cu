@@ -184,7 +184,7 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
   const long long per_item = total / ((long long)kBatchItemsPerCta * resident_ctas(variant));
   auto run_of = [&](const Plan& q) {
     if (q.call.tail.tiles() > 0) return 1;
-    return (int)std::max<long long>(1, std::min<long long>(per_item, 1LL << 30) / q.call.ck);
+    return chunk_run(per_item, q.call.ck);
   };
 
   // Per-call table in the next pinned slot.

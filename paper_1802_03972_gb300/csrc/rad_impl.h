@@ -69,6 +69,17 @@ constexpr int kItemCost = 45;
 // 1.85e12 updates/s with 5, 1.94 with 8, 1.98 with 12, 2.04 with 20; 64 jobs of
 // 1e3-1e4 particles 1.23, 1.26, 1.27, 1.27).
 constexpr int kBatchItemsPerCta = 20;
+// ... of at most kMaxRun particles: next to a large job per_item (the particles of a
+// work item that give those many) is long, and a small job's whole tile in one item,
+// the launch's last, kept a few blocks busy after all others.  22632 particles,
+// 1024 x 1024 bins take 8.66 ms; with 15163 particles, 128 x 16 bins, that take 0.06 ms
+// alone, 0.46 ms more without the limit, 0.31 with 4096, 0.16 with 2048, 0.07 with
+// 1024.  64 jobs of up to 1e6 particles: 1.97e12 updates/s without, 2.06 with each.
+constexpr int kMaxRun = 1024;
+inline int chunk_run(long long per_item, int ck) {
+  const long long run = (per_item < kMaxRun ? per_item : kMaxRun) / ck;
+  return run > 1 ? (int)run : 1;
+}
 
 // Wide calls (particles farther than half the fast phase range from the
 // call's reference point): a stable bucket sort along the grid's mean
