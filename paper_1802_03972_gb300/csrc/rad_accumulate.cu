@@ -157,7 +157,7 @@ __device__ __forceinline__ ItemRef decode_item(const JobStatic& J, const JobCall
 // Where an item's partial sums live: component comp of chunk ch at
 // base[ch * chunk_stride + comp * comp_stride + bin offset].  Coarse tiles:
 // J.partials [chunk][comp][bin], the bins those of the tiled frequencies (all, or
-// the ones above the low band: rows of n_omega - o_part per direction, so an
+// the ones above the low band: rows of part_row per direction, so an
 // alternative with few tiles and many chunks needs no room for the band's bins:
 // a context of 4096 x 256 bins with 3e5 particles holds 0.81 GB instead of
 // 3.23); fine tiles: their
@@ -174,7 +174,7 @@ __device__ __forceinline__ PartMap part_map(const JobStatic& J, const JobCall& K
   PartMap m;
   if (it.fine < 0) {
     m.base = J.partials;
-    m.comp_stride = (size_t)J.n_dir * (J.n_omega - J.o_part);
+    m.comp_stride = (size_t)J.part_bins;
     m.room = J.part_cap;
   } else {
     const long long tb = (long long)g.NT * g.WT;
@@ -779,7 +779,7 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
       const PartMap pm = part_map(J, K, si.it, g);
       float* part = pm.base + (size_t)chunk * pm.chunk_stride;
       const size_t cs = pm.comp_stride;
-      const size_t off = si.it.fine < 0 ? (size_t)my_d * (n_om - J.o_part) + (o_warp0 - J.o_part)
+      const size_t off = si.it.fine < 0 ? (size_t)my_d * J.part_row + o_warp0
                                         : (size_t)my_dl * g.WT + (o_warp0 - g.o0);
       float* q = part + off + r + (size_t)(4 * c) * cs;
       const int left = n_om - o_warp0 - r;  // rows past the grid are not written
@@ -1095,7 +1095,10 @@ __device__ __forceinline__ void settle_plan(BlockState& b) {
   b.low = b.J.low[b.plan.set];
   const LowSet& L = b.low;
   const LowCall& C = b.K.low[b.plan.set];
-  b.J.o_part = L.js;
+  // (rows without the band's bins; a frequency keeps its index)
+  b.J.partials -= L.js;
+  b.J.part_row -= L.js;
+  b.J.part_bins -= b.J.n_dir * L.js;
   b.J.n_tiles = L.n_tiles;
   b.J.n_seg = L.n_seg;
   for (int i = 0; i < kMaxSegs; ++i) b.J.seg[i] = L.seg[i];
@@ -1218,10 +1221,11 @@ __global__ void __launch_bounds__(THREADS, MINB) accumulate_kernel(const __grid_
   }
   // A single job's tables, before the wait where no kernel writes them.  (The
   // allocation-free entry's set-up kernel does: the pre-pass triggers before its own
-  // wait, so this kernel can be running before those writes are visible to it.)
-  if (a.n_jobs == 1 && !a.js_from_kernel) load_job<THREADS>(b, a, 0);
+  // wait, so this kernel can be running before those writes are visible to it.  That
+  // entry runs an FP32 variant: the others need no test.)
+  if (a.n_jobs == 1 && (TC || a.use_inline != kJsFromKernel)) load_job<THREADS>(b, a, 0);
   pdl_wait();
-  if (a.n_jobs == 1 && a.js_from_kernel) load_job<THREADS>(b, a, 0);
+  if (!TC && a.use_inline == kJsFromKernel) load_job<THREADS>(b, a, 0);
   // Whether any job of the launch is wide is final by now; without, the first
   // pass takes every item without looking at the jobs' flags.
   if (a.n_jobs == 1) __syncthreads();
@@ -1299,13 +1303,15 @@ __device__ __forceinline__ float4 load_quad(const float* p, bool vec, int live) 
   return v;
 }
 
+// LATE: the job table comes from a kernel (kJsFromKernel).
+template <bool LATE>
 __global__ void __launch_bounds__(kRedThreads) reduce_kernel(const __grid_constant__ LaunchArgs a) {
   __shared__ __align__(8) BlockState b;
   __shared__ float4 part[kRedGroups - 1][2][kRedBins];
   __shared__ float2 rot[kRedBins];
   pdl_trigger();
   if (a.n_jobs == 1) {
-    if (!a.js_from_kernel) load_job<kRedThreads>(b, a, 0);  // (as accumulate_kernel)
+    if (!LATE) load_job<kRedThreads>(b, a, 0);  // (as accumulate_kernel)
   } else {
     if (threadIdx.x < 32) {
       int n = 0;
@@ -1317,7 +1323,7 @@ __global__ void __launch_bounds__(kRedThreads) reduce_kernel(const __grid_consta
     load_job<kRedThreads>(b, a, b.job);
   }
   pdl_wait();
-  if (a.n_jobs == 1 && a.js_from_kernel) load_job<kRedThreads>(b, a, 0);
+  if (LATE) load_job<kRedThreads>(b, a, 0);
   __syncthreads();
   if (threadIdx.x == 0) settle_plan(b);
   __syncthreads();
@@ -1349,8 +1355,8 @@ __global__ void __launch_bounds__(kRedThreads) reduce_kernel(const __grid_consta
     const int i = s * kRedBins + 4 * q, ti = s * kRedBins + rt;
     d = g.d0 + (i >> sh), o = g.o0 + (i & (g.WT - 1));
     rd = g.d0 + (ti >> sh), ro = g.o0 + (ti & (g.WT - 1));
-    off = it.fine < 0 ? (size_t)d * (n_om - J.o_part) + (o - J.o_part) : (size_t)i;
-    part4 = it.fine >= 0 || om4;  // (o_part is a multiple of 64)
+    off = it.fine < 0 ? (size_t)d * J.part_row + o : (size_t)i;
+    part4 = it.fine >= 0 || om4;  // (js is a multiple of 64)
   } else {
     // the low band's bins, direction by direction
     const long long f = (local - hi_blocks) * kRedBins;
@@ -1484,7 +1490,7 @@ int reduce_blocks(const JobStatic& js, const LowSet* low_sets) {
 
 cudaError_t launch_reduce(const LaunchArgs& a, long long blocks, cudaStream_t s) {
   count_launches(1);
-  return launch_pdl(reduce_kernel, blocks, kRedThreads, 0, s, a);
+  return launch_pdl(a.use_inline == kJsFromKernel ? reduce_kernel<true> : reduce_kernel<false>, blocks, kRedThreads, 0, s, a);
 }
 
 // Variants (rad_impl.h: variant_info): 0 FP32 256x2, 1 FP32 256x4, 2 FP32 128x2,

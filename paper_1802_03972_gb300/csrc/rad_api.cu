@@ -537,7 +537,6 @@ double evaluated_share(const rad_ctx* c, int set) {
 
 rad_status reserve_call(rad_ctx* c, const JobStatic& js, int variant, long long n, CallPlan& plan) {
   const rad_status last = c->last_err;
-  plan = plan_call(c, js, variant, n);
   rad_status s = ensure_capacity(c, n, plan.part_floats, plan.fine_floats, plan.low_floats);
   if (s != RAD_ENOMEM || plan.low_ok == 0) return s;
   rad_log(1, "no device memory for the low band's buffers: bin tiles until the context is reset");
@@ -580,7 +579,8 @@ void plan_grid(rad_ctx* c, const double* omega, int n_omega, int n_dir, int prec
   memset(&js, 0, sizeof(js));
   js.n_omega = n_omega;
   js.n_dir = n_dir;
-  js.n_bins = c->n_bins;
+  js.n_bins = js.part_bins = c->n_bins;
+  js.part_row = n_omega;
   c->tab_floats = (size_t)kOmTab * n_omega;
   if (prec == RAD_PREC_MIXED && !literal) c->n_low = low_alternatives(js, omega, c->tab_floats, c->low, &c->low_full);
   fill_tiles(js, c->tile.variant, c->tile.omega_tile, c->n_low);
@@ -648,7 +648,7 @@ rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const do
                                      c->f64_chunks, c->h_js.status, c->stream));
   }
   const int variant = c->tile.variant;
-  CallPlan plan;
+  CallPlan plan = plan_call(c, c->h_js, variant, n);
   rad_status s = reserve_call(c, c->h_js, variant, n, plan);
   if (s != RAD_OK) return s;
   LaunchArgs a;

@@ -114,7 +114,7 @@ struct CallPlan {
   int ck = 0, n_chunks = 0;
   TailPlan tail;
   unsigned low_ok = 0;  // the alternatives that pay for this call (bits)
-  LowCall low[kLowSets] = {};
+  LowCall low[kLowSets];  // (of those)
   long long hi_items = 0, low_items = 0;
   // of partials, partials_f and partials_l, the most over the alternatives
   long long part_floats = 0, fine_floats = 0, low_floats = 0;
@@ -132,8 +132,8 @@ size_t context_bytes_at(const rad_ctx* c, const CallLimits& limits);
 // A call's evaluated updates as a share of its particles x bins when it takes
 // alternative `set` of the low band (-1: none): tiles and nodes against all tiles.
 double evaluated_share(const rad_ctx* c, int set);
-// Plans a call and makes room for it.  The low band is taken only where its buffers
-// fit: without memory for them the call is planned again without it.
+// Makes room for a planned call.  The low band is taken only where its buffers fit:
+// without memory for them the call is planned again without it.
 rad_status reserve_call(rad_ctx* c, const JobStatic& js, int variant, long long n, CallPlan& plan);
 rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const double* beta,
                               const double* bdot, const double* w, double t, double dt);

@@ -175,8 +175,7 @@ struct JobStatic {
   int bpt, n_tiles, n_seg;
   TileSeg seg[kMaxSegs];
   float tau_fast;                 // |delta tau| bound of the fast phase path, s
-  int o_part;                     // first frequency of partials' rows (0; a call that takes the low band: its js)
-  long long part_cap;             // capacity of partials, in floats
+  int part_row;                   // partials' row: n_omega (a call that takes the low band: less its js)
   long long n_cap;                // capacity of rec, in particles
   const float* om_tab;
   const double* om_turns;
@@ -184,7 +183,7 @@ struct JobStatic {
   const float* dir_tab;
   const double* dirs;
   float* state;
-  float* partials;                // per call [n_chunks][kComps][n_dir][n_omega - o_part]
+  float* partials;                // per call [n_chunks][kComps][n_dir][part_row]
   // the fine-chunked last tiles of a call (see TailPlan): per level l,
   // [n_chunks_f[l]][kComps][tail_tiles[l]][nt * wt], level 1 after level 0;
   // fine_cap floats
@@ -217,9 +216,13 @@ struct JobStatic {
   int* ext;                       // [6] a call's smallest / largest coordinate along fr1, fr2, axis (ordered ints)
   LowPlan* plan;
   float* rec_s;                   // [rec_s_cap][20] records in cell order
-  long long rec_s_cap;
   float* partials_l;              // low_cap floats: the low bands' chunk sums, [chunk][8][n_dir][js]
   long long low_cap;
+  // (last: what a kernel reads first lies in few lines; in the middle these cost a
+  // step of 64 particles 0.2 of 14.5 us)
+  long long rec_s_cap;
+  long long part_cap;             // capacity of partials, in floats
+  int part_bins;                  // partials' component stride: part_row x n_dir
 };
 
 // Per-call data of one job.
@@ -320,15 +323,16 @@ inline void set_tail(Call& K, const TailPlan& t) {
   }
 }
 
+constexpr int kJsFromKernel = 2;
 struct LaunchArgs {
   const JobStatic* js;   // device [n_jobs]
   const JobCall* jc;     // device [n_jobs] (unused when use_inline)
   int n_jobs;
-  int use_inline;        // 1: single job, call passed by value below
-  // 1: js is written by a kernel of the same chain (the allocation-free entry's
-  // set-up), so it may be read only after pdl_wait; 0: by a copy that is complete
-  // before the chain's first kernel starts
-  int js_from_kernel;
+  // 1: single job, call passed by value below; 2 (kJsFromKernel): and js is written by
+  // a kernel of the same chain (the allocation-free entry's set-up), so it may be
+  // read only after pdl_wait, not, as otherwise, by a copy that is complete before
+  // the chain's first kernel starts
+  int use_inline;
   long long n_items;
   long long n_items_low; // low-band work items (0: none possible)
   // the counter block (kCounterWords), zero before the launch

@@ -170,7 +170,8 @@ extern "C" rad_status rad_accumulate_static(const double* omega, int32_t n_omega
   memset(&js, 0, sizeof(js));
   js.n_omega = n_omega;
   js.n_dir = n_dir;
-  js.n_bins = n_omega * n_dir;
+  js.n_bins = js.part_bins = n_omega * n_dir;
+  js.part_row = n_omega;
   fill_tiles(js, variant, default_omega_tile(variant, n_omega), 0);
   if (js.n_tiles > kMaxTiles) return RAD_EINVAL;
   int ck = auto_chunk_for(variant, n, js.n_tiles, false);  // (no fine-chunked tail here)
@@ -202,8 +203,7 @@ extern "C" rad_status rad_accumulate_static(const double* omega, int32_t n_omega
   memset(&a, 0, sizeof(a));
   a.js = reinterpret_cast<const JobStatic*>(base + kOffJob);
   a.n_jobs = 1;
-  a.use_inline = 1;
-  a.js_from_kernel = 1;
+  a.use_inline = kJsFromKernel;
   a.n_items = (long long)js.n_tiles * n_chunks;
   a.item_counter = reinterpret_cast<unsigned long long*>(base + kOffCounter);
   JobCall& K = a.inline_call;
