@@ -238,7 +238,10 @@ rad_status rad_state_merge(rad_ctx* ctx, const void* host_buf, size_t n);
  *  omega_tile frequencies per tile: a multiple of 32 x frequencies per thread x
  *            passes, at most 256 x frequencies per thread x passes; directions
  *            per tile follow from the block's bin count.  RAD_EINVAL otherwise.
- *  chunk     macro-particles per work item (multiple of 256), 0 = automatic. */
+ *  chunk     macro-particles per work item (multiple of 256), 0 = automatic.
+ * Only the default tile (variant 9, its default omega_tile, automatic chunk) takes
+ * a large call's lowest frequencies from nodes (the low band); a call with any
+ * other tile evaluates every bin. */
 typedef struct {
   int32_t variant;
   int32_t omega_tile;
@@ -251,9 +254,12 @@ rad_status rad_set_tile(rad_ctx* ctx, const rad_tile* tile);
 
 /* rad_tune - time candidate tiles on synthetic particles (n of them, or fewer
  * when n x bins is large; the chunk size is then left automatic) and keep the
- * fastest for this context's grid shape.  Results are cached per shape
- * bucket in memory and, when the environment variable RAD_TUNE_CACHE names a
- * file, on disk.  Leaves the accumulators unchanged. */
+ * fastest for this context's grid shape.  Where calls of n particles may take the
+ * low band (rad_tile), the fastest and the default tile are compared once more on a
+ * call large enough for it.  Results are cached per shape bucket in memory and,
+ * when the environment variable RAD_TUNE_CACHE names a file, on disk (one line of
+ * seven numbers each; lines of six, from before the band, count for calls that
+ * cannot take it).  Leaves the accumulators unchanged. */
 rad_status rad_tune(rad_ctx* ctx, int64_t n);
 
 /* Batched accumulation: one step of many independent jobs in one persistent

@@ -442,6 +442,18 @@ size_t context_bytes(const rad_ctx* c, const JobStatic& js) {
   return b + sizeof(float) * (size_t)(js.part_cap + js.fine_cap + js.low_cap);
 }
 
+// An alternative that pays for a call of n particles, in one chunk at best.
+static bool low_pays(const rad_ctx* c, const LowSet& L, long long n, long long resident) {
+  return low_cells(c, L, n, (c->n_dir + 7) / 8, 1, resident) >= kLowCellsMin;
+}
+
+bool low_possible(const rad_ctx* c, long long n) {
+  if (n < kLowMin || n >= (1LL << 31)) return false;
+  for (int s = 0; s < c->n_low; ++s)
+    if (low_pays(c, c->low[s], n, resident_ctas(kDefaultVariant))) return true;
+  return false;
+}
+
 CallLimits call_limits(const rad_ctx* c, long long n, bool band) {
   const JobStatic& js = c->h_js;
   const long long R = resident_ctas(kDefaultVariant);
@@ -475,7 +487,7 @@ CallLimits call_limits(const rad_ctx* c, long long n, bool band) {
   const long long dirs8 = (js.n_dir + 7) / 8;
   for (int s = 0; band && n >= kLowMin && s < c->n_low; ++s) {
     const LowSet& L = c->low[s];
-    if (low_cells(c, L, std::min(n, (1LL << 31) - 1), dirs8, 1, R) < kLowCellsMin) continue;  // at no size up to n
+    if (!low_pays(c, L, std::min(n, (1LL << 31) - 1), R)) continue;  // at no size up to n
     tiling(L.n_tiles, (long long)js.n_dir * (js.n_omega - L.js), kLowMin);
     const long long n_lo = std::min((long long)kLowItemsPerCta * R / dirs8 + 1, (n + kLowChunkMin - 1) / kLowChunkMin);
     lim.low = std::max(lim.low, n_lo * kComps * js.n_dir * L.js);

@@ -132,6 +132,8 @@ size_t context_bytes_at(const rad_ctx* c, const CallLimits& limits);
 // A call's evaluated updates as a share of its particles x bins when it takes
 // alternative `set` of the low band (-1: none): tiles and nodes against all tiles.
 double evaluated_share(const rad_ctx* c, int set);
+// Whether a call of n particles may take the low band (with the default tile).
+bool low_possible(const rad_ctx* c, long long n);
 // Makes room for a planned call.  The low band is taken only where its buffers fit:
 // without memory for them the call is planned again without it.
 rad_status reserve_call(rad_ctx* c, const JobStatic& js, int variant, long long n, CallPlan& plan);

@@ -2,6 +2,9 @@
 // (threads x frequencies per thread), frequency-tile width and particles per
 // work item, timed with CUDA events on synthetic particles, cached per grid
 // shape bucket in memory and optionally in the file named by RAD_TUNE_CACHE.
+// A call that may take the low band can do so with the default tile only, and the
+// bounded trials may be too small for it, so there the default tile and the trials'
+// best are timed again on a larger call.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -22,7 +25,8 @@ using namespace radimpl;
 
 namespace {
 
-using Key = std::tuple<int, int, int>;  // n_omega, n_dir, log2 bucket of n
+// n_omega, n_dir, log2 bucket of n, whether a call of n may take the low band
+using Key = std::tuple<int, int, int, int>;
 
 std::mutex g_mu;
 std::map<Key, rad_tile> g_cache;
@@ -41,11 +45,14 @@ void load_cache_locked() {
   if (!path || !*path) return;
   FILE* f = fopen(path, "r");
   if (!f) return;
-  int no, nd, b, v, wt, ck;
-  while (fscanf(f, "%d %d %d %d %d %d", &no, &nd, &b, &v, &wt, &ck) == 6) {
+  char line[256];
+  while (fgets(line, sizeof(line), f)) {
+    // (lines of six numbers were written before the low band, and hold without it)
+    int no, nd, b, v, wt, ck, band = 0;
+    if (sscanf(line, "%d %d %d %d %d %d %d", &no, &nd, &b, &v, &wt, &ck, &band) < 6) continue;
     if (v < 0 || v >= kNumVariants || !valid_omega_tile(v, wt) || ck < 0 || ck % kChunkAlign) continue;
     rad_tile t{v, wt, ck, 0};
-    g_cache[Key(no, nd, b)] = t;
+    g_cache[Key(no, nd, b, band != 0)] = t;
   }
   fclose(f);
 }
@@ -56,8 +63,8 @@ void store_cache_locked(const Key& k, const rad_tile& t) {
   if (!path || !*path) return;
   FILE* f = fopen(path, "a");
   if (!f) return;
-  fprintf(f, "%d %d %d %d %d %d\n", std::get<0>(k), std::get<1>(k), std::get<2>(k), t.variant,
-          t.omega_tile, t.chunk);
+  fprintf(f, "%d %d %d %d %d %d %d\n", std::get<0>(k), std::get<1>(k), std::get<2>(k), t.variant,
+          t.omega_tile, t.chunk, std::get<3>(k));
   fclose(f);
 }
 
@@ -97,7 +104,8 @@ extern "C" rad_status rad_tune(rad_ctx* c, int64_t n) {
   if (check_device(c) != RAD_OK) return RAD_EINVAL;
   if (c->prec != RAD_PREC_MIXED) return RAD_OK;  // the FP64 kernel has no tiles
   if (c->h_js.literal) return RAD_OK;             // the literal sum has one variant
-  const Key key(c->n_omega, c->n_dir, bucket(n));
+  const bool band = low_possible(c, n);
+  const Key key(c->n_omega, c->n_dir, bucket(n), band);
   {
     std::lock_guard<std::mutex> lk(g_mu);
     load_cache_locked();
@@ -118,22 +126,43 @@ extern "C" rad_status rad_tune(rad_ctx* c, int64_t n) {
   // Time on a bounded particle count so a trial costs milliseconds.
   const long long nt = std::min<long long>(n, std::max<long long>(
       4096, (long long)(2.0e9 / ((double)c->n_bins + 1.0))));
+  // The second comparison, where the band may be taken: up to 3e10 updates (15 ms).
+  const long long nb = band ? std::min<long long>(n, std::max<long long>(nt, std::min<long long>(
+                                  1 << 22, (long long)(3.0e10 / ((double)c->n_bins + 1.0))))) : nt;
   double *r = nullptr, *b = nullptr, *bd = nullptr, *w = nullptr;
   void* saved = nullptr;
   rad_status st = RAD_OK;
   const size_t blob = rad_state_size(c);
   rad_tile orig = c->tile;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (cudaMalloc(&r, sizeof(double) * 3 * nt) != cudaSuccess ||
-      cudaMalloc(&b, sizeof(double) * 3 * nt) != cudaSuccess ||
-      cudaMalloc(&bd, sizeof(double) * 3 * nt) != cudaSuccess ||
-      cudaMalloc(&w, sizeof(double) * nt) != cudaSuccess || !(saved = malloc(blob))) {
+  if (cudaMalloc(&r, sizeof(double) * 3 * nb) != cudaSuccess ||
+      cudaMalloc(&b, sizeof(double) * 3 * nb) != cudaSuccess ||
+      cudaMalloc(&bd, sizeof(double) * 3 * nb) != cudaSuccess ||
+      cudaMalloc(&w, sizeof(double) * nb) != cudaSuccess || !(saved = malloc(blob))) {
     st = RAD_ENOMEM;
   }
   if (st == RAD_OK) st = rad_state_export(c, saved, blob);
-  if (st == RAD_OK) {
-    fill_synthetic<<<(unsigned)((nt + 255) / 256), 256, 0, c->stream>>>(nt, r, b, bd, w);
+  auto fill = [&](long long m) {
+    fill_synthetic<<<(unsigned)((m + 255) / 256), 256, 0, c->stream>>>(m, r, b, bd, w);
     count_launches(1);
+  };
+  // Time of two calls of m particles with a tile, after one to warm up; < 0: not valid here.
+  auto trial = [&](const rad_tile& t, long long m) -> float {
+    if (rad_set_tile(c, &t) != RAD_OK) return -1.0f;
+    float ms_sum = 0.f;
+    for (int rep = 0; rep < 3 && st == RAD_OK; ++rep) {
+      cudaEventRecord(e0, c->stream);
+      st = rad_accumulate(c, m, r, b, bd, w, 1e-15, 1e-16);
+      cudaEventRecord(e1, c->stream);
+      if (cudaEventSynchronize(e1) != cudaSuccess) st = RAD_ECUDA;
+      float ms = 0.f;
+      cudaEventElapsedTime(&ms, e0, e1);
+      if (rep > 0) ms_sum += ms;
+    }
+    return ms_sum;
+  };
+  if (st == RAD_OK) {
+    fill(nt);
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
   }
@@ -156,21 +185,23 @@ extern "C" rad_status rad_tune(rad_ctx* c, int64_t n) {
         if (ck2 == ck) continue;
         t.chunk = ck2;
       }
-      if (rad_set_tile(c, &t) != RAD_OK) continue;
-      float ms_sum = 0.f;
-      for (int rep = 0; rep < 3 && st == RAD_OK; ++rep) {
-        cudaEventRecord(e0, c->stream);
-        st = rad_accumulate(c, nt, r, b, bd, w, 1e-15, 1e-16);
-        cudaEventRecord(e1, c->stream);
-        if (cudaEventSynchronize(e1) != cudaSuccess) st = RAD_ECUDA;
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (rep > 0) ms_sum += ms;  // first repetition is warm-up
-      }
-      if (st == RAD_OK && ms_sum < best_ms) {
-        best_ms = ms_sum;
+      const float ms = trial(t, nt);
+      if (st == RAD_OK && ms >= 0.f && ms < best_ms) {
+        best_ms = ms;
         best = c->tile;
       }
+    }
+  }
+  const rad_tile def{kDefaultVariant, default_omega_tile(kDefaultVariant, c->n_omega), 0, 0};
+  if (st == RAD_OK && band &&
+      (best.variant != def.variant || best.omega_tile != def.omega_tile || best.chunk != def.chunk)) {
+    fill(nb);
+    const float ms_best = trial(best, nb);
+    const float ms_def = st == RAD_OK ? trial(def, nb) : 0.f;
+    // (a call of n takes the band where only more than 2^22 particles pay for it)
+    if (ms_def <= ms_best || !low_possible(c, nb)) {
+      best = def;
+      best_ms = ms_def;
     }
   }
   if (st == RAD_OK) st = rad_set_tile(c, &best);
