@@ -57,6 +57,11 @@ rad_status rad_selftest_phase(rad_ctx* ctx, int32_t n_tau, const float* th, cons
  * times < 1. */
 rad_status rad_selftest_fail_alloc(rad_ctx* ctx, int32_t nth, int32_t times);
 
+/* rad_selftest_give_up - marks the context, after its queued work, as a kernel whose
+ * bounded wait gave up does: the next synchronising call reports RAD_ETIMEOUT.
+ * Errors: RAD_EINVAL, RAD_ECUDA, RAD_ESTATE. */
+rad_status rad_selftest_give_up(rad_ctx* ctx);
+
 /* rad_selftest_memory - *bytes (host) = device bytes the context holds in its tables,
  * accumulators, records, sort buffers and partial sums (not the copies of
  * host arrays, in-situ steps or profiling counters).  Mixed-precision contexts only.

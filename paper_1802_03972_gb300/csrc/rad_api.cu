@@ -432,7 +432,7 @@ size_t context_bytes(const rad_ctx* c, const JobStatic& js) {
   size_t b = 2 * sizeof(double) * c->n_omega + sizeof(float) * c->tab_floats +
              (3 * sizeof(double) + kDirTab * sizeof(float)) * (size_t)c->n_dir + 4 * sizeof(double) +
              kStatusWords * sizeof(int) + sizeof(c->low) + kCounterWords * sizeof(unsigned long long) +
-             sizeof(JobStatic) + (3 * sizeof(double) + 2 * kComps * sizeof(float)) * nb;
+             sizeof(JobStatic) + kMaxSpecies * sizeof(int) + (3 * sizeof(double) + 2 * kComps * sizeof(float)) * nb;
   if (js.literal) b += 8 * sizeof(float) * nb + sizeof(float) * c->n_omega + sizeof(float) * (size_t)(js.part_cap / 2);
   b += sizeof(float) * kRecFields * n;
   if (n > 0)
@@ -831,7 +831,7 @@ rad_status rad_create(const double* omega, int32_t n_omega, const double* dirs, 
   chk(dmalloc(&c->d_status, kStatusWords + sizeof(c->low) / sizeof(int)));
   chk(dmalloc(&c->d_counter, kCounterWords));
   chk(dmalloc(&c->d_js, 1));
-  chk(dmalloc(&c->d_spec, (size_t)3 * c->n_bins));
+  chk(dmalloc(&c->d_spec, (size_t)3 * c->n_bins + kMaxSpecies / 2));  // (and the species' status words)
   if (prec == RAD_PREC_MIXED) {
     chk(dmalloc(&c->d_state, (size_t)2 * kComps * c->n_bins));
     if (literal) {
@@ -940,13 +940,8 @@ rad_status rad_accumulate(rad_ctx* c, int64_t n, const double* r, const double* 
   return enqueue_accumulate(c, n, r, beta, beta_dot, w, t, dt);
 }
 
-static rad_status check_status_word(rad_ctx* c) {
-  int st = 0;
-  rad_status s = cuda_check(c, cudaMemcpyAsync(&st, c->d_status, sizeof(int),
-                                               cudaMemcpyDeviceToHost, c->stream));
-  if (s != RAD_OK) return s;
-  s = cuda_check(c, cudaStreamSynchronize(c->stream));
-  if (s != RAD_OK) return s;
+// What a context's status word, read after its queued work, says.
+static rad_status settle_status(rad_ctx* c, int st) {
   if (st & ST_BOUNDS) {
     // A debug build's index check failed: a sizing error inside the library.
     rad_log(1, "an index check of the debug build failed (status 0x%x)", st);
@@ -960,11 +955,20 @@ static rad_status check_status_word(rad_ctx* c) {
   }
   if (st & ST_BAD_PARTICLE) {
     const int keep = st & ~ST_BAD_PARTICLE;
-    s = cuda_check(c, cudaMemcpy(c->d_status, &keep, sizeof(int), cudaMemcpyHostToDevice));
+    const rad_status s = cuda_check(c, cudaMemcpy(c->d_status, &keep, sizeof(int), cudaMemcpyHostToDevice));
     if (s != RAD_OK) return s;
     return fail(c, RAD_EDATA);
   }
   return RAD_OK;
+}
+
+static rad_status check_status_word(rad_ctx* c) {
+  int st = 0;
+  rad_status s = cuda_check(c, cudaMemcpyAsync(&st, c->d_status, sizeof(int),
+                                               cudaMemcpyDeviceToHost, c->stream));
+  if (s != RAD_OK) return s;
+  s = cuda_check(c, cudaStreamSynchronize(c->stream));
+  return s == RAD_OK ? settle_status(c, st) : s;
 }
 
 rad_status rad_sync(rad_ctx* c) {
@@ -1034,25 +1038,22 @@ rad_status rad_spectrum_species(rad_ctx* const* ctxs, const rad_ff* ffs, int32_t
     a.kind[i] = ff.kind;
     a.flags[i] = ff.flags;
     a.width[i] = ff.width;
+    a.status[i] = c->d_status;
   }
+  a.gathered = reinterpret_cast<int*>(c0->d_spec + (size_t)3 * c0->n_bins);
   // Every species' queued work must be complete before its state is read: on one
-  // stream it is by order, else the host waits for each first.  A species that
-  // saw invalid particles is reported after the spectra are written.
+  // stream it is by order, and the kernel gathers the status words for one copy, else
+  // the host waits for each first.  A species that saw invalid particles is reported
+  // after the spectra are written; one that has failed before anything is.
   rad_status data = RAD_OK;
-  auto check_all = [&]() -> rad_status {
+  bool one_stream = true;
+  for (int i = 1; i < n_species; ++i) one_stream = one_stream && ctxs[i]->stream == c0->stream;
+  if (!one_stream)
     for (int i = 0; i < n_species; ++i) {
       const rad_status s = check_status_word(ctxs[i]);
       if (s == RAD_EDATA) data = RAD_EDATA;
       else if (s != RAD_OK) return s;
     }
-    return RAD_OK;
-  };
-  bool one_stream = true;
-  for (int i = 1; i < n_species; ++i) one_stream = one_stream && ctxs[i]->stream == c0->stream;
-  if (!one_stream) {
-    const rad_status s = check_all();
-    if (s != RAD_OK) return s;
-  }
   double* outs[3] = {coh, inc, tot};
   double* dev_out[3];
   bool host[3];
@@ -1063,12 +1064,24 @@ rad_status rad_spectrum_species(rad_ctx* const* ctxs, const rad_ff* ffs, int32_t
   rad_status s = cuda_check(c0, launch_readout_species(a, c0->n_omega, c0->n_bins, c0->d_omega,
                                                        c0->d_dirs, dev_out[0], dev_out[1],
                                                        dev_out[2], c0->stream));
+  if (one_stream && s == RAD_OK) {
+    int st[kMaxSpecies];
+    s = cuda_check(c0, cudaMemcpyAsync(st, a.gathered, sizeof(int) * n_species, cudaMemcpyDeviceToHost, c0->stream));
+    if (s == RAD_OK) s = cuda_check(c0, cudaStreamSynchronize(c0->stream));
+    for (int i = 0; s == RAD_OK && i < n_species; ++i) {
+      s = settle_status(ctxs[i], st[i]);
+      if (s == RAD_EDATA) {
+        data = RAD_EDATA;
+        s = RAD_OK;
+      }
+    }
+  }
   for (int i = 0; s == RAD_OK && i < 3; ++i) {
     if (!host[i]) continue;
     s = cuda_check(c0, cudaMemcpyAsync(outs[i], dev_out[i], sizeof(double) * c0->n_bins,
                                        cudaMemcpyDeviceToHost, c0->stream));
   }
-  if (s == RAD_OK) s = one_stream ? check_all() : cuda_check(c0, cudaStreamSynchronize(c0->stream));
+  if (s == RAD_OK) s = cuda_check(c0, cudaStreamSynchronize(c0->stream));
   if (s != RAD_OK) return s;
   return data;
 }

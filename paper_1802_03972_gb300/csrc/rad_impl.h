@@ -450,6 +450,8 @@ struct SpeciesArgs {
   const double* state64[kMaxSpecies];
   int kind[kMaxSpecies], flags[kMaxSpecies];
   double width[kMaxSpecies];
+  const int* status[kMaxSpecies];    // the species' status words ...
+  int* gathered;                     // ... which the kernel copies here
 };
 cudaError_t launch_readout_species(const SpeciesArgs& a, int n_omega, int n_bins,
                                    const double* omega, const double* dirs, double* coh,

@@ -667,6 +667,10 @@ __global__ void __launch_bounds__(128) readout_species_kernel(
     double* tot) {
   constexpr int NU = MIXED ? 4 : 6;  // real components of U (and of V)
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < a.n_species) a.gathered[t] = *a.status[t];
+  // (a failed species' sums are incomplete: nothing is written, the host reports it)
+  for (int s = 0; s < a.n_species; ++s)
+    if (*a.status[s] & (ST_TIMEOUT | ST_BOUNDS)) return;
   if (t >= stride || t >= n_bins) return;
   const double om = omega[(int)(t % n_omega)];
   double u[kReadBins][NU] = {}, ii[kReadBins] = {};  // (stride: at most kReadBins bins per thread)

@@ -107,6 +107,16 @@ rad_status rad_selftest_fail_alloc(rad_ctx* c, int32_t nth, int32_t times) {
   return RAD_OK;
 }
 
+rad_status rad_selftest_give_up(rad_ctx* c) {
+  if (!c) return RAD_EINVAL;
+  if (c->failed) return RAD_ESTATE;
+  if (check_device(c) != RAD_OK) return RAD_EINVAL;
+  const int word = ST_TIMEOUT;
+  rad_status s = cuda_check(c, cudaStreamSynchronize(c->stream));
+  if (s == RAD_OK) s = cuda_check(c, cudaMemcpy(c->d_status, &word, sizeof(int), cudaMemcpyHostToDevice));
+  return s;
+}
+
 rad_status rad_selftest_memory(const rad_ctx* c, int64_t* bytes) {
   if (!c || !bytes || c->prec != RAD_PREC_MIXED) return RAD_EINVAL;
   *bytes = (int64_t)context_bytes(c, c->h_js);

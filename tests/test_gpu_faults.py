@@ -225,3 +225,30 @@ def test_a_call_after_one_that_stayed_out_of_memory(nth):
         gpu_run(wl, [1], ctx=ctx)
         for x, y in zip(ctx.spectrum(), gpu_run(wl, [1]).spectrum()):
             np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("streams", ["one", "two"])
+@pytest.mark.parametrize("device_out", [False, True])
+@pytest.mark.parametrize("which", [0, 1])
+def test_species_readout_with_a_failed_species_writes_nothing(which, device_out, streams):
+    """A species whose kernel gave up has incomplete sums: the readout reports it and leaves the outputs as they were."""
+    wl = jobs()[0]
+    ctxs = [rad.Context(wl.omega, wl.dirs, wl.ff_kind, wl.ff_width,
+                        stream=torch.cuda.Stream() if streams == "two" else None) for _ in range(2)]
+    torch.cuda.synchronize()
+    for k, c in enumerate(ctxs):
+        gpu_run(wl, [k], ctx=c)
+    ffs = [(rad.FF_GAUSS, 1e-7), (rad.FF_CIC, 1e-7)]
+    good = rad.spectrum_species(ctxs, ffs)
+    assert all(np.all(np.isfinite(x)) and np.any(x > 0) for x in good)
+    ctxs[which].selftest_give_up()
+    shape = (wl.dirs.shape[0], wl.omega.shape[0])
+    out = [torch.full(shape, -7.0, dtype=torch.float64, device="cuda") if device_out else np.full(shape, -7.0)
+           for _ in range(3)]
+    torch.cuda.synchronize()
+    with pytest.raises(rad.RadError) as ei:
+        rad.spectrum_species(ctxs, ffs, out=out)
+    assert ei.value.status == rad.RAD_ETIMEOUT
+    torch.cuda.synchronize()
+    for o in out:
+        assert bool((o == -7.0).all())
