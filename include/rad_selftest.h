@@ -57,6 +57,12 @@ rad_status rad_selftest_phase(rad_ctx* ctx, int32_t n_tau, const float* th, cons
  * times < 1. */
 rad_status rad_selftest_fail_alloc(rad_ctx* ctx, int32_t nth, int32_t times);
 
+/* rad_selftest_band - what the context's last call took from nodes (the low band):
+ * *bins (host) = the lowest frequencies of each direction, 0 if none, and *cells
+ * (host) the cells of particles it was cut into.  Waits for the context's work.
+ * Mixed-precision contexts only.  Errors: RAD_EINVAL, RAD_ECUDA, RAD_ESTATE. */
+rad_status rad_selftest_band(rad_ctx* ctx, int32_t* bins, int32_t* cells);
+
 /* rad_selftest_give_up - marks the context, after its queued work, as a kernel whose
  * bounded wait gave up does: the next synchronising call reports RAD_ETIMEOUT.
  * Errors: RAD_EINVAL, RAD_ECUDA, RAD_ESTATE. */

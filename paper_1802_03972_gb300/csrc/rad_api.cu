@@ -663,6 +663,7 @@ rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const do
   CallPlan plan = plan_call(c, c->h_js, variant, n);
   rad_status s = reserve_call(c, c->h_js, variant, n, plan);
   if (s != RAD_OK) return s;
+  c->last_low = plan.low_ok;
   LaunchArgs a;
   memset(&a, 0, sizeof(a));
   a.js = c->d_js;

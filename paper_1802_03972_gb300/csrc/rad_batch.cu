@@ -209,6 +209,7 @@ rad_status BatchCore::run(rad_ctx* const* jobs, const rad_step* steps, int n_job
     K.dt = st.dt;
     const int run = run_of(plan[p]);
     plan[p].call.fill(K, plan[p].js, run);
+    jobs[plan[p].job]->last_low = plan[p].call.low_ok;
     K.item_begin = items;
     K.low_begin = low_items;
     K.block_begin = blocks;

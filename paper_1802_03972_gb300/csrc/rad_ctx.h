@@ -64,6 +64,7 @@ struct rad_ctx {
   double low_full = 0.0;         // cost of the full tiling, in full tiles
   radimpl::LowSet low[radimpl::kLowSets]{};
   long long generation = 0;      // bumped whenever d_js changes
+  unsigned last_low = 0;         // low_ok of the last call: with none its plan was not written
   size_t tab_floats = 0;         // of d_om_tab: om_tab, then the low band's tables
   // Some call's low-band buffers did not fit the device: calls take the bin tiles, as
   // they do without the band, until rad_reset.

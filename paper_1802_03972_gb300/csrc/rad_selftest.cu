@@ -107,6 +107,21 @@ rad_status rad_selftest_fail_alloc(rad_ctx* c, int32_t nth, int32_t times) {
   return RAD_OK;
 }
 
+rad_status rad_selftest_band(rad_ctx* c, int32_t* bins, int32_t* cells) {
+  if (!c || !bins || !cells) return RAD_EINVAL;
+  if (c->failed) return RAD_ESTATE;
+  if (check_device(c) != RAD_OK || c->prec != RAD_PREC_MIXED) return RAD_EINVAL;
+  *bins = *cells = 0;
+  rad_status s = cuda_check(c, cudaDeviceSynchronize());  // (a batch's work runs on a stream of its own)
+  if (s != RAD_OK || c->last_low == 0) return s;
+  LowPlan p;
+  s = cuda_check(c, cudaMemcpy(&p, c->h_js.plan, sizeof(p), cudaMemcpyDeviceToHost));
+  if (s != RAD_OK || p.set < 0) return s;
+  *bins = c->low[p.set].js;
+  *cells = p.cells;
+  return RAD_OK;
+}
+
 rad_status rad_selftest_give_up(rad_ctx* c) {
   if (!c) return RAD_EINVAL;
   if (c->failed) return RAD_ESTATE;

@@ -288,9 +288,9 @@ void rad_server::loop() {
       rs = core.run(ctxs.data(), steps.data(), (int)ctxs.size(), false);
       for (size_t i = 0; i < ctxs.size() && rs == RAD_OK; ++i) {
         h_sets[i] = -1;
-        const bool may = plan_call(ctxs[i], ctxs[i]->h_js, kDefaultVariant, steps[i].n).low_ok != 0;
-        if (may && cudaMemcpyAsync(&h_sets[i], &ctxs[i]->h_js.plan->set, sizeof(int), cudaMemcpyDeviceToHost,
-                                   compute) != cudaSuccess)
+        if (ctxs[i]->last_low != 0 &&
+            cudaMemcpyAsync(&h_sets[i], &ctxs[i]->h_js.plan->set, sizeof(int), cudaMemcpyDeviceToHost, compute) !=
+                cudaSuccess)
           rs = RAD_ECUDA;
       }
       if (rs == RAD_OK && cudaStreamSynchronize(compute) != cudaSuccess) rs = RAD_ECUDA;

@@ -38,7 +38,7 @@ EXPORTS = [
     "rad_static_status",
     "rad_spectrum_literal", "rad_push_step", "rad_push_flush",
     "rad_selftest_wait", "rad_selftest_stage1", "rad_selftest_phase", "rad_selftest_fail_alloc",
-    "rad_selftest_memory", "rad_selftest_limit", "rad_selftest_give_up",
+    "rad_selftest_memory", "rad_selftest_limit", "rad_selftest_give_up", "rad_selftest_band",
 ]
 FF_LITERAL = 2  # rad_ff.flags at creation: also accumulate the paper's literal sum
 # Round policies of the serving loop (rad_server_set_policy).
@@ -140,6 +140,7 @@ def load(path: str = LIB_PATH):
         "rad_selftest_phase": (st, [vp, i32, vp, vp, vp, vp]),
         "rad_selftest_fail_alloc": (st, [vp, i32, i32]),
         "rad_selftest_give_up": (st, [vp]),
+        "rad_selftest_band": (st, [vp, ctypes.POINTER(i32), ctypes.POINTER(i32)]),
         "rad_selftest_memory": (st, [vp, ctypes.POINTER(i64)]),
         "rad_selftest_limit": (st, [vp, i64, ctypes.POINTER(i64)]),
         "rad_accumulate_static": (st, [vp, i32, vp, i32, i64, vp, vp, vp, vp, dbl, dbl, vp, vp]),
@@ -393,6 +394,12 @@ class Context:
     def selftest_fail_alloc(self, nth: int, times: int = 1) -> None:
         """rad_selftest_fail_alloc: the nth next buffer allocation of this context's calls and the times - 1 after it fail."""
         _check(self._lib.rad_selftest_fail_alloc(self._h, int(nth), int(times)), "rad_selftest_fail_alloc")
+
+    def selftest_band(self) -> tuple:
+        """rad_selftest_band: (frequencies, cells) that the last call took from nodes, (0, 0) if none."""
+        bins, cells = ctypes.c_int32(), ctypes.c_int32()
+        _check(self._lib.rad_selftest_band(self._h, ctypes.byref(bins), ctypes.byref(cells)), "rad_selftest_band")
+        return bins.value, cells.value
 
     def selftest_give_up(self) -> None:
         """rad_selftest_give_up: as if a bounded wait of one of this context's kernels had given up."""
