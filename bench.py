@@ -165,14 +165,12 @@ def kernel_hash() -> str:
     return h.hexdigest()[:16]
 
 
-def evaluated_share(n_omega: int, tile) -> float:
-    """Share of a step's updates whose sin/cos the accumulate kernel evaluates on the
-    benchmark's large log grids: with the default tiling a call of this size takes its
-    lowest n_omega / 2 bins from 64 nodes per direction (LowSet in csrc/rad_impl.h) and
-    evaluates the others; any other tiling evaluates all."""
-    if tile[0] == 9 and tile[1] == 512 and tile[2] == 0 and n_omega in (512, 1024):
-        return (n_omega // 2 + 64) / n_omega
-    return 1.0
+def evaluated_share(ctx, n_omega: int) -> float:
+    """Share of a step's updates whose sin/cos the accumulate kernel evaluated in the context's
+    last call: the frequencies that it took from 64 nodes per direction (the low band, as the
+    device decided; LowSet in csrc/rad_impl.h) cost the nodes' instead."""
+    bins, _ = ctx.selftest_band()
+    return (n_omega - bins + 64) / n_omega if bins else 1.0
 
 
 def traffic_per_launch(updates_per_step: int, tile):
@@ -605,7 +603,7 @@ def insitu_leg(n_total: int = 10_000_000, n_chunk: int = 1_000_000, fp64_sample:
     mhz = ctx.profile_clock()
     ctx.profile(False)
     sm = torch.cuda.get_device_properties(0).multi_processor_count
-    peak = sm * MUFU_PER_CLK_SM * SM_MAX_MHZ * 1e6 / (MUFU_PER_UPDATE * evaluated_share(1024, tile))
+    peak = sm * MUFU_PER_CLK_SM * SM_MAX_MHZ * 1e6 / (MUFU_PER_UPDATE * evaluated_share(ctx, 1024))
     achieved = upd / (acc_ms / 1e3)
     out = {"workload": "1e7 macro-particles (10 calls of 1e6), 1024 log omega 1e14-1e20 rad/s, "
                        "32x32 directions +-10 mrad, CIC 0.1 um; readouts CIC and TSC",
@@ -873,7 +871,7 @@ def main():
     sm = torch.cuda.get_device_properties(dev).multi_processor_count
     acc_s = acc_ms / max(calls, 1) / 1e3
     achieved = upd / acc_s if acc_s > 0 else None
-    share = evaluated_share(int(wl.omega.shape[0]), tile)
+    share = evaluated_share(ctx, int(wl.omega.shape[0]))
     peak = sm * MUFU_PER_CLK_SM * SM_MAX_MHZ * 1e6 / (MUFU_PER_UPDATE * share)
     roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": UNIT,
             "frac": achieved / peak if achieved else None, "traffic": traffic_per_launch(upd, tile),
