@@ -126,26 +126,30 @@ extern "C" rad_status rad_tune(rad_ctx* c, int64_t n) {
   // Time on a bounded particle count so a trial costs milliseconds.
   const long long nt = std::min<long long>(n, std::max<long long>(
       4096, (long long)(2.0e9 / ((double)c->n_bins + 1.0))));
-  // The second comparison, where the band may be taken: up to 3e10 updates (15 ms).
-  const long long nb = band ? std::min<long long>(n, std::max<long long>(nt, std::min<long long>(
-                                  1 << 22, (long long)(3.0e10 / ((double)c->n_bins + 1.0))))) : nt;
   double *r = nullptr, *b = nullptr, *bd = nullptr, *w = nullptr;
   void* saved = nullptr;
   rad_status st = RAD_OK;
   const size_t blob = rad_state_size(c);
   rad_tile orig = c->tile;
+  const bool low_nomem = c->low_nomem;  // (a shortage of the trials' is not the caller's)
   cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (cudaMalloc(&r, sizeof(double) * 3 * nb) != cudaSuccess ||
-      cudaMalloc(&b, sizeof(double) * 3 * nb) != cudaSuccess ||
-      cudaMalloc(&bd, sizeof(double) * 3 * nb) != cudaSuccess ||
-      cudaMalloc(&w, sizeof(double) * nb) != cudaSuccess || !(saved = malloc(blob))) {
-    st = RAD_ENOMEM;
-  }
-  if (st == RAD_OK) st = rad_state_export(c, saved, blob);
-  auto fill = [&](long long m) {
+  // Inputs of m particles in place of the last.
+  auto fill = [&](long long m) -> bool {
+    for (double** p : {&r, &b, &bd, &w}) {
+      cudaFree(*p);
+      *p = nullptr;
+    }
+    if (cudaMalloc(&r, sizeof(double) * 3 * m) != cudaSuccess || cudaMalloc(&b, sizeof(double) * 3 * m) != cudaSuccess ||
+        cudaMalloc(&bd, sizeof(double) * 3 * m) != cudaSuccess || cudaMalloc(&w, sizeof(double) * m) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
     fill_synthetic<<<(unsigned)((m + 255) / 256), 256, 0, c->stream>>>(m, r, b, bd, w);
     count_launches(1);
+    return true;
   };
+  if (!(saved = malloc(blob)) || !fill(nt)) st = RAD_ENOMEM;
+  if (st == RAD_OK) st = rad_state_export(c, saved, blob);
   // Time of two calls of m particles with a tile, after one to warm up; < 0: not valid here.
   auto trial = [&](const rad_tile& t, long long m) -> float {
     if (rad_set_tile(c, &t) != RAD_OK) return -1.0f;
@@ -162,7 +166,6 @@ extern "C" rad_status rad_tune(rad_ctx* c, int64_t n) {
     return ms_sum;
   };
   if (st == RAD_OK) {
-    fill(nt);
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
   }
@@ -195,15 +198,25 @@ extern "C" rad_status rad_tune(rad_ctx* c, int64_t n) {
   const rad_tile def{kDefaultVariant, default_omega_tile(kDefaultVariant, c->n_omega), 0, 0};
   if (st == RAD_OK && band &&
       (best.variant != def.variant || best.omega_tile != def.omega_tile || best.chunk != def.chunk)) {
-    fill(nb);
-    const float ms_best = trial(best, nb);
-    const float ms_def = st == RAD_OK ? trial(def, nb) : 0.f;
-    // (a call of n takes the band where only more than 2^22 particles pay for it)
-    if (ms_def <= ms_best || !low_possible(c, nb)) {
+    // up to 3e10 updates (15 ms) and 2^22 particles; where that is too few for the
+    // band or finds no memory, the default tile
+    const long long nb = std::min<long long>(n, std::max<long long>(nt, std::min<long long>(
+        1 << 22, (long long)(3.0e10 / ((double)c->n_bins + 1.0)))));
+    float ms_best = 0.f, ms_def = 0.f;
+    if (low_possible(c, nb) && fill(nb)) {
+      ms_best = trial(best, nb);
+      ms_def = st == RAD_OK ? trial(def, nb) : 0.f;
+    }
+    if (st == RAD_ENOMEM) {
+      st = RAD_OK;
+      ms_def = ms_best = 0.f;
+    }
+    if (ms_def <= ms_best) {
       best = def;
-      best_ms = ms_def;
+      if (ms_def > 0.f) best_ms = ms_def;
     }
   }
+  c->low_nomem = low_nomem;
   if (st == RAD_OK) st = rad_set_tile(c, &best);
   if (st == RAD_OK) st = rad_state_import(c, saved, blob);
   if (st == RAD_OK) {

@@ -48,3 +48,23 @@ def test_tuned_contexts_keep_the_band(n, n_omega, side):
     ctx = rad.Context(inputs.omega_log(1e14, 1e20, n_omega), inputs.dirs_grid(0.01, side, side), rad.FF_GAUSS, 1e-7)
     assert ctx.tune(n) == (9, 512, 0)
     ctx.close()
+
+
+@pytest.mark.parametrize("nth", range(6, 16))
+def test_a_shortage_during_the_trials_does_not_outlast_them(nth):
+    """The nth buffer that a trial allocates is refused, a band buffer at some nth: the tuner goes on without the band, and
+    the caller's next call, with memory for it, takes it."""
+    from gpu_util import gpu_run
+    n_omega = 512 + 4 * nth  # (a shape of its own: results are cached)
+    wl = inputs.Workload("tune", inputs.omega_log(1e14, 1e20, n_omega), inputs.dirs_grid(0.01, 8, 8),
+                         inputs.BetatronBunch(60000, seed=81), 4, 1e-16, inputs.FF_GAUSS, 1e-7)
+    ctx = rad.Context(wl.omega, wl.dirs, wl.ff_kind, wl.ff_width)
+    ctx.selftest_fail_alloc(nth)
+    try:
+        ctx.tune(60000)
+    except rad.RadError as e:  # a buffer of a candidate without the band
+        assert e.status == rad.RAD_ENOMEM
+    ctx.selftest_fail_alloc(0)
+    ctx.set_tile(9, 0, 0)
+    assert gpu_run(wl, [0], ctx=ctx).selftest_band()[0] > 0
+    ctx.close()
