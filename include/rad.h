@@ -336,9 +336,12 @@ rad_status rad_server_create(size_t hbm_budget, int32_t max_slots, void* stream,
  *     large jobs that have waited long are not passed over indefinitely;
  *   RAD_SERVE_OLDEST_BACKFILL (default, round_updates = 2e9): the oldest job
  *     with a step ready always; the others, least served first, each only if
- *     the round's updates stay within max(round_updates, 17/16 of the oldest
- *     job's step), so the oldest job runs at >= 16/17 of its own pace (the tail
- *     latency of a FIFO queue) while small jobs progress in the margin.
+ *     the round's work stays within max(round_updates, 17/16 of the oldest job's
+ *     step), so small jobs progress in a margin of a large one's rounds.  Work
+ *     here is the updates that are evaluated: a step that takes its lowest
+ *     frequencies from nodes (rad_tile) counts the nodes instead.  The margin
+ *     bounds work, not time: many small steps take longer than their updates at a
+ *     large step's rate.
  * round_updates >= 1 for all but RAD_SERVE_ALL, which ignores it.  Takes effect
  * from the next round.  RAD_EINVAL for an unknown policy or round_updates < 1. */
 enum { RAD_SERVE_ALL = 0, RAD_SERVE_OLDEST = 1, RAD_SERVE_LEAST_SERVED = 2, RAD_SERVE_LEAST_SERVED_AGED = 3,

@@ -672,9 +672,9 @@ rad_status enqueue_accumulate(rad_ctx* c, long long n, const double* r, const do
   a.use_inline = 1;
   a.n_items = plan.items(c->h_js, 1);
   a.n_items_low = plan.low_items;
-  a.item_counter = c->d_counter;  // [0], [1]: item counters; [2]: the wide flag
+  a.item_counter = c->d_counter;
   // A call of at most one sorted group is never wide (the pre-pass does not
-  // flag it): it needs neither the wide-call kernels nor the second kernel.
+  // flag it): it needs neither the wide-call kernels nor the wide pass.
   a.any_wide = n > kGroup ? c->h_js.wide_flag : nullptr;
   JobCall& K = a.inline_call;
   K.n = n;

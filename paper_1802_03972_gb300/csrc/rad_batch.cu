@@ -73,7 +73,7 @@ rad_status BatchCore::init(int max_jobs, cudaStream_t s) {
       cudaEventCreateWithFlags(&ev_out, cudaEventDisableTiming) != cudaSuccess)
     return RAD_ECUDA;
   if (cudaMalloc(&d_js, sizeof(JobStatic) * cap) != cudaSuccess) return RAD_ENOMEM;
-  // Counter block: the two kernels' item counters, the launch's wide flag, then
+  // Counter block (kCounterWords: item counters, the launch's flags), then
   // one wide flag (int) per job slot; zeroed before every round.
   counter_bytes = kCounterWords * sizeof(unsigned long long) + sizeof(int) * (size_t)cap;
   if (cudaMalloc(&d_counter, counter_bytes) != cudaSuccess) return RAD_ENOMEM;

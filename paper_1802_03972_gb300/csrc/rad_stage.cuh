@@ -247,6 +247,9 @@ __device__ __forceinline__ void store_record_xt(float th, float tl, const float 
                       a[2] - __uint_as_float(h2), a[3] - __uint_as_float(h3));
 }
 
+// (The bin tiles' loop, process_item_tc, has this step written out: through the
+// function, with the same registers, the LWFA step takes 4733 us instead of 4715 and
+// 50000 particles, 256 x 64 bins 2205 instead of 2190.)
 // Variant 9's 8-particle step at kk over a warp's NB frequency blocks (lane (r, c) of
 // the fragments; xr_off: its cross-term pair within particle kk + r's row).
 // The main product's k = c and k = c + 4 are particles kk + 2c and kk + 2c + 1

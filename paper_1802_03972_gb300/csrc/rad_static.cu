@@ -27,7 +27,6 @@ constexpr size_t kOffOmTab = 1280;                              // float[kOmTab]
 constexpr size_t kOffOmTurns = kOffOmTab + 4 * kOmTab * RAD_STATIC_MAX_OMEGA;  // double[MAX_OMEGA]
 constexpr size_t kOffDirTab = kOffOmTurns + 8 * RAD_STATIC_MAX_OMEGA;       // float[12][MAX_DIRS]
 constexpr size_t kOffDirs = kOffDirTab + 4 * 12 * RAD_STATIC_MAX_DIRS;      // double[MAX_DIRS][3]
-constexpr int kMaxTiles = 8192;
 constexpr size_t kOffRec = kOffDirs + 8 * 3 * RAD_STATIC_MAX_DIRS;          // float[MAX_PARTICLES][20]
 constexpr int kMaxChunks = 4;  // at RAD_STATIC_MAX_BINS bins; in proportion more for fewer
 constexpr size_t kOffPart = kOffRec + 4 * (size_t)kRecFields * RAD_STATIC_MAX_PARTICLES;
@@ -173,7 +172,6 @@ extern "C" rad_status rad_accumulate_static(const double* omega, int32_t n_omega
   js.n_bins = js.part_bins = n_omega * n_dir;
   js.part_row = n_omega;
   fill_tiles(js, variant, default_omega_tile(variant, n_omega), 0);
-  if (js.n_tiles > kMaxTiles) return RAD_EINVAL;
   int ck = auto_chunk_for(variant, n, js.n_tiles, false);  // (no fine-chunked tail here)
   int n_chunks = (int)((n + ck - 1) / ck);
   const int max_chunks = (int)((long long)kMaxChunks * RAD_STATIC_MAX_BINS / js.n_bins);
