@@ -49,6 +49,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "rad_device.cuh"
 #include "rad_impl.h"
@@ -779,8 +780,12 @@ __device__ __forceinline__ bool process_item_tc(const JobStatic& J, const JobCal
       const PartMap pm = part_map(J, K, si.it, g);
       float* part = pm.base + (size_t)chunk * pm.chunk_stride;
       const size_t cs = pm.comp_stride;
-      const size_t off = si.it.fine < 0 ? (size_t)my_d * J.part_row + o_warp0
-                                        : (size_t)my_dl * g.WT + (o_warp0 - g.o0);
+      // (32 bits, enough for 2^31 bins: in 64 the loop above spills differently, and 20000
+      // particles, 250 x 40 bins take 159.0 us instead of 156.9; the wide pass the other
+      // way round, 2064 us instead of 2035 for 1e5 particles over 2 mm, 512 x 64 bins)
+      using Off = std::conditional_t<WIDE, size_t, unsigned>;
+      const Off off = si.it.fine < 0 ? (Off)my_d * (Off)J.part_row + (Off)o_warp0
+                                     : (Off)(my_dl * g.WT + (o_warp0 - g.o0));
       float* q = part + off + r + (size_t)(4 * c) * cs;
       const int left = n_om - o_warp0 - r;  // rows past the grid are not written
       const bool mine = c < 2 && my_d_raw < J.n_dir &&
@@ -1304,8 +1309,12 @@ __device__ __forceinline__ float4 load_quad(const float* p, bool vec, int live) 
 }
 
 // LATE: the job table comes from a kernel (kJsFromKernel).
+// One block per SM by its registers: launched while the accumulate kernel still runs
+// (pdl_trigger), two would fit in next to its blocks, and the next step's accumulate
+// blocks then found the SMs unevenly taken (2000 particles, 125 x 60 bins: 53 us a step
+// at 64 registers, 33 at 71 and more).
 template <bool LATE>
-__global__ void __launch_bounds__(kRedThreads) reduce_kernel(const __grid_constant__ LaunchArgs a) {
+__global__ void __launch_bounds__(kRedThreads, 1) reduce_kernel(const __grid_constant__ LaunchArgs a) {
   __shared__ __align__(8) BlockState b;
   __shared__ float4 part[kRedGroups - 1][2][kRedBins];
   __shared__ float2 rot[kRedBins];
