@@ -1309,12 +1309,14 @@ __device__ __forceinline__ float4 load_quad(const float* p, bool vec, int live) 
 }
 
 // LATE: the job table comes from a kernel (kJsFromKernel).
-// One block per SM by its registers: launched while the accumulate kernel still runs
-// (pdl_trigger), two would fit in next to its blocks, and the next step's accumulate
-// blocks then found the SMs unevenly taken (2000 particles, 125 x 60 bins: 53 us a step
-// at 64 registers, 33 at 71 and more).
-template <bool LATE>
-__global__ void __launch_bounds__(kRedThreads, 1) reduce_kernel(const __grid_constant__ LaunchArgs a) {
+// PER_SM: blocks per SM by the registers.  One for a single job: launched while the
+// accumulate kernel still runs (pdl_trigger), two would fit in next to its blocks, and
+// the next step's accumulate blocks then found the SMs unevenly taken (2000
+// particles, 125 x 60 bins: 53 us a step at 64 registers, 33 at 71 and more).  Two for
+// a batch, whose next round begins with copies (64 jobs of 1e3-1e4 particles: 1.31e12
+// updates/s, with one 1.26e12).
+template <bool LATE, int PER_SM>
+__global__ void __launch_bounds__(kRedThreads, PER_SM) reduce_kernel(const __grid_constant__ LaunchArgs a) {
   __shared__ __align__(8) BlockState b;
   __shared__ float4 part[kRedGroups - 1][2][kRedBins];
   __shared__ float2 rot[kRedBins];
@@ -1499,7 +1501,10 @@ int reduce_blocks(const JobStatic& js, const LowSet* low_sets) {
 
 cudaError_t launch_reduce(const LaunchArgs& a, long long blocks, cudaStream_t s) {
   count_launches(1);
-  return launch_pdl(a.use_inline == kJsFromKernel ? reduce_kernel<true> : reduce_kernel<false>, blocks, kRedThreads, 0, s, a);
+  auto* const kernel = a.use_inline == kJsFromKernel ? reduce_kernel<true, 1>
+                       : a.use_inline                ? reduce_kernel<false, 1>
+                                                     : reduce_kernel<false, 2>;
+  return launch_pdl(kernel, blocks, kRedThreads, 0, s, a);
 }
 
 // Variants (rad_impl.h: variant_info): 0 FP32 256x2, 1 FP32 256x4, 2 FP32 128x2,
