@@ -115,7 +115,7 @@ struct rad_server {
   size_t footprint = 0, peak_footprint = 0;
   // The oldest job with bounded backfill, rounds of at least ~1 ms of GB300
   // work.  12 jobs of 50-500 steps, arriving at 0.7 of the GPU's rate: mean latency
-  // 2.37 s, median 3.08, 99th percentile 3.89, against 2.39, 2.90 and 3.49 one job at
+  // 2.35 s, median 3.06, 99th percentile 3.88, against 2.39, 2.91 and 3.49 one job at
   // a time in arrival order: the jobs of a few per cent of the work end in half the
   // time (1.5 instead of 3.5 s) and the large one before them a seventh later.
   int policy = RAD_SERVE_OLDEST_BACKFILL;
