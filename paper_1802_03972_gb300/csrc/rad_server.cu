@@ -213,9 +213,9 @@ void rad_server::loop() {
                        [](const Job* a, const Job* b) { return a->served < b->served; });
     // Oldest job with bounded backfill: the oldest ready job always gets its
     // step, and other jobs (least served first) join only while the round's
-    // work stays within max(round_updates, 17/16 of the head's step).  The head
-    // of the queue then runs at >= 16/17 of its own pace, while small jobs progress
-    // in the margin instead of waiting behind large ones.  Work counts evaluated
+    // work stays within max(round_updates, 17/16 of the head's step), so small jobs
+    // progress in a margin of a large one's rounds instead of waiting behind it.  The
+    // margin bounds work, not time: many small steps take longer.  Work counts evaluated
     // updates: a step that takes its lowest frequencies from nodes costs about half
     // its particles x bins, and a margin counted in those slowed it by an eighth.
     const bool backfill = policy == RAD_SERVE_OLDEST_BACKFILL;
